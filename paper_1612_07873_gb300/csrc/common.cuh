@@ -241,6 +241,15 @@ __device__ __forceinline__ uint4 ld_stream16(const void* p) {
   return r;
 }
 
+// A read-only 16-byte load that stays where it is written (ahead of a wait).
+__device__ __forceinline__ uint4 ld_early16(const void* p) {
+  uint4 r;
+  asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+               : "l"(p));
+  return r;
+}
+
 // The same load with an L2 cache policy (createpolicy): evict-last for data
 // another CTA reads again soon, evict-first for data's last use.
 __device__ __forceinline__ uint4 ld_stream16_hint(const void* p, uint64_t pol) {

@@ -1,7 +1,9 @@
 // Fine Wilson-clover operator of Eq. (2): gauge import, clover term A_x
 // and the stencil apply (one thread per site and vector).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "async_copy.cuh"
 #include "kernels.cuh"
@@ -223,7 +225,8 @@ __device__ M3 field_strength(const cpx<double>* __restrict__ U, const Geom& g, i
 // so per chirality A = c_sw (i/2) [s1 (x) G1 + s2 (x) G2 + s3 (x) G3].
 // Clover term A_x of Eq. (2) (Sec. 3.2).
 __global__ void k_clover(const cpx<double>* __restrict__ U, Geom g, double csw,
-                         double* __restrict__ out64, float* __restrict__ out32) {
+                         double* __restrict__ out64, float* __restrict__ out32,
+                         float4* __restrict__ out32t) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= g.vol) return;
   int c[4];
@@ -267,6 +270,10 @@ __global__ void k_clover(const cpx<double>* __restrict__ U, Geom g, double csw,
     if (out32) {
       float* o32 = out32 + size_t(s) * 72 + chi * 36;
       for (int i = 0; i < 36; ++i) o32[i] = float(o64[i]);
+      // transposed: word w of every site adjacent
+      for (int w = 0; w < 9; ++w)
+        out32t[size_t(chi * 9 + w) * g.vol + s] = make_float4(
+            float(o64[4 * w]), float(o64[4 * w + 1]), float(o64[4 * w + 2]), float(o64[4 * w + 3]));
     }
   }
 }
@@ -280,6 +287,9 @@ __global__ void k_clover(const cpx<double>* __restrict__ U, Geom g, double csw,
 // vector-fastest, so the nvec CTAs of one site chunk run close together and
 // the chunk's links and clover come from DRAM once and from L2 for the
 // other vectors.
+// A: the clover, FP32 as 18 words of 16 B by site ([word][site]: adjacent
+// lanes read adjacent words; records of 288 B per lane cost eight times the
+// L1 wavefronts and bound the kernel), FP64 as records.
 // Eq. (2): the Wilson-clover matrix on one or several vectors.
 template <typename R, int LF, int MINB>
 __global__ void __launch_bounds__(128, MINB) k_wilson(cpx<R>* __restrict__ out, const cpx<R>* __restrict__ in,
@@ -343,9 +353,15 @@ __global__ void __launch_bounds__(128, MINB) k_wilson(cpx<R>* __restrict__ out, 
   {
     constexpr int W = sizeof(R) * 72 / 16;
     uint4 w[W];
-    const uint4* p = reinterpret_cast<const uint4*>(A + size_t(s) * 72);
+    if constexpr (std::is_same<R, float>::value) {
+      const uint4* p = reinterpret_cast<const uint4*>(A) + s;
 #pragma unroll
-    for (int i = 0; i < W; ++i) w[i] = __ldg(p + i);
+      for (int i = 0; i < W; ++i) w[i] = __ldg(p + size_t(i) * g.vol);
+    } else {
+      const uint4* p = reinterpret_cast<const uint4*>(A + size_t(s) * 72);
+#pragma unroll
+      for (int i = 0; i < W; ++i) w[i] = __ldg(p + i);
+    }
     clover_accum(reinterpret_cast<const R*>(w), diag, psi, acc);
   }
   const size_t V = g.vol;
@@ -563,10 +579,27 @@ __global__ void __launch_bounds__(128) k_wilson_tile(cpx<float>* __restrict__ ou
 // in the boxes' own order, x fastest): [interior][x-][x+][y-][y+][z-][z+]
 // [t-][t+] spinors, then [link mu interior] x 4, [x-][y-][z-][t-] links,
 // then (several vectors) the second spinor buffer.
-// Tensor maps (innermost first): spinors (24 floats, Lx, Ly, Lz, Lt nvec),
-// links (12 floats, Lx, Ly, Lz, 4 Lt) -- direction mu as time slices
-// mu Lt.. of the [mu][site] store.  Index 0: the interior box, 1 + mu: the
-// face box of direction mu (extent 1 in mu).
+//
+// What bounds it: with thread-private 16-byte accesses to records of 96 B
+// (spinors), 48 B (links) and 288 B (clover), the L1 data pipe, before HBM.
+// Three choices cut its wavefronts:
+//  * a record of 96 B starts at bank 0, 8, 16 or 24, so the eight lanes of
+//    a 16-byte phase collide two by two; lanes of every second group of four
+//    read the record's halves (chiralities) in the other order, 12 banks
+//    on, and keep the two halves exchanged throughout: the projections of
+//    directions 0..2 change sign for them (C_mu = -B_mu), those of direction
+//    3 do not (C_3 = B_3), and their accumulators hold the other chirality
+//    first (see hop_halves);
+//  * the clover is read from a transposed store, [word][site], where the
+//    16-byte words of consecutive sites are adjacent;
+//  * x is merged into the innermost tensor dimension, so a copy moves rows
+//    of BX records instead of single records.
+// Extents that the block does not divide leave partial blocks: the faces
+// sit at the valid extent, the rest of a box is zero-filled (or holds sites
+// nobody reads) and the surplus threads repeat a valid site without storing.
+// Tensor maps (innermost first): spinors (24 Lx floats, Ly, Lz, Lt, nvec),
+// links (12 Lx floats, Ly, Lz, Lt, 4).  Index 0: the interior box, 1 + mu:
+// the face box of direction mu (extent 1 in mu).
 struct WilsonTileMaps {
   CUtensorMap sp[5];
   CUtensorMap lk[5];
@@ -581,7 +614,6 @@ struct WilsonBlock {
   __host__ __device__ static constexpr int F(int mu) { return NS / B(mu); }  // face records
   static constexpr int NSP = NS + 2 * (F(0) + F(1) + F(2) + F(3));  // spinor records
   static constexpr int NLK = 4 * NS + F(0) + F(1) + F(2) + F(3);      // link records
-  static constexpr size_t SMEM = size_t(NSP) * 96 + size_t(NLK) * 48;
   // first record of spinor face (mu, side): side 0 at x_mu - 1, 1 at x_mu + B_mu
   __host__ __device__ static constexpr int face_sp(int mu, int side) {
     int o = NS;
@@ -594,209 +626,306 @@ struct WilsonBlock {
     for (int nu = 0; nu < mu; ++nu) o += F(nu);
     return o;
   }
+  // the same for a direction known at run time
+  __device__ static __forceinline__ int face_sp_rt(int mu, int side) {
+    const int f = mu == 0 ? F(0) : mu == 1 ? F(1) : mu == 2 ? F(2) : F(3);
+    return (mu == 0   ? face_sp(0, 0)
+            : mu == 1 ? face_sp(1, 0)
+            : mu == 2 ? face_sp(2, 0)
+                      : face_sp(3, 0)) +
+           side * f;
+  }
+  __device__ static __forceinline__ int face_lk_rt(int mu) {
+    return mu == 0 ? face_lk(0) : mu == 1 ? face_lk(1) : mu == 2 ? face_lk(2) : face_lk(3);
+  }
 };
 
-template <int BX, int BY, int BZ, int BT>
-__global__ void __launch_bounds__(BX * BY * BZ * BT, 3)
-    k_wilson_blk(cpx<float>* __restrict__ out, const float* __restrict__ A, Geom g, float diag,
-                 size_t vstride, int nvec, int antiperiodic,
+// One vector: a grid of resident CTAs walks the blocks, so that launch,
+// barrier set-up and the record offsets of a thread are paid once, not per
+// block.  Several vectors: a CTA per block (they amortise the set-up, and
+// static block lists measured 12 % slower).
+// Measured, 8x2x2x2 block: one 32^3x64 vector 318 -> 265 us (672 B/site with
+// two-row links: 5.3 TB/s), eight 24^3x48 vectors 491 -> 437 us.  L1
+// wavefronts fell from 65-70 to 38-45 % of their peak; what is left is
+// latency (issue slots 37-50 % busy with 6-10 warps per SM; two threads per
+// site doubled the warps and gained nothing).
+// MINB: resident CTAs per SM that the register budget allows; MULTI: several
+// vectors per launch.
+template <int BX, int BY, int BZ, int BT, int MINB, bool MULTI>
+__global__ void __launch_bounds__(BX * BY * BZ * BT, MINB)
+    k_wilson_blk(cpx<float>* __restrict__ out, const float4* __restrict__ A, Geom g, float diag,
+                 size_t vstride, int nvec, int antiperiodic, int nblocks,
                  const __grid_constant__ WilsonTileMaps maps, int* __restrict__ err) {
   using WB = WilsonBlock<BX, BY, BZ, BT>;
   constexpr int NS = WB::NS;
   extern __shared__ __align__(128) unsigned char wsm[];
   unsigned char* lk = wsm + size_t(WB::NSP) * 96;   // link records
-  // spinor buffers: vector v in buffer v & 1 (every offset a multiple of 128 B)
+  // spinor buffers, used in turn (every offset a multiple of 128 B)
   unsigned char* const sp0 = wsm;
-  unsigned char* const sp1 = lk + size_t(WB::NLK) * 48;
+  unsigned char* const sp1 = MULTI ? lk + size_t(WB::NLK) * 48 : wsm;
   __shared__ uint64_t bar[2];
-  const int tid = threadIdx.x;
-  const int st = tid;  // the thread's site in the block
-  // block origin and this thread's site
-  int o[4];
-  {
-    int b = blockIdx.x;
-    const int n0 = g.L[0] / BX, n1 = g.L[1] / BY, n2 = g.L[2] / BZ;
-    o[0] = (b % n0) * BX;
-    b /= n0;
-    o[1] = (b % n1) * BY;
-    b /= n1;
-    o[2] = (b % n2) * BZ;
-    o[3] = (b / n2) * BT;
-  }
-  const int l[4] = {st % BX, (st / BX) % BY, (st / (BX * BY)) % BZ, st / (BX * BY * BZ)};
-  const int lstride[4] = {1, BX, BX * BY, BX * BY * BZ};
-  const int site = (o[0] + l[0]) + g.L[0] * ((o[1] + l[1]) + g.L[1] * ((o[2] + l[2]) + g.L[2] * (o[3] + l[3])));
-  // face index of this site in the face boxes of mu (the other three
-  // coordinates, in order)
-  auto fidx = [&](int mu) {
-    int f = 0, m = 1;
-#pragma unroll
-    for (int nu = 0; nu < 4; ++nu)
-      if (nu != mu) {
-        f += l[nu] * m;
-        m *= WB::B(nu);
-      }
-    return f;
-  };
-  int nf[4], nb[4], lb[4];
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
-    nf[mu] = l[mu] + 1 < WB::B(mu) ? st + lstride[mu] : WB::face_sp(mu, 1) + fidx(mu);
-    nb[mu] = l[mu] > 0 ? st - lstride[mu] : WB::face_sp(mu, 0) + fidx(mu);
-    lb[mu] = l[mu] > 0 ? mu * NS + st - lstride[mu] : WB::face_lk(mu) + fidx(mu);
-  }
-  const bool tlast = antiperiodic && o[3] + l[3] == g.L[3] - 1;
-  const bool tfirst = antiperiodic && o[3] + l[3] == 0;
+  const int tid = threadIdx.x, lane = tid & 31;
   if (tid == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
     fence_mbar_init();
   }
   __syncthreads();
-  // wrapped coordinates of the faces
-  int wm[4], wp[4];
+  const int n0 = (g.L[0] + BX - 1) / BX, n1 = (g.L[1] + BY - 1) / BY,
+            n2 = (g.L[2] + BZ - 1) / BZ;
+  const bool even = g.L[0] % BX == 0 && g.L[1] % BY == 0 && g.L[2] % BZ == 0 && g.L[3] % BT == 0;
+  // which half of a record this lane reads first, and the sign that the
+  // exchange of halves brings to directions 0..2
+  const int swap = (tid >> 2) & 1;
+  const float sg = swap ? -1.f : 1.f;
+  const int h0 = swap * 48, h1 = 48 - h0;
+  // this thread's site in the block and the records of its neighbours and
+  // backward links, for a block of valid extents be
+  int l[4], st, nf[4], nb[4], lb[4];
+  bool valid;
+  auto place = [&](const int be[4]) {
+    l[0] = tid % BX;
+    l[1] = (tid / BX) % BY;
+    l[2] = (tid / (BX * BY)) % BZ;
+    l[3] = tid / (BX * BY * BZ);
+    valid = true;
 #pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
-    wm[mu] = o[mu] == 0 ? g.L[mu] - 1 : o[mu] - 1;
-    wp[mu] = o[mu] + WB::B(mu) == g.L[mu] ? 0 : o[mu] + WB::B(mu);
-  }
-  // the site's clover, loaded while the first copies are in flight
-  float clv[72];
-  {
-    const uint4* p = reinterpret_cast<const uint4*>(A + size_t(site) * 72);
+    for (int mu = 0; mu < 4; ++mu) {
+      valid = valid && l[mu] < be[mu];
+      l[mu] = min(l[mu], be[mu] - 1);
+    }
+    const int lstride[4] = {1, BX, BX * BY, BX * BY * BZ};
+    st = l[0] + BX * (l[1] + BY * (l[2] + BZ * l[3]));
 #pragma unroll
-    for (int i = 0; i < 18; ++i) reinterpret_cast<uint4*>(clv)[i] = __ldg(p + i);
-  }
-  const int Lt = g.L[3];
-  // thread 0: the tensor copies of vector v's spinor tile (and, for v = 0,
-  // of the links) into buffer v & 1, completing on barrier v & 1
-  auto issue = [&](int v) {
-    unsigned char* sp = (v & 1) ? sp1 : sp0;
-    uint64_t* b = (v & 1) ? &bar[1] : &bar[0];
-    // the reads of this buffer two vectors ago are ordered before the
-    // copies that overwrite it
-    fence_proxy_async_smem();
-    const uint32_t bytes = uint32_t(WB::NSP) * 96u + (v == 0 ? uint32_t(WB::NLK) * 48u : 0u);
-    mbar_arrive_expect_tx(b, bytes);
-    const int tv = v * Lt;
-    tma_load_5d(sp, &maps.sp[0], 0, o[0], o[1], o[2], o[3] + tv, b);
+    for (int mu = 0; mu < 4; ++mu) {
+      // index of the site in the face boxes of mu (the other coordinates, in order)
+      int f = 0, m = 1;
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu)
-#pragma unroll
-      for (int side = 0; side < 2; ++side) {
-        int c[4] = {o[0], o[1], o[2], o[3]};
-        c[mu] = side ? wp[mu] : wm[mu];
-        tma_load_5d(sp + size_t(WB::face_sp(mu, side)) * 96, &maps.sp[1 + mu], 0, c[0], c[1],
-                    c[2], c[3] + tv, b);
-      }
-    if (v == 0) {
-#pragma unroll
-      for (int mu = 0; mu < 4; ++mu)
-        tma_load_5d(lk + size_t(mu) * NS * 48, &maps.lk[0], 0, o[0], o[1], o[2], o[3] + mu * Lt,
-                    b);
-#pragma unroll
-      for (int mu = 0; mu < 4; ++mu) {
-        int c[4] = {o[0], o[1], o[2], o[3]};
-        c[mu] = wm[mu];
-        tma_load_5d(lk + size_t(WB::face_lk(mu)) * 48, &maps.lk[1 + mu], 0, c[0], c[1], c[2],
-                    c[3] + mu * Lt, b);
-      }
+      for (int nu = 0; nu < 4; ++nu)
+        if (nu != mu) {
+          f += l[nu] * m;
+          m *= WB::B(nu);
+        }
+      nf[mu] = l[mu] + 1 < be[mu] ? st + lstride[mu] : WB::face_sp(mu, 1) + f;
+      nb[mu] = l[mu] > 0 ? st - lstride[mu] : WB::face_sp(mu, 0) + f;
+      lb[mu] = l[mu] > 0 ? mu * NS + st - lstride[mu] : WB::face_lk(mu) + f;
     }
   };
-  if (tid == 0) issue(0);
-  for (int v = 0; v < nvec; ++v) {
-    // buffer (v + 1) & 1 was last read for vector v - 1, before the block
-    // barrier that ended that vector
-    if (tid == 0 && v + 1 < nvec) issue(v + 1);
-    const unsigned char* sp = (v & 1) ? sp1 : sp0;
-    if (!mbar_wait(&bar[v & 1], uint32_t((v >> 1) & 1))) {
-      // the copies did not land within the budget: record it, give the
-      // copies in flight (this vector's and the next one's) a second
-      // bounded wait and leave
-      if (tid == 0) {
-        atomicOr(err, 1);
-        mbar_wait(&bar[v & 1], uint32_t((v >> 1) & 1));
-        if (v + 1 < nvec) mbar_wait(&bar[(v + 1) & 1], uint32_t(((v + 1) >> 1) & 1));
-      }
-      return;
+  {
+    const int be[4] = {BX, BY, BZ, BT};
+    place(be);
+  }
+  // warp 0 issues the copies, one per lane: lane 0 the spinor interior, 1 +
+  // 2 mu + side its faces, 9 + mu the link interiors, 13 + mu the backward
+  // link faces
+  const bool is_link = lane >= 9, is_face = is_link ? lane >= 13 : lane > 0;
+  const int imu = !is_face ? 0 : is_link ? lane - 13 : (lane - 1) >> 1;  // face direction
+  const int iside = is_link ? 0 : (lane - 1) & 1;
+  const CUtensorMap* imap = (is_link ? maps.lk : maps.sp) + (is_face ? 1 + imu : 0);
+  uint32_t ioff = 0;  // destination, bytes from the start of its buffer
+  if (is_link) {
+    ioff = 48u * uint32_t(is_face ? WB::face_lk_rt(imu) : (lane - 9) * NS);
+  } else if (is_face) {
+    ioff = 96u * uint32_t(WB::face_sp_rt(imu, iside));
+  }
+  int it = 0;  // tiles issued and consumed so far: tile `it` in buffer it & 1 (MULTI) or 0
+  for (int blk = blockIdx.x; blk < nblocks; blk += gridDim.x) {
+    // block origin and valid extents
+    int o[4], be[4];
+    {
+      int b = blk;
+      o[0] = (b % n0) * BX;
+      b /= n0;
+      o[1] = (b % n1) * BY;
+      b /= n1;
+      o[2] = (b % n2) * BZ;
+      o[3] = (b / n2) * BT;
+#pragma unroll
+      for (int mu = 0; mu < 4; ++mu) be[mu] = min(WB::B(mu), g.L[mu] - o[mu]);
     }
-    cpx<float> psi[12], acc[12], u[9];
-    auto load_spinor = [&](int rec) {
-      const uint4* q = reinterpret_cast<const uint4*>(sp + size_t(rec) * 96);
+    int ic[4];
+    if (tid < 32) {
 #pragma unroll
-      for (int i = 0; i < 6; ++i) reinterpret_cast<uint4*>(psi)[i] = q[i];
-    };
-    auto load_link = [&](int rec, bool neg) {
-      const uint4* q = reinterpret_cast<const uint4*>(lk + size_t(rec) * 48);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) reinterpret_cast<uint4*>(u)[i] = q[i];
-      const float sg = neg ? -1.f : 1.f;
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const int b = (a + 1) % 3, cc = (a + 2) % 3;
-        u[6 + a] = sg * conj(u[b] * u[3 + cc] - u[cc] * u[3 + b]);
+      for (int mu = 0; mu < 4; ++mu) {
+        // a face sits at the wrapped coordinate next to the block
+        const int lo = o[mu] == 0 ? g.L[mu] - 1 : o[mu] - 1;
+        const int hi = o[mu] + be[mu] == g.L[mu] ? 0 : o[mu] + be[mu];
+        ic[mu] = is_face && mu == imu ? (iside ? hi : lo) : o[mu];
       }
+    }
+    // the copies of vector v's spinor tile (and, for v = 0, of the links)
+    // as tile k, completing on its buffer's barrier.  Every thread has passed
+    // a block barrier since that buffer (and, for v = 0, the links) was read;
+    // the fence orders those reads before the copies.
+    auto issue = [&](int v, int k) {
+      uint64_t* b = MULTI && (k & 1) ? &bar[1] : &bar[0];
+      if (lane == 0) {
+        fence_proxy_async_smem();
+        mbar_arrive_expect_tx(
+            b, uint32_t(WB::NSP) * 96u + (v == 0 ? uint32_t(WB::NLK) * 48u : 0u));
+      }
+      __syncwarp();
+      if (lane < (v == 0 ? 17 : 9))
+        tma_load_5d((is_link ? lk : (k & 1) ? sp1 : sp0) + ioff, imap,
+                    (is_link ? 12 : 24) * ic[0], ic[1], ic[2], ic[3],
+                    is_link ? (is_face ? imu : lane - 9) : v, b);
     };
-    load_spinor(st);
+    if (tid < 32) issue(0, it);
+    if (!even) place(be);
+    const int site = (o[0] + l[0]) +
+                     g.L[0] * ((o[1] + l[1]) + g.L[1] * ((o[2] + l[2]) + g.L[2] * (o[3] + l[3])));
+    const bool tlast = antiperiodic && o[3] + l[3] == g.L[3] - 1;
+    const bool tfirst = antiperiodic && o[3] + l[3] == 0;
+    // the site's clover, loaded while the first copies are in flight: the
+    // block of the first half's chirality, then the other
+    float clv[72];
+    {
+      const float4* a = A + size_t(swap * 9) * g.vol + site;
+      const float4* b = A + size_t((1 - swap) * 9) * g.vol + site;
 #pragma unroll
-    for (int i = 0; i < 12; ++i) acc[i] = cpx<float>(0.f, 0.f);
-    clover_accum(clv, diag, psi, acc);
-#define GB_BLK_HOP(MU)                         \
-  {                                            \
-    load_spinor(nf[MU]);                       \
-    load_link(MU * NS + st, MU == 3 && tlast); \
-    hop_accum<MU, true>(u, psi, acc);          \
-    load_spinor(nb[MU]);                       \
-    load_link(lb[MU], MU == 3 && tfirst);      \
-    hop_accum<MU, false>(u, psi, acc);         \
-  }
-    GB_BLK_HOP(0) GB_BLK_HOP(1) GB_BLK_HOP(2) GB_BLK_HOP(3)
+      for (int i = 0; i < 9; ++i, a += g.vol, b += g.vol) {
+        reinterpret_cast<uint4*>(clv)[i] = ld_early16(a);
+        reinterpret_cast<uint4*>(clv)[9 + i] = ld_early16(b);
+      }
+    }
+    for (int v = 0; v < (MULTI ? nvec : 1); ++v, ++it) {
+      // the other buffer was last read before the barrier that ended tile it - 1
+      if (MULTI && tid < 32 && v + 1 < nvec) issue(v + 1, it + 1);
+      const unsigned char* sp = (it & 1) ? sp1 : sp0;
+      uint64_t* wb = MULTI && (it & 1) ? &bar[1] : &bar[0];
+      const uint32_t ph = uint32_t(MULTI ? it >> 1 : it) & 1u;
+      if (!mbar_wait(wb, ph)) {
+        // the copies did not land within the budget: record it, give the
+        // copies in flight (this tile's and the next one's) a second bounded
+        // wait and leave
+        if (tid == 0) {
+          atomicOr(err, 1);
+          mbar_wait(wb, ph);
+          if (MULTI && v + 1 < nvec)
+            mbar_wait((it & 1) ? &bar[0] : &bar[1], uint32_t((it + 1) >> 1) & 1u);
+        }
+        return;
+      }
+      cpx<float> ax[6], ay[6];
+      // the operands of one hop: both halves of the neighbour and the link's
+      // two rows, loaded one hop ahead of their use
+      struct Hop {
+        uint4 x[3], y[3], k[3];
+      };
+      auto load_spinor = [&](int rec, Hop& q) {
+        const unsigned char* p = sp + size_t(rec) * 96;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) q.x[i] = reinterpret_cast<const uint4*>(p + h0)[i];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) q.y[i] = reinterpret_cast<const uint4*>(p + h1)[i];
+      };
+      auto load_hop = [&](int rec, int link, Hop& q) {
+        load_spinor(rec, q);
+        const uint4* p = reinterpret_cast<const uint4*>(lk + size_t(link) * 48);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) q.k[i] = p[i];
+      };
+      auto hop = [&](auto mu, auto fwd, const Hop& q, bool neg) {
+        cpx<float> u[9];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) reinterpret_cast<uint4*>(u)[i] = q.k[i];
+        const float sn = neg ? -1.f : 1.f;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int b = (a + 1) % 3, cc = (a + 2) % 3;
+          u[6 + a] = sn * conj(u[b] * u[3 + cc] - u[cc] * u[3 + b]);
+        }
+        hop_halves<decltype(mu)::value, decltype(fwd)::value>(
+            u, reinterpret_cast<const cpx<float>*>(q.x),
+            reinterpret_cast<const cpx<float>*>(q.y), ax, ay, sg);
+      };
+      Hop q[2];
+      load_spinor(st, q[1]);
+      if (MULTI) load_hop(nf[0], st, q[0]);
+#pragma unroll
+      for (int i = 0; i < 6; ++i) ax[i] = ay[i] = cpx<float>(0.f, 0.f);
+      clover_block_accum(clv, diag, reinterpret_cast<const cpx<float>*>(q[1].x), ax);
+      clover_block_accum(clv + 36, diag, reinterpret_cast<const cpx<float>*>(q[1].y), ay);
+      // (one vector: only now, when the clover's registers are free)
+      if (!MULTI) load_hop(nf[0], st, q[0]);
+#define GB_BLK_HOP(MU)                                                                \
+  load_hop(nb[MU], lb[MU], q[1]);                                                     \
+  hop(std::integral_constant<int, MU>{}, std::true_type{}, q[0], MU == 3 && tlast);   \
+  if (MU < 3) load_hop(nf[(MU + 1) & 3], (MU + 1) * NS + st, q[0]);                   \
+  hop(std::integral_constant<int, MU>{}, std::false_type{}, q[1], MU == 3 && tfirst);
+      GB_BLK_HOP(0) GB_BLK_HOP(1) GB_BLK_HOP(2) GB_BLK_HOP(3)
 #undef GB_BLK_HOP
-    uint4* op = reinterpret_cast<uint4*>(out + size_t(v) * vstride + size_t(site) * 12);
+      if (valid) {
+        unsigned char* op =
+            reinterpret_cast<unsigned char*>(out + size_t(v) * vstride + size_t(site) * 12);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) op[i] = reinterpret_cast<const uint4*>(acc)[i];
-    // every thread is done with the tile before the next vector's copies
-    __syncthreads();
+        for (int i = 0; i < 3; ++i) {
+          reinterpret_cast<uint4*>(op + h0)[i] = reinterpret_cast<const uint4*>(ax)[i];
+          reinterpret_cast<uint4*>(op + h1)[i] = reinterpret_cast<const uint4*>(ay)[i];
+        }
+      }
+      // every thread is done with the tile before the copies of another one
+      __syncthreads();
+    }
   }
+}
+
+// resident CTAs of the device for a kernel at a shared-memory size
+template <typename K>
+int resident_ctas(K kern, int threads, size_t smem) {
+  int dev = 0, sms = 0, per = 0;
+  GB_CHECK(cudaGetDevice(&dev));
+  GB_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  GB_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem));
+  return sms * (per > 0 ? per : 1);
 }
 
 // Host side of k_wilson_blk: the ten tensor maps (spinors of `in` over
 // nvec vectors stored back to back, two-row links) and the launch.
-template <int BX, int BY, int BZ, int BT>
+template <int BX, int BY, int BZ, int BT, int MINB, int MINM>
 void launch_wilson_blk(cpx<float>* out, const cpx<float>* in, const cpx<float>* U12,
-                       const float* A, const Geom& g, float diag, size_t vstride, int nvec,
+                       const float4* A, const Geom& g, float diag, size_t vstride, int nvec,
                        int ap, int* err, cudaStream_t st) {
   using WB = WilsonBlock<BX, BY, BZ, BT>;
   WilsonTileMaps m;
   const cuuint64_t X = g.L[0], Y = g.L[1], Z = g.L[2], T = g.L[3];
-  const cuuint64_t sd[5] = {24, X, Y, Z, T * cuuint64_t(nvec)};
-  const cuuint64_t ss[4] = {96, 96 * X, 96 * X * Y, 96 * X * Y * Z};
-  const cuuint64_t ld[5] = {12, X, Y, Z, 4 * T};
-  const cuuint64_t ls[4] = {48, 48 * X, 48 * X * Y, 48 * X * Y * Z};
-  const cuuint32_t box[5] = {24, BX, BY, BZ, BT};
-  const cuuint32_t lbox[5] = {12, BX, BY, BZ, BT};
+  const cuuint64_t sd[5] = {24 * X, Y, Z, T, cuuint64_t(nvec)};
+  const cuuint64_t ss[4] = {96 * X, 96 * X * Y, 96 * X * Y * Z, 96 * X * Y * Z * T};
+  const cuuint64_t ld[5] = {12 * X, Y, Z, T, 4};
+  const cuuint64_t ls[4] = {48 * X, 48 * X * Y, 48 * X * Y * Z, 48 * X * Y * Z * T};
+  const cuuint32_t box[5] = {24 * BX, BY, BZ, BT, 1};
+  const cuuint32_t lbox[5] = {12 * BX, BY, BZ, BT, 1};
   m.sp[0] = make_map_5d(in, sd, ss, box);
   m.lk[0] = make_map_5d(U12, ld, ls, lbox);
   for (int mu = 0; mu < 4; ++mu) {
-    cuuint32_t fb[5] = {24, BX, BY, BZ, BT}, fl[5] = {12, BX, BY, BZ, BT};
-    fb[1 + mu] = 1;
-    fl[1 + mu] = 1;
+    cuuint32_t fb[5] = {24 * BX, BY, BZ, BT, 1}, fl[5] = {12 * BX, BY, BZ, BT, 1};
+    fb[mu] = mu == 0 ? 24 : 1;
+    fl[mu] = mu == 0 ? 12 : 1;
     m.sp[1 + mu] = make_map_5d(in, sd, ss, fb);
     m.lk[1 + mu] = make_map_5d(U12, ld, ls, fl);
   }
-  auto k = k_wilson_blk<BX, BY, BZ, BT>;
+  // several vectors: shared memory allows few CTAs, so registers are not
+  // held down for more
+  auto k = nvec > 1 ? k_wilson_blk<BX, BY, BZ, BT, MINM, true>
+                    : k_wilson_blk<BX, BY, BZ, BT, MINB, false>;
   // several vectors: a second spinor buffer after the links
-  const size_t smem = WB::SMEM + (nvec > 1 ? size_t(WB::NSP) * 96 : 0);
+  const size_t smem =
+      size_t(WB::NSP) * 96 * (nvec > 1 ? 2 : 1) + size_t(WB::NLK) * 48;
   GB_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-  k<<<g.vol / WB::NS, WB::NS, smem, st>>>(out, A, g, diag, vstride, nvec, ap, m, err);
+  GB_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                cudaSharedmemCarveoutMaxShared));
+  const int blocks = ceil_div(g.L[0], BX) * ceil_div(g.L[1], BY) * ceil_div(g.L[2], BZ) *
+                     ceil_div(g.L[3], BT);
+  const int grid = nvec > 1 ? blocks : std::min(blocks, resident_ctas(k, WB::NS, smem));
+  k<<<grid, WB::NS, smem, st>>>(out, A, g, diag, vstride, nvec, ap, blocks, m, err);
 }
 
-// the tiled form needs block-divisible extents and 16-byte aligned operands
-bool wilson_blk_ok(const Geom& g, const int b[4], const void* in, const void* U, const void* A) {
+// the tiled form needs extents of at least a block and 16-byte aligned operands
+bool wilson_blk_ok(const Geom& g, const int b[4], const void* in, const void* out, const void* U) {
   for (int mu = 0; mu < 4; ++mu)
-    if (g.L[mu] % b[mu]) return false;
-  return reinterpret_cast<uintptr_t>(in) % 16 == 0 && reinterpret_cast<uintptr_t>(U) % 16 == 0 &&
-         reinterpret_cast<uintptr_t>(A) % 16 == 0;
+    if (g.L[mu] < b[mu]) return false;
+  return reinterpret_cast<uintptr_t>(in) % 16 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0 &&
+         reinterpret_cast<uintptr_t>(U) % 16 == 0;
 }
 }  // namespace
 
@@ -816,6 +945,7 @@ void fine_operator_build(mg_ctx* c, const void* gauge_ext, cudaStream_t st) {
     GB_LAUNCH_CHECK();
     L.clover32.alloc(size_t(L.g.vol) * 72 * sizeof(float));
     c32 = L.clover32.as<float>();
+    L.clover32t.alloc(size_t(L.g.vol) * 72 * sizeof(float));
     // two-row link form, used only if every link rebuilds to FP32 precision
     L.gauge12.alloc(size_t(4) * L.g.vol * 6 * sizeof(cpx<float>));
     DevBuf dev;
@@ -860,7 +990,8 @@ void fine_operator_build(mg_ctx* c, const void* gauge_ext, cudaStream_t st) {
     c->launches++;
   }
   k_clover<<<ceil_div(L.g.vol, 128), 128, 0, st>>>(L.gauge64.as<cpx<double>>(), L.g, c->p.csw,
-                                                    L.clover64.as<double>(), c32);
+                                                    L.clover64.as<double>(), c32,
+                                                    L.clover32t.as<float4>());
   GB_LAUNCH_CHECK();
   c->launches += L.prec == MG_F32 ? 3 : 2;
   L.diag = 4.0 + c->p.mass;
@@ -886,10 +1017,12 @@ void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st) {
     //   8 / 9   links (stored / two-row) and clover of 32 sites staged in
     //           shared memory, warps looping over the vectors (nvec >= 4)
     //   10 / 11 8-real links, default registers / at least 4 CTAs per SM
-    //   12 / 13 tiled: a 4x4x4x2 / 4x4x2x2 block with its halo staged in
-    //           shared memory by tensor copies (two-row links)
+    //   12 .. 15 tiled: a 4x4x4x2 / 4x4x2x2 / 8x2x2x2 / 8x4x2x2 block with
+    //           its halo staged in shared memory by tensor copies (two-row
+    //           links)
     // Two-row and 8-real policies are candidates only when the field allows
-    // them; tiled ones when the extents divide into blocks.
+    // them; tiled ones when every extent holds a block (extents it does not
+    // divide leave partial blocks).
     GB_REQUIRE(L.gauge32.p, MG_ERR_STATE, "FP32 fine operator not built");
     const unsigned gx = ceil_div(L.g.vol, 128);
     const int ap = c->p.t_antiperiodic;
@@ -897,6 +1030,8 @@ void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st) {
     const cpx<float>* U12 = L.gauge12.as<cpx<float>>();
     const cpx<float>* U8 = L.gauge8.as<cpx<float>>();
     const float* A = L.clover32.as<float>();
+    const float4* At = L.clover32t.as<float4>();
+    const float* Ac = L.clover32t.as<float>();
     auto* o = (cpx<float>*)out.p;
     auto* i = (const cpx<float>*)in.p;
     const float dg = float(L.diag);
@@ -904,29 +1039,31 @@ void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st) {
     int* err = c->status.as<int>() + 1;
     auto launch = [&](int q) {
       switch (q) {
-        case 1: k_wilson<float, 12, 0><<<grid, 128, 0, st>>>(o, i, U12, A, L.g, dg, vs, nvec, ap); break;
-        case 2: k_wilson<float, 18, 2><<<grid, 128, 0, st>>>(o, i, U18, A, L.g, dg, vs, nvec, ap); break;
-        case 3: k_wilson<float, 12, 2><<<grid, 128, 0, st>>>(o, i, U12, A, L.g, dg, vs, nvec, ap); break;
-        case 4: k_wilson<float, 12, 4><<<grid, 128, 0, st>>>(o, i, U12, A, L.g, dg, vs, nvec, ap); break;
-        case 5: k_wilson<float, 12, 6><<<grid, 128, 0, st>>>(o, i, U12, A, L.g, dg, vs, nvec, ap); break;
+        case 1: k_wilson<float, 12, 0><<<grid, 128, 0, st>>>(o, i, U12, Ac, L.g, dg, vs, nvec, ap); break;
+        case 2: k_wilson<float, 18, 2><<<grid, 128, 0, st>>>(o, i, U18, Ac, L.g, dg, vs, nvec, ap); break;
+        case 3: k_wilson<float, 12, 2><<<grid, 128, 0, st>>>(o, i, U12, Ac, L.g, dg, vs, nvec, ap); break;
+        case 4: k_wilson<float, 12, 4><<<grid, 128, 0, st>>>(o, i, U12, Ac, L.g, dg, vs, nvec, ap); break;
+        case 5: k_wilson<float, 12, 6><<<grid, 128, 0, st>>>(o, i, U12, Ac, L.g, dg, vs, nvec, ap); break;
         case 6: k_wilson_mv<float, 2><<<dim3(gx, nvec / 2), 128, 0, st>>>(o, i, U18, A, L.g, dg, vs); break;
         case 7: k_wilson_mv<float, 4><<<dim3(gx, nvec / 4), 128, 0, st>>>(o, i, U18, A, L.g, dg, vs); break;
         case 8: k_wilson_tile<false><<<gt, 128, 0, st>>>(o, i, U18, A, L.g, dg, vs, nvec, ap); break;
         case 9: k_wilson_tile<true><<<gt, 128, 0, st>>>(o, i, U12, A, L.g, dg, vs, nvec, ap); break;
-        case 10: k_wilson<float, 8, 0><<<grid, 128, 0, st>>>(o, i, U8, A, L.g, dg, vs, nvec, ap); break;
-        case 11: k_wilson<float, 8, 4><<<grid, 128, 0, st>>>(o, i, U8, A, L.g, dg, vs, nvec, ap); break;
-        case 12: launch_wilson_blk<4, 4, 4, 2>(o, i, U12, A, L.g, dg, vs, nvec, ap, err, st); break;
-        case 13: launch_wilson_blk<4, 4, 2, 2>(o, i, U12, A, L.g, dg, vs, nvec, ap, err, st); break;
-        default: k_wilson<float, 18, 0><<<grid, 128, 0, st>>>(o, i, U18, A, L.g, dg, vs, nvec, ap); break;
+        case 10: k_wilson<float, 8, 0><<<grid, 128, 0, st>>>(o, i, U8, Ac, L.g, dg, vs, nvec, ap); break;
+        case 11: k_wilson<float, 8, 4><<<grid, 128, 0, st>>>(o, i, U8, Ac, L.g, dg, vs, nvec, ap); break;
+        case 12: launch_wilson_blk<4, 4, 4, 2, 3, 2>(o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
+        case 13: launch_wilson_blk<4, 4, 2, 2, 6, 3>(o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
+        case 14: launch_wilson_blk<8, 2, 2, 2, 6, 3>(o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
+        case 15: launch_wilson_blk<8, 4, 2, 2, 3, 2>(o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
+        default: k_wilson<float, 18, 0><<<grid, 128, 0, st>>>(o, i, U18, Ac, L.g, dg, vs, nvec, ap); break;
       }
     };
     std::vector<int> cands = {0, 2};
     if (L.gauge12_ok) cands.insert(cands.end(), {1, 3, 4, 5});
     if (L.gauge8_ok) cands.insert(cands.end(), {10, 11});
     if (L.gauge12_ok) {
-      const int b12[4] = {4, 4, 4, 2}, b13[4] = {4, 4, 2, 2};
-      if (wilson_blk_ok(L.g, b12, i, U12, A)) cands.push_back(12);
-      if (wilson_blk_ok(L.g, b13, i, U12, A)) cands.push_back(13);
+      const int blk[4][4] = {{4, 4, 4, 2}, {4, 4, 2, 2}, {8, 2, 2, 2}, {8, 4, 2, 2}};
+      for (int k = 0; k < 4; ++k)
+        if (wilson_blk_ok(L.g, blk[k], i, o, U12)) cands.push_back(12 + k);
     }
     if (nvec % 2 == 0) cands.push_back(6);
     if (nvec % 4 == 0) cands.push_back(7);

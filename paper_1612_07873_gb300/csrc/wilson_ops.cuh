@@ -99,6 +99,58 @@ __device__ __forceinline__ void hop_accum(const cpx<R>* __restrict__ U, const cp
   }
 }
 
+// hop_accum on a spinor and an accumulator kept as two halves of one
+// chirality each, first the upper (sg = 1) or the lower half (sg = -1).  With
+// CB = 1 the projection (1 -+ g) psi = [h; -+C h], h = psi_u -+ B psi_l, reads
+// [-+B h'; h'] with h' = psi_l -+ C psi_u from the lower half, and C_mu =
+// -B_mu for mu < 3, C_3 = B_3: the same steps with the sign sg on the terms
+// that cross the halves, for mu < 3.
+template <int MU, bool FWD, typename R>
+__device__ __forceinline__ void hop_halves(const cpx<R>* __restrict__ U, const cpx<R> x[6],
+                                           const cpx<R> y[6], cpx<R> ax[6], cpx<R> ay[6], R sg) {
+  cpx<R> h[2][3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    cpx<R> b[2];
+    Bmul<MU>(y[k], y[3 + k], b[0], b[1]);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      if constexpr (MU == 3) {
+        h[s][k] = FWD ? x[3 * s + k] - b[s] : x[3 * s + k] + b[s];
+      } else {
+        h[s][k] = cpx<R>(fma(FWD ? -sg : sg, b[s].re, x[3 * s + k].re),
+                         fma(FWD ? -sg : sg, b[s].im, x[3 * s + k].im));
+      }
+    }
+  }
+  const R half = R(0.5), hs = MU == 3 ? half : half * sg;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    cpx<R> w[2], c[2];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      cpx<R> t(R(0), R(0));
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        if (FWD)
+          cmac(t, U[a * 3 + b], h[s][b]);
+        else
+          cmac_conj(t, U[b * 3 + a], h[s][b]);  // (U^dag)_{ab} = conj(U_{ba})
+      }
+      w[s] = t;
+    }
+    Cmul<MU>(w[0], w[1], c[0], c[1]);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      ax[3 * s + a] -= half * w[s];
+      if (FWD)
+        ay[3 * s + a] += hs * c[s];
+      else
+        ay[3 * s + a] -= hs * c[s];
+    }
+  }
+}
+
 // Runtime-mu dispatch of hop_accum.
 template <typename R>
 __device__ __forceinline__ void hop_accum_rt(int mu, bool fwd, const cpx<R>* __restrict__ U,

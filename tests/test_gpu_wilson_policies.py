@@ -202,3 +202,30 @@ def test_tiled_policy_in_setup(gpu_lib, policy):
     assert err < 1e-5, (policy, err)
     gb.mg_tune_set(f"wilson/v{vol}/n{nv}/c1", -1)
     mg.close()
+
+
+@pytest.mark.parametrize("nrhs", [1, 3])
+@pytest.mark.parametrize("dims", [(10, 6, 6, 6), (8, 4, 4, 2), (14, 10, 4, 4)])
+@pytest.mark.parametrize("policy", [12, 13, 14, 15])
+def test_tiled_policy_partial_blocks(gpu_lib, policy, dims, nrhs):
+    """Extents that the block does not divide (partial blocks at the upper
+    faces, their neighbours at the wrapped coordinates) and extents equal to
+    the block's, one and several vectors, against the oracle."""
+    gb = gpu_lib
+    vol = lat.volume(dims)
+    key = f"wilson/v{vol}/n{nrhs}/c1"
+    gb.mg_tune_set(key, policy)
+    mg, U = make_ctx(gb, dims, [(2, 2, 2, 2)], [2], prec_fine=1, prec_coarse=1, eps=0.5)
+    psi = syn.gaussian_field((nrhs, vol, 12), 79)
+    out = torch.full(psi.shape, float("nan"), dtype=torch.complex64, device="cuda")
+    if nrhs == 1:
+        gb.mg_wilson_clover_apply(mg.ctx, out, to_dev(psi, torch.complex64))
+    else:
+        gb.mg_wilson_clover_apply_multi(mg.ctx, out, to_dev(psi, torch.complex64), nrhs)
+    gb.mg_device_status(mg.ctx)
+    assert gb.mg_tune_get(key) == policy
+    op = oracle_fine(U, dims)
+    err = rel_l2(to_np(out), np.stack([op.apply(p) for p in psi]))
+    assert err < 1e-5, (policy, err)
+    gb.mg_tune_set(key, -1)
+    mg.close()
