@@ -241,6 +241,21 @@ __device__ __forceinline__ uint4 ld_stream16(const void* p) {
   return r;
 }
 
+// Read-only 32-byte load (sm_100 and later; 32-byte aligned): a warp's access
+// to records of 96 B touches each of their cache lines once per instruction,
+// so wider words mean fewer passes of the L1 data pipe.
+__device__ __forceinline__ void ld_nc32(const void* p, float v[8]) {
+  asm volatile("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]),
+                 "=f"(v[6]), "=f"(v[7])
+               : "l"(p));
+}
+__device__ __forceinline__ void st32(void* p, const float v[8]) {
+  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]),
+               "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+
 // A read-only 16-byte load that stays where it is written (ahead of a wait).
 __device__ __forceinline__ uint4 ld_early16(const void* p) {
   uint4 r;

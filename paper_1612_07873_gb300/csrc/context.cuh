@@ -119,6 +119,10 @@ struct Level {
   // Hermitian 6x6 chirality blocks, [V/2][72] reals; coarse: [V/2][col][row]
   // complex), both in the vector precision
   DevBuf ainv, xinv;
+  // FP32 two-row fine level: the operator of the red-black kernels by parity,
+  // 16-byte words of consecutive compact sites adjacent -- links
+  // [parity][mu][3][V/2], clover [parity][18][V/2], A_e^-1 [18][V/2]
+  DevBuf eo_links, eo_clover, eo_ainv;
   bool have_schur = false;
   bool have_raw = false, have_V = false;
 

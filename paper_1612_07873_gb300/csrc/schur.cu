@@ -15,6 +15,8 @@
 // fused epilogue (EoMode): H in, A^-1 H in, A xc - H in, xc - H in,
 // A^-1 (xc - H in).  S costs two launches (A^-1 H on the even sites, then
 // A xc - H on the odd ones).
+#include <type_traits>
+
 #include "coarse_ops.cuh"
 #include "kernels.cuh"
 #include "wilson_ops.cuh"
@@ -136,6 +138,131 @@ __global__ void __launch_bounds__(128) k_wilson_eo(cpx<R>* __restrict__ out,
   uint4* o = reinterpret_cast<uint4*>(out + size_t(h) * 12);
 #pragma unroll
   for (int i = 0; i < int(sizeof(cpx<R>) * 12 / 16); ++i) o[i] = reinterpret_cast<const uint4*>(y)[i];
+}
+
+// The same hops and epilogues for FP32 two-row links from the by-parity
+// transposed stores.  Reading records per lane (96 B spinors, 48 B links at
+// every other site, 288 B clover) bound k_wilson_eo by the L1 data pipe
+// (81-90 % of its peak: each 16-byte word of a record costs a pass over 24 to
+// 36 cache lines per warp).  Here the links, the clover and A^-1 are read
+// from stores in which the words of consecutive compact sites are adjacent,
+// and the spinor records in 32-byte words: about a third of the passes.
+// CTAs are ordered vector-fastest, so several vectors share the operator
+// through L2.
+// Sec. 3.3: the hops of Eq. (2) between parities, fused epilogue.
+template <int MODE>
+__global__ void __launch_bounds__(128, 4)
+    k_wilson_eo_t(float* __restrict__ out, const float* __restrict__ in,
+                  const float* __restrict__ xc, const uint4* __restrict__ links,
+                  const uint4* __restrict__ site_op, Geom g, float diag, int p, int nvec,
+                  size_t hstride, int antiperiodic) {
+  const int vec = blockIdx.x % nvec;
+  const int h = (blockIdx.x / nvec) * blockDim.x + threadIdx.x;
+  const int vh = g.vol >> 1;
+  if (h >= vh) return;
+  const size_t off = size_t(vec) * hstride * 2;
+  in += off;
+  out += off;
+  const int s = eo_site(g, h, p);
+  int c[4];
+  site_coords(g, s, c);
+  cpx<float> acc[12];
+#pragma unroll
+  for (int i = 0; i < 12; ++i) acc[i] = cpx<float>(0.f, 0.f);
+  auto load_spinor = [&](const float* base, int hh, cpx<float> psi[12]) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      ld_nc32(base + size_t(hh) * 24 + 8 * i, reinterpret_cast<float*>(psi) + 8 * i);
+  };
+  auto hop = [&](auto muc, auto fwdc, int hh, const uint4* lp, bool neg) {
+    cpx<float> psi[12], u[9];
+    uint4 w[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) w[i] = __ldg(lp + size_t(i) * vh);
+    load_spinor(in, hh, psi);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) u[i] = reinterpret_cast<const cpx<float>*>(w)[i];
+    const float sg = neg ? -1.f : 1.f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int b = (a + 1) % 3, cc = (a + 2) % 3;
+      u[6 + a] = sg * conj(u[b] * u[3 + cc] - u[cc] * u[3 + b]);
+    }
+    hop_accum<decltype(muc)::value, decltype(fwdc)::value>(u, psi, acc);
+  };
+  const bool tlast = antiperiodic && c[3] == g.L[3] - 1, tfirst = antiperiodic && c[3] == 0;
+  // forward links of this parity, backward links of the other one
+  const uint4* lf = links + size_t(p) * 12 * vh + h;
+  const uint4* lb = links + size_t(1 - p) * 12 * vh;
+#define GB_EOT_HOP(MU)                                                                          \
+  {                                                                                             \
+    const int hf = neighbour(g, s, c, 1 + 2 * MU) >> 1;                                         \
+    hop(std::integral_constant<int, MU>{}, std::true_type{}, hf, lf + size_t(3 * MU) * vh,      \
+        MU == 3 && tlast);                                                                      \
+    const int hb = neighbour(g, s, c, 2 + 2 * MU) >> 1;                                         \
+    hop(std::integral_constant<int, MU>{}, std::false_type{}, hb, lb + size_t(3 * MU) * vh + hb, \
+        MU == 3 && tfirst);                                                                     \
+  }
+  GB_EOT_HOP(0) GB_EOT_HOP(1) GB_EOT_HOP(2) GB_EOT_HOP(3)
+#undef GB_EOT_HOP
+  auto site_apply = [&](float dg, const cpx<float> x[12], cpx<float> y[12]) {
+#pragma unroll
+    for (int chi = 0; chi < 2; ++chi) {
+      uint4 w[9];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) w[i] = __ldg(site_op + size_t(chi * 9 + i) * vh + h);
+      clover_block_accum(reinterpret_cast<const float*>(w), dg, x + 6 * chi, y + 6 * chi);
+    }
+  };
+  cpx<float> y[12];
+  if constexpr (MODE == EO_HOP) {
+#pragma unroll
+    for (int i = 0; i < 12; ++i) y[i] = acc[i];
+  } else if constexpr (MODE == EO_AINV_HOP) {
+#pragma unroll
+    for (int i = 0; i < 12; ++i) y[i] = cpx<float>(0.f, 0.f);
+    site_apply(0.f, acc, y);
+  } else {
+    cpx<float> psi[12];
+    load_spinor(xc + off, h, psi);
+    if constexpr (MODE == EO_A_XC_MINUS_HOP) {
+#pragma unroll
+      for (int i = 0; i < 12; ++i) y[i] = -acc[i];
+      site_apply(diag, psi, y);
+    } else if constexpr (MODE == EO_XC_MINUS_HOP) {
+#pragma unroll
+      for (int i = 0; i < 12; ++i) y[i] = psi[i] - acc[i];
+    } else {  // EO_AINV_XC_MINUS_HOP
+#pragma unroll
+      for (int i = 0; i < 12; ++i) {
+        acc[i] = psi[i] - acc[i];
+        y[i] = cpx<float>(0.f, 0.f);
+      }
+      site_apply(0.f, acc, y);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+    st32(out + size_t(h) * 24 + 8 * i, reinterpret_cast<const float*>(y) + 8 * i);
+}
+
+// The by-parity transposed stores of k_wilson_eo_t: two-row links, clover
+// records and A_e^-1 records (one thread per compact site and parity).
+// Sec. 3.3: the fine operator by parity.
+__global__ void k_eo_transpose(uint4* __restrict__ links, uint4* __restrict__ clover,
+                               uint4* __restrict__ ainvt, const uint4* __restrict__ U12,
+                               const uint4* __restrict__ A, const uint4* __restrict__ ainv,
+                               Geom g) {
+  const int vh = g.vol >> 1;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= g.vol) return;
+  const int p = t / vh, h = t - p * vh;
+  const int s = eo_site(g, h, p);
+  for (int k = 0; k < 12; ++k)  // k = 3 mu + word
+    links[(size_t(p) * 12 + k) * vh + h] = U12[(size_t(k / 3) * g.vol + s) * 3 + k % 3];
+  for (int k = 0; k < 18; ++k) clover[(size_t(p) * 18 + k) * vh + h] = A[size_t(s) * 18 + k];
+  if (p == 0)
+    for (int k = 0; k < 18; ++k) ainvt[size_t(k) * vh + h] = ainv[size_t(h) * 18 + k];
 }
 
 // (4 + m + A_x)^-1 for the even sites: two 6x6 Hermitian chirality blocks,
@@ -522,6 +649,8 @@ void coarse_eo(const Level& L, Vec out, Vec in, const void* xc, int p, cudaStrea
   GB_REQUIRE(ok, MG_ERR_ARG, "red-black: unsupported coarse dof count");
 }
 
+bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
+
 template <int MODE>
 void fine_eo(mg_ctx* c, Vec out, Vec in, const void* xc, int p, cudaStream_t st) {
   Level& L = c->L[0];
@@ -532,7 +661,15 @@ void fine_eo(mg_ctx* c, Vec out, Vec in, const void* xc, int p, cudaStream_t st)
         (cpx<double>*)out.p, (const cpx<double>*)in.p, (const cpx<double>*)xc,
         L.gauge64.as<cpx<double>>(), L.clover64.as<double>(), L.ainv.as<double>(), L.g, L.diag,
         p, in.n, ap);
-  else if (L.gauge12_ok)  // two-row links: a third fewer link bytes, read twice per S
+  else if (L.gauge12_ok && aligned32(out.p) && aligned32(in.p) && (!xc || aligned32(xc)))
+    // two-row links from the transposed stores: 24^3x48, one vector, both
+    // kernels of S 156 -> 100 us (floor 84 us: every link is read by both)
+    k_wilson_eo_t<MODE><<<ceil_div(L.g.vol / 2, 128) * in.nr, 128, 0, st>>>(
+        (float*)out.p, (const float*)in.p, (const float*)xc, L.eo_links.as<uint4>(),
+        MODE == EO_A_XC_MINUS_HOP ? L.eo_clover.as<uint4>() + size_t(p) * 9 * L.g.vol
+                                  : L.eo_ainv.as<uint4>(),
+        L.g, float(L.diag), p, in.nr, in.n, ap);
+  else if (L.gauge12_ok)  // vectors off 32-byte boundaries: records by 16-byte words
     k_wilson_eo<float, MODE, true><<<grid, 128, 0, st>>>(
         (cpx<float>*)out.p, (const cpx<float>*)in.p, (const cpx<float>*)xc,
         L.gauge12.as<cpx<float>>(), L.clover32.as<float>(), L.ainv.as<float>(), L.g,
@@ -570,6 +707,16 @@ void schur_prepare(mg_ctx* c, int level, cudaStream_t st) {
       L.ainv.alloc(n * sizeof(float));
       k_clover_inverse<float><<<ceil_div(L.g.vol, 128), 128, 0, st>>>(
           L.ainv.as<float>(), L.clover64.as<double>(), L.g, L.diag, c->status.as<int>());
+      if (L.gauge12_ok) {
+        GB_LAUNCH_CHECK();
+        L.eo_links.alloc(size_t(L.g.vol) * 12 * 16);
+        L.eo_clover.alloc(size_t(L.g.vol) * 18 * 16);
+        L.eo_ainv.alloc(size_t(vh) * 18 * 16);
+        k_eo_transpose<<<ceil_div(L.g.vol, 128), 128, 0, st>>>(
+            L.eo_links.as<uint4>(), L.eo_clover.as<uint4>(), L.eo_ainv.as<uint4>(),
+            L.gauge12.as<uint4>(), L.clover32.as<uint4>(), L.ainv.as<uint4>(), L.g);
+        c->launches++;
+      }
     }
   } else {
     GB_REQUIRE(L.have_op && L.links.p, MG_ERR_STATE, "red-black: coarse operator missing");

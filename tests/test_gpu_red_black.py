@@ -143,3 +143,26 @@ def test_odd_extent_level_has_no_red_black_form(gpu_lib):
     st = gb.mg_gcr_solve(mg.ctx, xs, b, 1e-10, 200)
     assert st["true_residual"] <= 1e-10
     mg.close()
+
+
+@pytest.mark.parametrize("offset", [0, 2])
+@pytest.mark.parametrize("special", [True, False])
+@pytest.mark.parametrize("dims,nr", [((4, 6, 2, 10), 3), ((14, 2, 8, 4), 1)])
+def test_schur_apply_fine_stores(gpu_lib, dims, nr, special, offset):
+    """The FP32 red-black kernels against the oracle: by-parity transposed
+    stores (SU(3) links, vectors on 32-byte boundaries), records (vectors 16
+    bytes off: offset 2 complex numbers; links off SU(3)); a last thread
+    block that is partly filled, several vectors."""
+    gb = gpu_lib
+    U = syn.gauge_field(dims, 0.5, 94) * (1.0 if special else 1.05)
+    mg, _ = make_ctx(gb, dims, [(2, 2, 2, 2)], [2], prec_fine=1, prec_coarse=1, U=U, red_black=1)
+    S = rb.SchurOp(dirac.wilson_clover_op(U, dims, -0.2, 1.0, True))
+    x = syn.gaussian_field((nr, lat.volume(dims) // 2, 12), 95)
+    bx = torch.zeros(x.size + 4, dtype=torch.complex64, device="cuda")
+    by = torch.zeros_like(bx)
+    xd, yd = bx[offset:offset + x.size].view(x.shape), by[offset:offset + x.size].view(x.shape)
+    xd.copy_(to_dev(x, torch.complex64))
+    gb.mg_schur_apply(mg.ctx, 0, yd, xd, nrhs=nr)
+    err = rel_l2(to_np(yd), np.stack([S.apply(v) for v in x]))
+    assert err < 1e-5, err
+    mg.close()
