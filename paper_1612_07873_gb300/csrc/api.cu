@@ -391,12 +391,15 @@ mg_status mg_schur_apply(mg_ctx* c, int level, void* y, const void* x, int nrhs,
     vx.prec = vy.prec = vt.prec = L.vprec;
     vx.n = vy.n = vt.n = L.vec_elems() / 2;
     vx.nr = vy.nr = vt.nr = nrhs;
-    DevBuf tmp;
-    tmp.alloc(L.vec_bytes() / 2 * nrhs);
+    // (refused inside a stream capture: the temporary belongs to this call)
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    GB_CHECK(cudaStreamIsCapturing(S(stream), &cs));
+    GB_REQUIRE(cs == cudaStreamCaptureStatusNone, MG_ERR_CUDA,
+               "schur_apply: not possible inside a stream capture");
+    TempBuf tmp(c->temps, L.vec_bytes() / 2 * nrhs, S(stream));
     vt.p = tmp.p;
     eo_apply(c, level, EO_AINV_HOP, vt, vx, nullptr, 0, S(stream));
     eo_apply(c, level, EO_A_XC_MINUS_HOP, vy, vt, x, 1, S(stream));
-    GB_CHECK(cudaStreamSynchronize(S(stream)));
   });
 }
 

@@ -3,6 +3,7 @@
 #pragma once
 
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -37,6 +38,46 @@ struct DevBuf {
   }
   template <typename T>
   T* as() const { return static_cast<T*>(p); }
+};
+
+// Temporary device memory of a context's calls: stream-ordered allocations
+// from a memory pool of the context's device.  The pool orders the reuse of a
+// block behind its last user's stream, so calls on several streams or threads
+// never share one; it keeps up to `kKeep` bytes between calls, gives the rest
+// back, and is destroyed with the context.
+struct TempPool {
+  static constexpr unsigned long long kKeep = 1ull << 30;
+  cudaMemPool_t pool = nullptr;
+  std::once_flag once;
+  ~TempPool() {
+    if (pool) cudaMemPoolDestroy(pool);
+  }
+  void* get(size_t n, cudaStream_t st) {
+    std::call_once(once, [&] {
+      cudaMemPoolProps pr = {};
+      pr.allocType = cudaMemAllocationTypePinned;
+      pr.location.type = cudaMemLocationTypeDevice;
+      GB_CHECK(cudaGetDevice(&pr.location.id));
+      GB_CHECK(cudaMemPoolCreate(&pool, &pr));
+      unsigned long long keep = kKeep;
+      GB_CHECK(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
+    });
+    void* p = nullptr;
+    if (cudaMallocFromPoolAsync(&p, n, pool, st) != cudaSuccess) {
+      cudaGetLastError();
+      throw Error(MG_ERR_OOM, "temporary of " + std::to_string(n) + " bytes failed");
+    }
+    return p;
+  }
+};
+// One temporary, freed in stream order at the end of the scope.
+struct TempBuf {
+  void* p;
+  cudaStream_t st;
+  TempBuf(TempPool& pool, size_t n, cudaStream_t s) : p(pool.get(n, s)), st(s) {}
+  TempBuf(const TempBuf&) = delete;
+  TempBuf& operator=(const TempBuf&) = delete;
+  ~TempBuf() { cudaFreeAsync(p, st); }
 };
 
 // One recorded launch of an instrumented kernel class.
@@ -158,6 +199,7 @@ struct mg_ctx {
   gbmg::DevBuf batch_partials; // batched reductions: [nvec][2][blocks] double2
   gbmg::DevBuf batch_scalars;  // batched reductions: [2 * 64] double2
   double* h_scalars = nullptr; // pinned host mirror
+  gbmg::TempPool temps;        // temporaries of single calls
   // solver workspace (allocated on first solve)
   struct SolverWS;
   std::unique_ptr<SolverWS> ws;

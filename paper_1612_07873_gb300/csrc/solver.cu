@@ -388,15 +388,24 @@ void setup_sweeps(mg_ctx* c, int l, const void* init, cudaStream_t st) {
   const int nv = L.nvec;
   const size_t n = L.vec_elems();
   GB_REQUIRE(nv <= 64, MG_ERR_ARG, "setup: at most 64 null vectors");
-  L.raw.alloc(size_t(nv) * n * 16);
-  // all nv vectors back to back: X[v] at offset v * n
-  DevBuf xb, tb, qb;
-  const size_t bytes = size_t(nv) * n * prec_bytes_complex(L.vprec);
-  xb.alloc(bytes);
-  tb.alloc(bytes);
-  qb.alloc(bytes);
-  Vec X = vbuf(xb, L.vprec, n), T = vbuf(tb, L.vprec, n), Q = vbuf(qb, L.vprec, n);
-  Vec Xall = vbuf(xb, L.vprec, n * nv);
+  // all nv vectors back to back: X[v] at offset v * n.  The sweeps work in
+  // the buffers that this setup fills at its end anyway (raw vectors, blocked
+  // orthonormal vectors, prolongator), so a repeated setup allocates nothing:
+  // 16 B per entry in raw and orth64, the vector precision's size in Vp.
+  const size_t elems = size_t(nv) * n, bytes = elems * prec_bytes_complex(L.vprec);
+  L.raw.alloc(elems * 16);
+  L.orth64.alloc(elems * 16);
+  L.Vp.alloc(bytes);
+  L.have_raw = L.have_V = false;
+  const bool f64 = L.vprec == MG_F64;
+  auto at = [&](DevBuf& b, size_t off, size_t len) {
+    Vec v = vbuf(b, L.vprec, len);
+    v.p = static_cast<char*>(b.p) + off;
+    return v;
+  };
+  Vec X = at(L.orth64, 0, n), Xall = at(L.orth64, 0, n * nv);
+  Vec T = f64 ? at(L.Vp, 0, n) : at(L.orth64, bytes, n);
+  Vec Q = f64 ? at(L.raw, 0, n) : at(L.Vp, 0, n);
   Vec raw = vbuf(L.raw, MG_F64, n * nv);
   if (init) {
     Vec in;
@@ -411,17 +420,13 @@ void setup_sweeps(mg_ctx* c, int l, const void* init, cudaStream_t st) {
   // coarse levels apply the operator to all vectors at once (interleaved
   // [site][dof][vec] operand layout): on the tensor cores for 16-bit stores,
   // with the FP32 multi-RHS stream for FP32 stores
-  DevBuf ib, ob;
-  const bool mrhs = l > 0 && coarse_apply_multi_fast(L, nv);
-  if (mrhs) {
-    ib.alloc(bytes);
-    ob.alloc(bytes);
-  }
+  // (interleaved copies in the two halves of raw, free until the end)
+  const bool mrhs = l > 0 && !f64 && coarse_apply_multi_fast(L, nv);
   auto apply_all = [&](Vec out, Vec in) {
     if (l == 0) {
       wilson_apply(c, out, in, nv, st);
     } else if (mrhs) {
-      Vec vi = vbuf(ib, L.vprec, n), vo = vbuf(ob, L.vprec, n);
+      Vec vi = at(L.raw, 0, n), vo = at(L.raw, bytes, n);
       blas_transpose(c, vi, in, nv, true, st);
       coarse_apply(c, l, vo.p, vi.p, nv, st);
       blas_transpose(c, out, vo, nv, false, st);
@@ -442,8 +447,6 @@ void setup_sweeps(mg_ctx* c, int l, const void* init, cudaStream_t st) {
   blas_normalise_batched(c, X, nv, st);
   blas_copy(c, raw, Xall, st);
   L.have_raw = true;
-  L.have_V = false;
-  GB_CHECK(cudaStreamSynchronize(st));
 }
 
 void gcr_solve_multi(mg_ctx* c, void* xp, const void* bp, int nr, double tol, int maxiter,
