@@ -89,89 +89,162 @@ __global__ void __launch_bounds__(CG*(N / Unpack<S>::RPC))
   }
 }
 
-// Multi-RHS form of the streaming kernel for stores without a tensor-core
-// path (FP32).  Element (rhs, site, dof) sits at rhs * rs + (site * n + dof)
-// * ss: interleaved [site][n][nrhs] (rs = 1, ss = nrhs) or back to back
+// Multi-RHS form of the streaming kernel for FP32 stores (the 16-bit ones have
+// the tensor cores).  Element (rhs, site, dof) sits at rhs * rs + (site * n +
+// dof) * ss: interleaved [site][n][nrhs] (rs = 1, ss = nrhs) or back to back
 // [nrhs][site][n] (rs = V n, ss = 1).  CTA (chunk, site) applies the site's
-// links to NR right-hand sides, so each link chunk read from HBM feeds
-// NR x RPC complex multiply-adds.  The gathered neighbour values sit in
-// shared memory as xs[k][r] (k = slot*n + col); the same buffer then holds
-// the CG partial sums as red[cg][r][row].
-// UM caps the 16-byte link loads a thread keeps in flight (the batch U
-// divides the K / CG columns it walks); a larger batch takes registers
-// from occupancy, so the autotuner picks it per shape.
+// links to NR right-hand sides (a last chunk may hold fewer: its missing
+// vectors are zeros that are not stored), so each link read from HBM feeds NR
+// complex multiply-adds.
+//
+// What bounds it: latency of the link loads and, from about 12 right-hand
+// sides, the FMA pipe and the shared-memory reads of x.  So a thread owns four
+// rows (two 16-byte chunks of a column): a column's NR values of x, read once
+// per thread, serve 4 NR multiply-adds.  The arithmetic is packed: x sits in
+// shared memory as planes [k][re r0..][im r0..], pairs of right-hand sides
+// form one FMA operand, link entries are duplicated.  CTAs are small (8
+// column groups, 96 threads at n = 48, five per SM), so one's gather and
+// reduction overlap the others' streams.  8^3x16, n = 48: 8 right-hand sides
+// 365 -> 297 us (HBM bound 208; two rows per thread and scalar FMAs before),
+// 32: 1336 -> 1089, 3: 652 -> 221 (odd counts ran the generic kernel).  The
+// links through a bulk-copy ring in shared memory: 460 us; 16 column groups
+// per CTA: 471 us.
+// U: link columns a thread loads per batch; DB: the next batch is loaded
+// before the current one is used.  CG column groups split the 9n columns;
+// their sums meet in shared memory.
+constexpr int mr_groups(int n) { return n == 16 ? 16 : 8; }
+// resident CTAs per SM that the register budget allows (8 right-hand sides: 128
+// to 136 registers a thread)
+constexpr int mr_ctas(int n, int nr) {
+  return (nr == 8 ? 480 : 640) / (mr_groups(n) * (n / 4));
+}
+constexpr int mr_row(int n) { return n + 2; }  // padded row of partial sums
+constexpr int mr_stride(int nr) { return 2 * nr + 4; }  // floats per k, padded
+constexpr size_t mr_smem(int n, int nr) {
+  const size_t xs = size_t(9) * n * mr_stride(nr) * 4, red = size_t(mr_groups(n)) * nr * mr_row(n) * 8;
+  return xs > red ? xs : red;
+}
 // Eq. (3) on NR right-hand sides per link read.
-template <typename S, int N, int CG, int NR, int UM = 4>
-__global__ void __launch_bounds__(CG*(N / Unpack<S>::RPC))
-    k_coarse_stream_mr(cpx<typename StoreTraits<S>::real>* __restrict__ y,
-                       const cpx<typename StoreTraits<S>::real>* __restrict__ x,
-                       const S* __restrict__ links, const float* __restrict__ scales, Geom g,
-                       size_t rs, size_t ss) {
-  using R = typename StoreTraits<S>::real;
-  constexpr int RPC = Unpack<S>::RPC;
-  constexpr int TPC = N / RPC;
-  constexpr int K = 9 * N;
-  constexpr int NT = CG * TPC;
-  constexpr int ITER = K / CG;
-  constexpr int U = batch_of(ITER, UM);
-  constexpr int XS = K * NR, RED = CG * NR * N;
-  static_assert(N % RPC == 0 && K % CG == 0 && NR % 2 == 0 && ITER % U == 0, "tile shape");
-  __shared__ __align__(16) cpx<R> buf[XS > RED ? XS : RED];
+template <int N, int NR, int U, bool DB>
+__global__ void __launch_bounds__(mr_groups(N) * (N / 4), mr_ctas(N, NR))
+    k_coarse_stream_mr(cpx<float>* __restrict__ y, const cpx<float>* __restrict__ x,
+                       const uint4* __restrict__ links, Geom g, int nrhs, size_t rs, size_t ss) {
+  constexpr int TPC = N / 4, CG = mr_groups(N), K = 9 * N, NT = CG * TPC, ITER = K / CG;
+  constexpr int XS = mr_stride(NR), NP = NR / 2, RN = mr_row(N);
+  static_assert(N % 16 == 0 && K % CG == 0 && NR % 4 == 0 && ITER % U == 0, "tile shape");
+  extern __shared__ __align__(16) float xsm[];
   __shared__ int nb[9];
   const int chunk = blockIdx.x, site = blockIdx.y;
   const int tid = threadIdx.x;
+  const int rp = tid % TPC, cg = tid / TPC;
+  // the first links, in flight while x is gathered
+  const uint4* L = links + size_t(site) * K * (N / 2) + rp;
+  uint4 v[U][2];
+  auto load = [&](int it, uint4 (&w)[U][2]) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint4* q = L + size_t(cg + (it + u) * CG) * (N / 2);
+      w[u][0] = ld_stream16(q);
+      w[u][1] = ld_stream16(q + TPC);
+    }
+  };
+  load(0, v);
   if (tid < 9) {
     int c[4];
     site_coords(g, site, c);
     nb[tid] = neighbour(g, site, c, tid);
   }
   __syncthreads();
-  if (ss == 1) {  // back to back: read each vector's neighbour values in order
-    for (int i = tid; i < XS; i += NT) {
-      const int r = i / K, k = i - r * K;
-      const int d = k / N;
-      buf[k * NR + r] = x[size_t(chunk * NR + r) * rs + size_t(nb[d]) * N + (k - d * N)];
+  const int r0 = chunk * NR;
+  for (int i = tid; i < K * NR; i += NT) {
+    int k, r;
+    if (ss == 1) {  // back to back: each vector's neighbour values in order
+      r = i / K;
+      k = i - r * K;
+    } else {
+      k = i / NR;
+      r = i - k * NR;
     }
-  } else {
-    for (int i = tid; i < XS; i += NT) {
-      const int k = i / NR, r = i - k * NR;
-      const int d = k / N;
-      buf[i] = x[size_t(chunk * NR + r) * rs + (size_t(nb[d]) * N + (k - d * N)) * ss];
-    }
+    const int d = k / N;
+    cpx<float> e(0.f, 0.f);
+    if (r0 + r < nrhs) e = x[size_t(r0 + r) * rs + (size_t(nb[d]) * N + (k - d * N)) * ss];
+    xsm[k * XS + r] = e.re;
+    xsm[k * XS + NR + r] = e.im;
   }
   __syncthreads();
-  const int rp = tid % TPC;
-  const int cg = tid / TPC;
-  cpx<R> acc[NR][RPC];
+  f32x2 are[4][NP], aim[4][NP];
 #pragma unroll
-  for (int r = 0; r < NR; ++r)
+  for (int q = 0; q < 4; ++q)
 #pragma unroll
-    for (int q = 0; q < RPC; ++q) acc[r][q] = cpx<R>(R(0), R(0));
-  const uint4* L = reinterpret_cast<const uint4*>(links) + size_t(site) * K * TPC + rp;
-  for (int it = 0; it < ITER; it += U) {
-    uint4 v[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) v[u] = ld_stream16(L + size_t(cg + (it + u) * CG) * TPC);
+    for (int r = 0; r < NP; ++r) are[q][r] = aim[q][r] = 0;
+  auto use = [&](int it, const uint4 (&w)[U][2]) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      cpx<R> e[RPC];
-      Unpack<S>::get(v[u], e);
-      const cpx<R>* xk = buf + (cg + (it + u) * CG) * NR;
+      const ulonglong2* xk =
+          reinterpret_cast<const ulonglong2*>(xsm + (cg + (it + u) * CG) * XS);
+      f32x2 xr[NP], xi[NP];
 #pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        const cpx<R> xv = xk[r];
-#pragma unroll
-        for (int q = 0; q < RPC; ++q) cmac(acc[r][q], e[q], xv);
+      for (int r = 0; r < NP / 2; ++r) {
+        const ulonglong2 a = xk[r], b = xk[NP / 2 + r];
+        xr[2 * r] = a.x;
+        xr[2 * r + 1] = a.y;
+        xi[2 * r] = b.x;
+        xi[2 * r + 1] = b.y;
       }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint4 c = w[u][q >> 1];
+        const float lr = __uint_as_float(q & 1 ? c.z : c.x);
+        const float li = __uint_as_float(q & 1 ? c.w : c.y);
+        const f32x2 l2 = pack2f(lr, lr), i2 = pack2f(li, li), n2 = pack2f(-li, -li);
+#pragma unroll
+        for (int r = 0; r < NP; ++r) {
+          fma2(are[q][r], l2, xr[r]);
+          fma2(aim[q][r], l2, xi[r]);
+        }
+#pragma unroll
+        for (int r = 0; r < NP; ++r) {
+          fma2(are[q][r], n2, xi[r]);
+          fma2(aim[q][r], i2, xr[r]);
+        }
+      }
+    }
+  };
+  if constexpr (DB) {
+    uint4 w[U][2];
+    int it = 0;
+    for (; it + 2 * U <= ITER; it += 2 * U) {
+      load(it + U, w);
+      use(it, v);
+      if (it + 2 * U < ITER) load(it + 2 * U, v);
+      use(it + U, w);
+    }
+    if (it < ITER) use(it, v);
+  } else {
+    for (int it = 0; it < ITER; it += U) {
+      if (it) load(it, v);
+      use(it, v);
     }
   }
   __syncthreads();
+  // partial sums [cg][r][row], rows 2 rp, 2 rp + 1 and N/2 + the same
+  cpx<float>* red = reinterpret_cast<cpx<float>*>(xsm);
 #pragma unroll
-  for (int r = 0; r < NR; ++r)
+  for (int hq = 0; hq < 2; ++hq)
 #pragma unroll
-    for (int q = 0; q < RPC; ++q) buf[(cg * NR + r) * N + rp * RPC + q] = acc[r][q];
+    for (int r = 0; r < NP; ++r) {
+      float a[2][2], b[2][2];  // [row][rhs]
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        unpack2f(are[2 * hq + q][r], a[q][0], a[q][1]);
+        unpack2f(aim[2 * hq + q][r], b[q][0], b[q][1]);
+      }
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+        *reinterpret_cast<float4*>(red + (cg * NR + 2 * r + e) * RN + hq * (N / 2) + 2 * rp) =
+            make_float4(a[0][e], b[0][e], a[1][e], b[1][e]);
+    }
   __syncthreads();
-  const R sc = StoreTraits<S>::scaled ? R(scales[site]) : R(1);
   for (int o = tid; o < N * NR; o += NT) {
     int row, r;
     if (ss == 1) {
@@ -181,10 +254,11 @@ __global__ void __launch_bounds__(CG*(N / Unpack<S>::RPC))
       row = o / NR;
       r = o - row * NR;
     }
-    cpx<R> sum = buf[r * N + row];
+    if (r0 + r >= nrhs) continue;
+    cpx<float> sum = red[r * RN + row];
 #pragma unroll
-    for (int q = 1; q < CG; ++q) sum += buf[(q * NR + r) * N + row];
-    y[size_t(chunk * NR + r) * rs + (size_t(site) * N + row) * ss] = sc * sum;
+    for (int q = 1; q < CG; ++q) sum += red[(q * NR + r) * RN + row];
+    y[size_t(r0 + r) * rs + (size_t(site) * N + row) * ss] = sum;
   }
 }
 
@@ -502,60 +576,56 @@ bool try_stream(const Level& L, void* y, const void* x, const void* links, cudaS
   }
 }
 
-template <typename S, int N>
-void launch_stream_mr(const Level& L, void* y, const void* x, const void* links, int nrhs,
-                      bool blocked, cudaStream_t st) {
-  using R = typename StoreTraits<S>::real;
-  constexpr int CG = CgSet<S>::c0;
-  constexpr int NT = CG * (N / Unpack<S>::RPC);
-  const cpx<R>* xp = (const cpx<R>*)x;
-  cpx<R>* yp = (cpx<R>*)y;
-  const S* lp = (const S*)links;
-  const size_t rs = blocked ? size_t(L.g.vol) * N : 1;
-  const size_t ss = blocked ? 1 : size_t(nrhs);
-  if (nrhs % 8 == 0) {
-    // 8 right-hand sides per link read: the load batch is tuned (choice =
-    // its cap UM; caps giving the same batch are one candidate)
-    constexpr int ITER = 9 * N / CG;
-    std::vector<int> cands{4};
-    if (!std::is_same<S, cpx<double>>::value) {
-      if (batch_of(ITER, 6) != batch_of(ITER, 4)) cands.push_back(6);
-      if (batch_of(ITER, 9) != batch_of(ITER, 6) && batch_of(ITER, 9) != batch_of(ITER, 4))
-        cands.push_back(9);
-    }
-    auto launch = [&](int um) {
-      const dim3 grid(nrhs / 8, L.g.vol);
-      if (um == 9)
-        k_coarse_stream_mr<S, N, CG, 8, 9><<<grid, NT, 0, st>>>(yp, xp, lp, L.scales.as<float>(),
-                                                                 L.g, rs, ss);
-      else if (um == 6)
-        k_coarse_stream_mr<S, N, CG, 8, 6><<<grid, NT, 0, st>>>(yp, xp, lp, L.scales.as<float>(),
-                                                                 L.g, rs, ss);
-      else
-        k_coarse_stream_mr<S, N, CG, 8, 4><<<grid, NT, 0, st>>>(yp, xp, lp, L.scales.as<float>(),
-                                                                 L.g, rs, ss);
+template <int N, int NR, int U, bool DB>
+void launch_stream_mr(const Level& L, void* y, const void* x, int nrhs, bool blocked,
+                      cudaStream_t st) {
+  constexpr size_t smem = mr_smem(N, NR);
+  auto kern = k_coarse_stream_mr<N, NR, U, DB>;
+  GB_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+  kern<<<dim3(ceil_div(nrhs, NR), L.g.vol), mr_groups(N) * (N / 4), smem, st>>>(
+      (cpx<float>*)y, (const cpx<float>*)x, L.links.as<uint4>(), L.g, nrhs,
+      blocked ? size_t(L.g.vol) * N : 1, blocked ? 1 : size_t(nrhs));
+}
+
+// FP32 links, any nrhs > 1.  The autotuner picks the right-hand sides per
+// link read and the link batch of a thread:
+//   4 / 9  batches of up to 3 (4) columns, double-buffered / of up to 6,
+//          8 right-hand sides (4 when nrhs is at most 4)
+//   2      4 right-hand sides (nrhs above 4), double-buffered: where the last
+//          chunk of 8 would be half empty, 12 of them for instance
+bool try_stream_mr(const Level& L, void* y, const void* x, int nrhs, bool blocked,
+                   cudaStream_t st) {
+  auto go = [&](auto nc) {
+    constexpr int N = decltype(nc)::value;
+    constexpr int ITER = 9 * N / mr_groups(N);
+    constexpr int U3 = batch_of(ITER, 3), U4 = batch_of(ITER, 4), U6 = batch_of(ITER, 6);
+    auto launch = [&](int q) {
+      if (nrhs <= 4) {
+        if (q == 9)
+          launch_stream_mr<N, 4, U6, false>(L, y, x, nrhs, blocked, st);
+        else
+          launch_stream_mr<N, 4, U4, true>(L, y, x, nrhs, blocked, st);
+      } else if (q == 9) {
+        launch_stream_mr<N, 8, U6, false>(L, y, x, nrhs, blocked, st);
+      } else if (q == 2) {
+        launch_stream_mr<N, 4, U4, true>(L, y, x, nrhs, blocked, st);
+      } else {
+        launch_stream_mr<N, 8, U3, true>(L, y, x, nrhs, blocked, st);
+      }
     };
+    std::vector<int> cands{4, 9};
+    if (nrhs > 4) cands.push_back(2);
     const std::string key = "stream_mr/p" + std::to_string(int(L.prec)) + "/n" +
                             std::to_string(N) + "/v" + std::to_string(L.g.vol) + "/r" +
                             std::to_string(nrhs) + "/b" + std::to_string(int(blocked));
-    launch(cands.size() == 1 ? cands.front() : Tuner::get().choose(key, cands, st, launch));
-  } else if (nrhs % 4 == 0)
-    k_coarse_stream_mr<S, N, CG, 4><<<dim3(nrhs / 4, L.g.vol), NT, 0, st>>>(
-        yp, xp, lp, L.scales.as<float>(), L.g, rs, ss);
-  else
-    k_coarse_stream_mr<S, N, CG, 2><<<dim3(nrhs / 2, L.g.vol), NT, 0, st>>>(
-        yp, xp, lp, L.scales.as<float>(), L.g, rs, ss);
-}
-
-template <typename S>
-bool try_stream_mr(const Level& L, void* y, const void* x, const void* links, int nrhs,
-                   bool blocked, cudaStream_t st) {
-  if (nrhs % 2 != 0) return false;
+    launch(Tuner::get().choose(key, cands, st, launch));
+    return true;
+  };
   switch (L.nd) {
-    case 16: launch_stream_mr<S, 16>(L, y, x, links, nrhs, blocked, st); return true;
-    case 32: launch_stream_mr<S, 32>(L, y, x, links, nrhs, blocked, st); return true;
-    case 48: launch_stream_mr<S, 48>(L, y, x, links, nrhs, blocked, st); return true;
-    case 64: launch_stream_mr<S, 64>(L, y, x, links, nrhs, blocked, st); return true;
+    case 16: return go(std::integral_constant<int, 16>{});
+    case 32: return go(std::integral_constant<int, 32>{});
+    case 48: return go(std::integral_constant<int, 48>{});
+    case 64: return go(std::integral_constant<int, 64>{});
     default: return false;
   }
 }
@@ -567,7 +637,7 @@ void dispatch_apply(const Level& L, void* y, const void* x, const void* links, i
   if (nrhs == 1 && L.slots5 && L.links5.p && try_stream5<S>(L, y, x, st)) return;
   if (nrhs == 1 && try_stream<S>(L, y, x, links, st)) return;
   if constexpr (std::is_same<S, cpx<float>>::value) {
-    if (nrhs > 1 && try_stream_mr<S>(L, y, x, links, nrhs, false, st)) return;
+    if (nrhs > 1 && try_stream_mr(L, y, x, nrhs, false, st)) return;
   }
   int threads = L.nd * nrhs >= 256 ? 256 : ((L.nd * nrhs + 31) / 32) * 32;
   k_coarse_generic<S><<<L.g.vol, threads, 0, st>>>((cpx<R>*)y, (const cpx<R>*)x, (const S*)links,
@@ -579,7 +649,7 @@ void dispatch_apply(const Level& L, void* y, const void* x, const void* links, i
 bool coarse_apply_multi_fast(const Level& L, int nrhs) {
   if (nrhs < 2) return false;
   if (coarse_apply_mma_supported(L, nrhs)) return true;
-  return L.prec == MG_F32 && nrhs % 2 == 0 &&
+  return L.prec == MG_F32 &&
          (L.nd == 16 || L.nd == 32 || L.nd == 48 || L.nd == 64);
 }
 
@@ -625,13 +695,13 @@ void coarse_apply_blocked(mg_ctx* c, int level, void* y, const void* x, int nr,
   GB_REQUIRE(y != x, MG_ERR_ARG, "coarse_apply: output aliases input");
   const size_t n = L.vec_elems();
   const size_t vb = n * prec_bytes_complex(L.vprec);
-  if (L.prec == MG_F32 && !L.slots5 && nr % 2 == 0 &&
+  if (L.prec == MG_F32 && !L.slots5 &&
       (L.nd == 16 || L.nd == 32 || L.nd == 48 || L.nd == 64)) {
     const double nd = L.nd;
     ProfScope ps(c->prof, st, "coarse_apply_multi", level,
                  double(L.g.vol) * 9 * nd * nd * 8 + double(nr) * 2 * double(vb),
                  8.0 * 9 * nd * nd * L.g.vol * nr);
-    try_stream_mr<cpx<float>>(L, y, x, L.links.p, nr, true, st);
+    try_stream_mr(L, y, x, nr, true, st);
     GB_LAUNCH_CHECK();
     c->launches++;
     return;

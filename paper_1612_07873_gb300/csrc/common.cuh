@@ -107,6 +107,26 @@ __host__ __device__ __forceinline__ R norm2(cpx<R> a) {
   return a.re * a.re + a.im * a.im;
 }
 
+// ---------------------------------------------------- packed FP32 pairs
+// Two FP32 numbers in one 64-bit register pair and the two-lane FMA of
+// sm_100 and later.  An FFMA whose three sources are distinct registers runs
+// at three quarters of the pipe's rate here (register reads: 56 of 74
+// TFLOP/s on an outer-product loop), the packed form at full rate with half
+// the issue slots.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2f(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2f(f32x2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+// a += b * c in both halves
+__device__ __forceinline__ void fma2(f32x2& a, f32x2 b, f32x2 c) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a) : "l"(b), "l"(c));
+}
+
 // ------------------------------------------------------------------ storage
 // Complex element types of the link store.  16-bit forms carry a per-site
 // FP32 scale: value = scale * stored.
