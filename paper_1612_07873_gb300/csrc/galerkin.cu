@@ -600,7 +600,9 @@ void galerkin_build(mg_ctx* c, int level, cudaStream_t st) {
     }
   } else {
     GB_REQUIRE(C.vprec == MG_F32, MG_ERR_ARG, "FP64 level above an FP32 level is not supported");
-    if (level == 0) {
+    if (galerkin_mma(c, level, st)) {
+      // (contractions on the tensor cores)
+    } else if (level == 0) {
       WilsonOp<float> op{F.gauge32.as<cpx<float>>(), F.clover32.as<float>(), float(F.diag)};
       launch_galerkin<float, float>(op, F.Vp.as<cpx<float>>(), m, nf, nv, C.links.as<cpx<float>>(),
                                     err, st);

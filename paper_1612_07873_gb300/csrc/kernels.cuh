@@ -131,6 +131,10 @@ void wilson16_apply(mg_ctx* c, Vec out, Vec in, cudaStream_t st);
 
 // ---------------------------------------------------------------- galerkin.cu
 void galerkin_build(mg_ctx* c, int level, cudaStream_t st);
+// ---------------------------------------------------------------- galerkin_mma.cu
+// the FP32 Wilson-clover level's product on the tensor cores; false (nothing
+// launched) where that form does not apply
+bool galerkin_mma(mg_ctx* c, int level, cudaStream_t st);
 
 // ---------------------------------------------------------------- solver.cu
 void level_apply(mg_ctx* c, int level, Vec out, Vec in, cudaStream_t st);
