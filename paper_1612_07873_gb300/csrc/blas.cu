@@ -21,9 +21,11 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 // Reduction grid: one block per 4096 elements, at most one full wave of
 // the reduction kernel (per_sm resident blocks of 256 threads: 4 for the
 // kernels of <= 64 registers a thread); a second, partly filled wave would
-// leave SMs idle at the end.  The grid depends only on the length and the
-// device.
-int red_blocks(size_t n, int per_sm = 4) {
+// leave SMs idle at the end.  nr vectors share the wave (their blocks run side
+// by side; one wave each made blocks of a few loads around two CTA-wide
+// reductions: 8 BF16 vectors of 16^3x32 44 us, 15 us to read them).  The grid
+// depends only on the lengths and the device.
+int red_blocks(size_t n, int per_sm = 4, int nr = 1) {
   static const int sms = [] {
     int dev = 0, v = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -31,7 +33,8 @@ int red_blocks(size_t n, int per_sm = 4) {
       return kMaxRedBlocks / 4;
     return v;
   }();
-  const int cap = per_sm * sms < kMaxRedBlocks ? per_sm * sms : kMaxRedBlocks;
+  const int wave = per_sm * sms < kMaxRedBlocks ? per_sm * sms : kMaxRedBlocks;
+  const int cap = wave / nr > 1 ? wave / nr : 1;
   long long b = (long long)((n + 4095) / 4096);
   if (b < 1) b = 1;
   if (b > cap) b = cap;
@@ -69,6 +72,47 @@ __device__ __forceinline__ double2 block_sum(double2 v, double2* sh) {
     }
   }
   return v;
+}
+
+// Exact FP32 -> FP64 conversion by integer operations.  The hardware
+// conversion runs on the FP64 pipe (two lanes per clock and SM on GB300: 16
+// cycles a warp), which bounds the kernels that mix FP32 and FP64 vectors;
+// zeros, subnormals, infinities and NaN take it.
+__device__ __noinline__ double f2d_special(float f) { return double(f); }
+__device__ __forceinline__ double f2d(float f) {
+  const uint32_t u = __float_as_uint(f), e = u & 0x7f800000u;
+  if (e == 0u || e == 0x7f800000u) {
+    // (a call: predicated or selected, the conversion would run every time)
+    return (u << 1) == 0u ? __hiloint2double(int(u), 0) : f2d_special(f);
+  }
+  const uint32_t hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u);
+  return __hiloint2double(int(hi), int(u << 29));
+}
+// FP64 -> FP32, round to nearest even, by integer operations likewise (results
+// in the normal range of FP32, below 2^127; others take the conversion)
+__device__ __noinline__ float d2f_special(double d) { return float(d); }
+__device__ __forceinline__ float d2f(double d) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+  const uint32_t e = uint32_t(u >> 52) & 0x7ffu;
+  if (e - 897u >= 253u) return (u << 1) == 0ull ? __uint_as_float(uint32_t(u >> 32)) : d2f_special(d);
+  const unsigned long long t = (u & 0x7fffffffffffffffull) - (896ull << 52);
+  const uint32_t r = uint32_t((t + 0x0fffffffull + ((t >> 29) & 1ull)) >> 29);
+  return __uint_as_float(r | (uint32_t(u >> 32) & 0x80000000u));
+}
+__device__ __forceinline__ cpx<float> narrow(cpx<double> a) {
+  return cpx<float>(d2f(a.re), d2f(a.im));
+}
+__device__ __forceinline__ cpx<float> narrow(cpx<float> a) { return a; }
+__device__ __forceinline__ cpx<double> widen(cpx<float> a) {
+  return cpx<double>(f2d(a.re), f2d(a.im));
+}
+__device__ __forceinline__ cpx<double> widen(cpx<double> a) { return a; }
+template <typename T, typename R>
+__device__ __forceinline__ cpx<T> to_acc(cpx<R> a) {
+  if constexpr (std::is_same<T, double>::value)
+    return widen(a);
+  else
+    return cpx<T>(a);
 }
 
 // Per-thread partial sums run in the arithmetic type T: FP32 when both
@@ -113,10 +157,10 @@ __global__ void k_dot_partial(const cpx<Ra>* __restrict__ a, const cpx<Rb>* __re
   for (int k = 0; k < kAcc; ++k) acc[k] = cpx<T>(T(0), T(0));
   grid_loop_acc(n, [&](size_t i, int k) {
     if constexpr (NORM) {
-      const cpx<T> x(a[i]);
+      const cpx<T> x = to_acc<T>(a[i]);
       acc[k].re = fma(x.re, x.re, fma(x.im, x.im, acc[k].re));
     } else {
-      cmac_conj(acc[k], cpx<T>(a[i]), cpx<T>(b[i]));
+      cmac_conj(acc[k], to_acc<T>(a[i]), to_acc<T>(b[i]));
     }
   });
   const cpx<T> t = (acc[0] + acc[1]) + (acc[2] + acc[3]);
@@ -399,8 +443,9 @@ __global__ void k_dot2_partial_b(const cpx<Ra>* __restrict__ p, const cpx<Rb>* _
 }
 
 // out[b] = sum of the nparts partials of row b (one block per row)
+// (inv: the imaginary part, zero for a norm, receives 1 / sqrt of the sum)
 __global__ void k_reduce_final_b(const double2* __restrict__ part, int nparts,
-                                 double2* __restrict__ out) {
+                                 double2* __restrict__ out, bool inv = false) {
   __shared__ double2 sh[32];
   const double2* src = part + size_t(blockIdx.x) * nparts;
   double2 acc = make_double2(0.0, 0.0);
@@ -409,21 +454,41 @@ __global__ void k_reduce_final_b(const double2* __restrict__ part, int nparts,
     acc.y += src[i].y;
   }
   acc = block_sum(acc, sh);
-  if (threadIdx.x == 0) out[blockIdx.x] = acc;
+  if (threadIdx.x == 0) {
+    if (inv) acc.y = acc.x > 0.0 ? 1.0 / sqrt(acc.x) : 0.0;
+    out[blockIdx.x] = acc;
+  }
 }
 
-// rows (2 v, 2 v + 1) of the dot2 partials into A[v] and B[v]
+// rows (2 v, 2 v + 1) of the dot2 partials into A[v] and B[v], and the MR
+// coefficient omega A[v] / B[v].re (0 for a zero denominator) into C[v]: one
+// FP64 division per vector here instead of one per warp of the update, where
+// the FP64 pipe's 16 cycles a warp instruction made it the longest part
 __global__ void k_reduce_final_pair(const double2* __restrict__ part, int nparts,
-                                    double2* __restrict__ A, double2* __restrict__ B) {
+                                    double2* __restrict__ A, double2* __restrict__ B,
+                                    double2* __restrict__ C, double omega) {
   __shared__ double2 sh[32];
-  const double2* src = part + size_t(blockIdx.x) * nparts;
-  double2 acc = make_double2(0.0, 0.0);
+  const int v = blockIdx.x;
+  const double2* src = part + size_t(2 * v) * nparts;
+  double2 acc = make_double2(0.0, 0.0), den = acc;
   for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
     acc.x += src[i].x;
     acc.y += src[i].y;
+    den.x += src[nparts + i].x;
   }
   acc = block_sum(acc, sh);
-  if (threadIdx.x == 0) (blockIdx.x & 1 ? B : A)[blockIdx.x >> 1] = acc;
+  __syncthreads();
+  den = block_sum(den, sh);
+  if (threadIdx.x == 0) {
+    A[v] = acc;
+    B[v] = make_double2(den.x, 0.0);
+    double2 a = make_double2(0.0, 0.0);
+    if (den.x > 0.0) {
+      const double f = omega / den.x;
+      a = make_double2(f * acc.x, f * acc.y);
+    }
+    C[v] = a;
+  }
 }
 
 // Per-RHS scalar of an update, formed once per warp (lane 0, broadcast):
@@ -438,8 +503,12 @@ __device__ __forceinline__ double2 warp_bcast(double2 v) {
 template <typename Ry, typename Rx>
 __global__ void k_copy(cpx<Ry>* __restrict__ y, const cpx<Rx>* __restrict__ x, size_t n) {
   for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n;
-       i += size_t(gridDim.x) * blockDim.x)
-    y[i] = cpx<Ry>(x[i]);
+       i += size_t(gridDim.x) * blockDim.x) {
+    if constexpr (std::is_same<Ry, float>::value)
+      y[i] = narrow(x[i]);
+    else
+      y[i] = to_acc<Ry>(x[i]);
+  }
 }
 
 // y += a x with a host constant
@@ -482,46 +551,43 @@ __global__ void k_sub(cpx<Ro>* __restrict__ o, const cpx<Rb>* __restrict__ b,
     o[i] = cpx<Ro>(cpx<T>(b[i]) - cpx<T>(ax[i]));
 }
 
-// x_v += a_v r_v ; r_v -= a_v p_v  with a_v = omega PR[v] / PP[v].re
-template <typename R>
-__global__ void k_mr_update(cpx<R>* __restrict__ x, cpx<R>* __restrict__ r,
+// x_v += a_v r_v ; r_v -= a_v p_v  with a_v = C[v] (k_reduce_final_pair).  The
+// steps at the ends of a smoothing leave out what is not needed: FIRST: x
+// starts at zero (written, not read); LAST: the residual is not used again
+// (p is not read, r not written).  The residual is read from rin, which may
+// be r.
+template <typename R, bool FIRST, bool LAST>
+__global__ void k_mr_update(cpx<R>* __restrict__ x, cpx<R>* r, const cpx<R>* rin,
                             const cpx<R>* __restrict__ p, size_t n,
-                            const double2* __restrict__ PR, const double2* __restrict__ PP,
-                            double omega) {
+                            const double2* __restrict__ C) {
   const int v = blockIdx.y;
-  double2 a = make_double2(0.0, 0.0);
-  if ((threadIdx.x & 31) == 0) {
-    const double den = PP[v].x;
-    if (den > 0.0) {
-      const double f = omega / den;
-      a = make_double2(f * PR[v].x, f * PR[v].y);
-    }
-  }
-  a = warp_bcast(a);
+  const double2 a = C[v];
   const cpx<R> ar(R(a.x), R(a.y));
   x += size_t(v) * n;
   r += size_t(v) * n;
+  rin += size_t(v) * n;
   p += size_t(v) * n;
   for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n;
        i += size_t(gridDim.x) * blockDim.x) {
-    cpx<R> ri = r[i], xi = x[i];
+    cpx<R> ri = rin[i], xi(R(0), R(0));
+    if (!FIRST) xi = x[i];
     cmac(xi, ar, ri);
-    cmac(ri, -ar, p[i]);
     x[i] = xi;
-    r[i] = ri;
+    if (!LAST) {
+      cmac(ri, -ar, p[i]);
+      r[i] = ri;
+    }
   }
 }
 
-// a_v, b_v *= 1 / sqrt(S[v].re)   (b may be null)
+// a_v, b_v *= S[v].im, the inverse norm left by the reduction (b may be null)
 template <typename Ra, typename Rb>
 __global__ void k_scale_invnorm(cpx<Ra>* __restrict__ a, cpx<Rb>* __restrict__ b, size_t n,
                                 const double2* __restrict__ S) {
   const int v = blockIdx.y;
-  double2 sv = make_double2(0.0, 0.0);
-  if ((threadIdx.x & 31) == 0) sv.x = S[v].x > 0.0 ? 1.0 / sqrt(S[v].x) : 0.0;
-  sv = warp_bcast(sv);
-  const Ra sa = Ra(sv.x);
-  const Rb sb = Rb(sv.x);
+  const double sv = S[v].y;
+  const Ra sa = Ra(sv);
+  const Rb sb = Rb(sv);
   a += size_t(v) * n;
   if (b) b += size_t(v) * n;
   for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n;
@@ -531,33 +597,47 @@ __global__ void k_scale_invnorm(cpx<Ra>* __restrict__ a, cpx<Rb>* __restrict__ b
   }
 }
 
-// x_v += S[v] z_v ; r_v -= S[v] w_v.  With FP32 directions z, w the products
-// are formed in FP32 (they carry the precision of z and w, no more) and only
-// the sums run in the precision of x and r; x and r receive the same scalar.
+// x_v += S[v] z_v ; r_v -= S[v] w_v, the partials of |r_v|^2 of the new
+// residual (sums in FP32 for FP32 residuals, FP64 otherwise, as k_dot_partial)
+// and, when rk is given, its FP32 copy: the next step's residual norm and
+// preconditioner input without reading r again.  With FP32 directions z, w the
+// products are formed in FP32 (they carry the precision of z and w, no more)
+// and only the sums run in the precision of x and r; x and r receive the same
+// scalar.
 template <typename Rx, typename Rz>
-__global__ void k_gcr_update(cpx<Rx>* __restrict__ x, cpx<Rx>* __restrict__ r,
-                             const cpx<Rz>* __restrict__ z, const cpx<Rz>* __restrict__ w,
-                             size_t n, const double2* __restrict__ S) {
+__global__ void __launch_bounds__(256)
+    k_gcr_update(cpx<Rx>* __restrict__ x, cpx<Rx>* __restrict__ r, const cpx<Rz>* __restrict__ z,
+                 const cpx<Rz>* __restrict__ w, size_t n, const double2* __restrict__ S,
+                 cpx<float>* __restrict__ rk, double2* __restrict__ part) {
   using T = typename std::conditional<std::is_same<Rz, float>::value, float, double>::type;
+  __shared__ double2 sh[32];
   const int v = blockIdx.y;
   const cpx<T> a(T(S[v].x), T(S[v].y));
   x += size_t(v) * n;
   r += size_t(v) * n;
   z += size_t(v) * n;
   w += size_t(v) * n;
-  for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n;
-       i += size_t(gridDim.x) * blockDim.x) {
+  if (rk) rk += size_t(v) * n;
+  Rx acc[kAcc];
+#pragma unroll
+  for (int k = 0; k < kAcc; ++k) acc[k] = Rx(0);
+  grid_loop_acc(n, [&](size_t i, int k) {
     cpx<Rx> xi = x[i], ri = r[i];
     if constexpr (std::is_same<T, float>::value) {
-      xi += cpx<Rx>(a * cpx<T>(z[i]));
-      ri -= cpx<Rx>(a * cpx<T>(w[i]));
+      xi += to_acc<Rx>(a * cpx<T>(z[i]));
+      ri -= to_acc<Rx>(a * cpx<T>(w[i]));
     } else {
       cmac(xi, cpx<Rx>(a), cpx<Rx>(z[i]));
       cmac(ri, -cpx<Rx>(a), cpx<Rx>(w[i]));
     }
     x[i] = xi;
     r[i] = ri;
-  }
+    if (rk) rk[i] = narrow(ri);
+    acc[k] = fma(ri.re, ri.re, fma(ri.im, ri.im, acc[k]));
+  });
+  const double t = double((acc[0] + acc[1]) + (acc[2] + acc[3]));
+  const double2 d = block_sum(make_double2(t, 0.0), sh);
+  if (threadIdx.x == 0) part[size_t(blockIdx.y) * gridDim.x + blockIdx.x] = d;
 }
 
 // ---- BF16 vectors (the 16-bit fine-level smoother): storage BF16, all
@@ -585,7 +665,8 @@ __global__ void k_copy_to16(bf16c* __restrict__ y, const cpx<float>* __restrict_
     }
   }
 }
-template <int W>
+// y = x, or y += x (ADD)
+template <int W, bool ADD>
 __global__ void k_copy_from16(cpx<float>* __restrict__ y, const bf16c* __restrict__ x, size_t n) {
   for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n / W;
        i += size_t(gridDim.x) * blockDim.x) {
@@ -594,10 +675,17 @@ __global__ void k_copy_from16(cpx<float>* __restrict__ y, const bf16c* __restric
       const bf16c* wc = reinterpret_cast<const bf16c*>(&w);
       const cpx<float> c0 = h2f(wc[0]), c1 = h2f(wc[1]), c2 = h2f(wc[2]), c3 = h2f(wc[3]);
       float4* y4 = reinterpret_cast<float4*>(y) + 2 * i;
-      y4[0] = make_float4(c0.re, c0.im, c1.re, c1.im);
-      y4[1] = make_float4(c2.re, c2.im, c3.re, c3.im);
+      float4 a = make_float4(c0.re, c0.im, c1.re, c1.im);
+      float4 b = make_float4(c2.re, c2.im, c3.re, c3.im);
+      if constexpr (ADD) {
+        const float4 p = y4[0], q = y4[1];
+        a = make_float4(p.x + a.x, p.y + a.y, p.z + a.z, p.w + a.w);
+        b = make_float4(q.x + b.x, q.y + b.y, q.z + b.z, q.w + b.w);
+      }
+      y4[0] = a;
+      y4[1] = b;
     } else {
-      y[i] = h2f(x[i]);
+      y[i] = ADD ? y[i] + h2f(x[i]) : h2f(x[i]);
     }
   }
 }
@@ -646,31 +734,25 @@ __global__ void k_dot2_partial_h(const bf16c* __restrict__ p, const bf16c* __res
   }
 }
 
-template <int W>
+template <int W, bool FIRST, bool LAST>
 __global__ void k_mr_update_h(bf16c* __restrict__ x, bf16c* __restrict__ r,
                               const bf16c* __restrict__ p, size_t n,
-                              const double2* __restrict__ PR, const double2* __restrict__ PP,
-                              double omega) {
+                              const double2* __restrict__ C) {
   const int v = blockIdx.y;
-  double2 a = make_double2(0.0, 0.0);
-  if ((threadIdx.x & 31) == 0) {
-    const double den = PP[v].x;
-    if (den > 0.0) {
-      const double f = omega / den;
-      a = make_double2(f * PR[v].x, f * PR[v].y);
-    }
-  }
-  a = warp_bcast(a);
+  const double2 a = C[v];
   const cpx<float> ar(float(a.x), float(a.y));
   x += size_t(v) * n;
   r += size_t(v) * n;
   p += size_t(v) * n;
   auto upd = [&](bf16c& xs, bf16c& rs, bf16c ps) {
-    cpx<float> ri = h2f(rs), xi = h2f(xs);
+    cpx<float> ri = h2f(rs), xi(0.f, 0.f);
+    if (!FIRST) xi = h2f(xs);
     cmac(xi, ar, ri);
-    cmac(ri, -ar, h2f(ps));
     xs = StoreTraits<bf16c>::pack(xi);
-    rs = StoreTraits<bf16c>::pack(ri);
+    if (!LAST) {
+      cmac(ri, -ar, h2f(ps));
+      rs = StoreTraits<bf16c>::pack(ri);
+    }
   };
   if constexpr (W == 4) {
     uint4* x4 = reinterpret_cast<uint4*>(x);
@@ -678,14 +760,15 @@ __global__ void k_mr_update_h(bf16c* __restrict__ x, bf16c* __restrict__ r,
     const uint4* p4 = reinterpret_cast<const uint4*>(p);
     for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n / 4;
          i += size_t(gridDim.x) * blockDim.x) {
-      uint4 wx = x4[i], wr = r4[i];
-      const uint4 wp = p4[i];
+      uint4 wx = make_uint4(0, 0, 0, 0), wp = wx, wr = r4[i];
+      if (!FIRST) wx = x4[i];
+      if (!LAST) wp = p4[i];
 #pragma unroll
       for (int j = 0; j < 4; ++j)
         upd(reinterpret_cast<bf16c*>(&wx)[j], reinterpret_cast<bf16c*>(&wr)[j],
             reinterpret_cast<const bf16c*>(&wp)[j]);
       x4[i] = wx;
-      r4[i] = wr;
+      if (!LAST) r4[i] = wr;
     }
   } else {
     for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n;
@@ -837,10 +920,10 @@ void blas_copy(mg_ctx* c, Vec d, Vec s, cudaStream_t st) {
                                                           n);
     } else {
       if (w4)
-        k_copy_from16<4><<<ew_blocks(n / 4), kThreads, 0, st>>>((cpx<float>*)d.p,
+        k_copy_from16<4, false><<<ew_blocks(n / 4), kThreads, 0, st>>>((cpx<float>*)d.p,
                                                                 (const bf16c*)s.p, n);
       else
-        k_copy_from16<1><<<ew_blocks(n), kThreads, 0, st>>>((cpx<float>*)d.p,
+        k_copy_from16<1, false><<<ew_blocks(n), kThreads, 0, st>>>((cpx<float>*)d.p,
                                                             (const bf16c*)s.p, n);
     }
     GB_LAUNCH_CHECK();
@@ -855,6 +938,20 @@ void blas_copy(mg_ctx* c, Vec d, Vec s, cudaStream_t st) {
   GB_DISPATCH2(d.prec, Ry, s.prec, Rx,
                (k_copy<Ry, Rx><<<ew_blocks(d.total()), kThreads, 0, st>>>(
                    (cpx<Ry>*)d.p, (const cpx<Rx>*)s.p, d.total())));
+  GB_LAUNCH_CHECK();
+  c->launches++;
+}
+
+void blas_add16(mg_ctx* c, Vec y, Vec x, cudaStream_t st) {
+  GB_REQUIRE(y.total() == x.total() && y.prec == MG_F32 && x.prec == MG_BF16, MG_ERR_ARG,
+             "add16: FP32 += BF16 of one length");
+  const size_t n = y.total();
+  if (n % 4 == 0 && aligned16(y.p) && aligned16(x.p))
+    k_copy_from16<4, true><<<ew_blocks(n / 4), kThreads, 0, st>>>((cpx<float>*)y.p,
+                                                                  (const bf16c*)x.p, n);
+  else
+    k_copy_from16<1, true><<<ew_blocks(n), kThreads, 0, st>>>((cpx<float>*)y.p,
+                                                              (const bf16c*)x.p, n);
   GB_LAUNCH_CHECK();
   c->launches++;
 }
@@ -890,10 +987,10 @@ void blas_sub(mg_ctx* c, Vec o, Vec b, Vec ax, cudaStream_t st) {
   c->launches++;
 }
 
-void blas_dot(mg_ctx* c, Vec a, Vec b, int slot, cudaStream_t st, bool fp64_partials) {
+void blas_dot(mg_ctx* c, Vec a, Vec b, int slot, cudaStream_t st, bool fp64_partials, bool inv) {
   check_nr(a);
   GB_REQUIRE(a.n == b.n && a.nr == b.nr, MG_ERR_ARG, "dot: shape mismatch");
-  const int nb = red_blocks(a.n);
+  const int nb = red_blocks(a.n, 4, a.nr);
   double2* part = partials(c, size_t(nb) * a.nr);
   const dim3 grid(nb, a.nr);
   const bool norm = a.p == b.p && a.prec == b.prec;
@@ -928,19 +1025,20 @@ void blas_dot(mg_ctx* c, Vec a, Vec b, int slot, cudaStream_t st, bool fp64_part
                      (const cpx<Ra>*)a.p, (const cpx<Rb>*)b.p, a.n, part)));
   }
   GB_LAUNCH_CHECK();
-  k_reduce_final_b<<<a.nr, 256, 0, st>>>(part, nb, srow(c, slot));
+  k_reduce_final_b<<<a.nr, 256, 0, st>>>(part, nb, srow(c, slot), inv && norm);
   GB_LAUNCH_CHECK();
   c->launches += 2;
 }
 
-void blas_norm2(mg_ctx* c, Vec a, int slot, cudaStream_t st, bool fp64_partials) {
-  blas_dot(c, a, a, slot, st, fp64_partials);
+void blas_norm2(mg_ctx* c, Vec a, int slot, cudaStream_t st, bool fp64_partials, bool inv) {
+  blas_dot(c, a, a, slot, st, fp64_partials, inv);
 }
 
-void blas_dot2(mg_ctx* c, Vec p, Vec r, int s_pr, int s_pp, cudaStream_t st) {
+void blas_dot2(mg_ctx* c, Vec p, Vec r, int s_pr, int s_pp, int s_a, double omega,
+               cudaStream_t st) {
   check_nr(p);
   GB_REQUIRE(p.n == r.n && p.nr == r.nr, MG_ERR_ARG, "dot2: shape mismatch");
-  const int nb = red_blocks(p.n);
+  const int nb = red_blocks(p.n, 4, p.nr);
   double2* part = partials(c, size_t(nb) * 2 * p.nr);
   if (p.prec == MG_BF16 || r.prec == MG_BF16) {
     GB_REQUIRE(p.prec == MG_BF16 && r.prec == MG_BF16, MG_ERR_ARG, "dot2: precision mix");
@@ -956,30 +1054,51 @@ void blas_dot2(mg_ctx* c, Vec p, Vec r, int s_pr, int s_pp, cudaStream_t st) {
                      (const cpx<Ra>*)p.p, (const cpx<Rb>*)r.p, p.n, part)));
   }
   GB_LAUNCH_CHECK();
-  k_reduce_final_pair<<<2 * p.nr, 256, 0, st>>>(part, nb, srow(c, s_pr), srow(c, s_pp));
+  k_reduce_final_pair<<<p.nr, 256, 0, st>>>(part, nb, srow(c, s_pr), srow(c, s_pp),
+                                            srow(c, s_a), omega);
   GB_LAUNCH_CHECK();
   c->launches += 2;
 }
 
-void blas_mr_update(mg_ctx* c, Vec x, Vec r, Vec p, int s_pr, int s_pp, double omega,
-                    cudaStream_t st) {
+void blas_mr_update(mg_ctx* c, Vec x, Vec r, Vec p, int s_a, cudaStream_t st, bool first,
+                    bool last, const void* rin) {
   check_nr(x);
   GB_REQUIRE(x.prec == r.prec && r.prec == p.prec, MG_ERR_ARG, "mr_update: precision mix");
-  if (x.prec == MG_BF16) {
-    if (x.n % 4 == 0 && aligned16(x.p) && aligned16(r.p) && aligned16(p.p))
-      k_mr_update_h<4><<<ew_grid_b(x.n / 4, x.nr), kThreads, 0, st>>>(
-          (bf16c*)x.p, (bf16c*)r.p, (const bf16c*)p.p, x.n, srow(c, s_pr), srow(c, s_pp), omega);
+  // one of the four kernels by (first, last)
+  auto pick = [&](auto&& go) {
+    if (first && last)
+      go(std::true_type{}, std::true_type{});
+    else if (first)
+      go(std::true_type{}, std::false_type{});
+    else if (last)
+      go(std::false_type{}, std::true_type{});
     else
-      k_mr_update_h<1><<<ew_grid_b(x.n, x.nr), kThreads, 0, st>>>(
-          (bf16c*)x.p, (bf16c*)r.p, (const bf16c*)p.p, x.n, srow(c, s_pr), srow(c, s_pp), omega);
+      go(std::false_type{}, std::false_type{});
+  };
+  if (x.prec == MG_BF16) {
+    GB_REQUIRE(!rin || rin == r.p, MG_ERR_ARG, "mr_update: BF16 residual in place only");
+    const bool w4 = x.n % 4 == 0 && aligned16(x.p) && aligned16(r.p) && aligned16(p.p);
+    pick([&](auto f, auto l) {
+      constexpr bool F = decltype(f)::value, L = decltype(l)::value;
+      if (w4)
+        k_mr_update_h<4, F, L><<<ew_grid_b(x.n / 4, x.nr), kThreads, 0, st>>>(
+            (bf16c*)x.p, (bf16c*)r.p, (const bf16c*)p.p, x.n, srow(c, s_a));
+      else
+        k_mr_update_h<1, F, L><<<ew_grid_b(x.n, x.nr), kThreads, 0, st>>>(
+            (bf16c*)x.p, (bf16c*)r.p, (const bf16c*)p.p, x.n, srow(c, s_a));
+    });
     GB_LAUNCH_CHECK();
     c->launches++;
     return;
   }
-  GB_DISPATCH1(x.prec, R,
-               (k_mr_update<R><<<ew_grid_b(x.n, x.nr), kThreads, 0, st>>>(
-                   (cpx<R>*)x.p, (cpx<R>*)r.p, (const cpx<R>*)p.p, x.n, srow(c, s_pr),
-                   srow(c, s_pp), omega)));
+  const void* ri = rin ? rin : r.p;
+  pick([&](auto f, auto l) {
+    constexpr bool F = decltype(f)::value, L = decltype(l)::value;
+    GB_DISPATCH1(x.prec, R,
+                 (k_mr_update<R, F, L><<<ew_grid_b(x.n, x.nr), kThreads, 0, st>>>(
+                     (cpx<R>*)x.p, (cpx<R>*)r.p, (const cpx<R>*)ri, (const cpx<R>*)p.p, x.n,
+                     srow(c, s_a))));
+  });
   GB_LAUNCH_CHECK();
   c->launches++;
 }
@@ -993,15 +1112,20 @@ void blas_scale_invnorm(mg_ctx* c, Vec a, Vec b, int slot, cudaStream_t st) {
   c->launches++;
 }
 
-void blas_gcr_update(mg_ctx* c, Vec x, Vec r, Vec z, Vec w, int slot, cudaStream_t st) {
+void blas_gcr_update(mg_ctx* c, Vec x, Vec r, Vec z, Vec w, int slot, int s_norm, void* rk,
+                     cudaStream_t st) {
   check_nr(x);
   GB_REQUIRE(x.prec == r.prec && z.prec == w.prec, MG_ERR_ARG, "gcr_update: precision mix");
+  const int nb = red_blocks(x.n, 4, x.nr);
+  double2* part = partials(c, size_t(nb) * x.nr);
   GB_DISPATCH2(x.prec, Rx, z.prec, Rz,
-               (k_gcr_update<Rx, Rz><<<ew_grid_b(x.n, x.nr), kThreads, 0, st>>>(
+               (k_gcr_update<Rx, Rz><<<dim3(nb, x.nr), kThreads, 0, st>>>(
                    (cpx<Rx>*)x.p, (cpx<Rx>*)r.p, (const cpx<Rz>*)z.p, (const cpx<Rz>*)w.p, x.n,
-                   srow(c, slot))));
+                   srow(c, slot), (cpx<float>*)rk, part)));
   GB_LAUNCH_CHECK();
-  c->launches++;
+  k_reduce_final_b<<<x.nr, 256, 0, st>>>(part, nb, srow(c, s_norm));
+  GB_LAUNCH_CHECK();
+  c->launches += 2;
 }
 
 void blas_read_slot(mg_ctx* c, int slot, int nr, double* out_re, cudaStream_t st) {
@@ -1026,7 +1150,7 @@ void blas_dot_multi(mg_ctx* c, const Vec* X, int m, Vec y, int slot, cudaStream_
   for (int j = 0; j < m; ++j) w2 = w2 && aligned16(X[j].p);
   // resident blocks per SM from the registers a thread: k_dot_multi <= 128;
   // k_dot_multi_ff<M> <= 64 up to M = 6, <= 80 up to M = 8, <= 128 beyond
-  const int nb = red_blocks(y.n, !w2 ? 2 : m <= 6 ? 4 : m <= 8 ? 3 : 2);
+  const int nb = red_blocks(y.n, !w2 ? 2 : m <= 6 ? 4 : m <= 8 ? 3 : 2, y.nr);
   double2* part = partials(c, size_t(nb) * m * y.nr);
   const dim3 grid(nb, y.nr);
   const auto* yp = (const cpx<float>*)y.p;
@@ -1102,7 +1226,7 @@ void blas_read_slot_c(mg_ctx* c, int slot, double out[2], cudaStream_t st) {
 
 void blas_dot2_batched(mg_ctx* c, Vec p, Vec r, int nvec, cudaStream_t st) {
   GB_REQUIRE(nvec >= 1 && nvec <= 64, MG_ERR_ARG, "dot2_batched: nvec out of range");
-  const int nb = red_blocks(p.n);
+  const int nb = red_blocks(p.n, 4, nvec);
   const size_t need = size_t(nvec) * 2 * nb * sizeof(double2);
   if (c->batch_partials.bytes < need) c->batch_partials.alloc(need);
   double2* part = c->batch_partials.as<double2>();

@@ -31,17 +31,28 @@ void blas_sub(mg_ctx* c, Vec out, Vec b, Vec ax, cudaStream_t st);
 // S[slot][v] = <a_v, b_v> = sum conj(a_v) b_v
 // fp64_partials: per-thread partial sums in FP64 even for FP32 data (the
 // outer GCR's orthogonalisation); otherwise FP32 data sums per thread in FP32
-void blas_dot(mg_ctx* c, Vec a, Vec b, int slot, cudaStream_t st, bool fp64_partials = false);
-void blas_norm2(mg_ctx* c, Vec a, int slot, cudaStream_t st, bool fp64_partials = false);
-// S[s_pr][v] = <p_v, r_v>, S[s_pp][v] = <p_v, p_v> in one pass
-void blas_dot2(mg_ctx* c, Vec p, Vec r, int s_pr, int s_pp, cudaStream_t st);
-// MR step per vector: a = omega S[s_pr]/S[s_pp].re ; x += a r ; r -= a p
-void blas_mr_update(mg_ctx* c, Vec x, Vec r, Vec p, int s_pr, int s_pp, double omega,
-                    cudaStream_t st);
-// a_v *= 1/sqrt(S[slot][v].re), b_v likewise
+// inv (norms): the slot's imaginary part is 1 / norm, for blas_scale_invnorm
+void blas_dot(mg_ctx* c, Vec a, Vec b, int slot, cudaStream_t st, bool fp64_partials = false,
+              bool inv = false);
+void blas_norm2(mg_ctx* c, Vec a, int slot, cudaStream_t st, bool fp64_partials = false,
+                bool inv = false);
+// S[s_pr][v] = <p_v, r_v>, S[s_pp][v] = <p_v, p_v> in one pass, and the MR
+// coefficient S[s_a][v] = omega S[s_pr][v] / S[s_pp][v].re (0 if that is 0)
+void blas_dot2(mg_ctx* c, Vec p, Vec r, int s_pr, int s_pp, int s_a, double omega,
+               cudaStream_t st);
+// MR step per vector: a = S[s_a] ; x += a r ; r -= a p.
+// first: x is taken as zero (not read); last: r is not updated.  rin: where the
+// residual is read from (null: r itself; FP32 / FP64 only)
+void blas_mr_update(mg_ctx* c, Vec x, Vec r, Vec p, int s_a, cudaStream_t st, bool first = false,
+                    bool last = false, const void* rin = nullptr);
+// y += x, x in BF16
+void blas_add16(mg_ctx* c, Vec y, Vec x, cudaStream_t st);
+// a_v *= S[slot][v].im (blas_norm2 with inv), b_v likewise
 void blas_scale_invnorm(mg_ctx* c, Vec a, Vec b, int slot, cudaStream_t st);
-// x_v += S[slot][v] z_v ; r_v -= S[slot][v] w_v
-void blas_gcr_update(mg_ctx* c, Vec x, Vec r, Vec z, Vec w, int slot, cudaStream_t st);
+// x_v += S[slot][v] z_v ; r_v -= S[slot][v] w_v ; S[s_norm][v] = |r_v|^2 ; an
+// FP32 copy of r into rk (or null)
+void blas_gcr_update(mg_ctx* c, Vec x, Vec r, Vec z, Vec w, int slot, int s_norm, void* rk,
+                     cudaStream_t st);
 // real parts of S[slot][0..nr) to the host (synchronises st)
 // Block (classical) Gram-Schmidt against m <= kCgs vectors X[j] in one
 // pass each: S[slot + j] = <X[j], y> (FP64-accurate when fp64_partials;
@@ -98,7 +109,8 @@ void block_orthonormalise(mg_ctx* c, int level, cudaStream_t st);
 // block-orthonormal null vectors of `level` into dst [Nv][V][nd] complex double
 void nullvecs_export(mg_ctx* c, int level, void* dst, cudaStream_t st);
 void restrict_apply(mg_ctx* c, int level, Vec coarse, Vec fine, cudaStream_t st);
-void prolong_apply(mg_ctx* c, int level, Vec fine, Vec coarse, cudaStream_t st);
+// fine = P coarse, or fine += P coarse (add)
+void prolong_apply(mg_ctx* c, int level, Vec fine, Vec coarse, cudaStream_t st, bool add = false);
 
 // ---------------------------------------------------------------- schur.cu
 // Red-black preconditioning (compact parity vectors: site s at s >> 1).

@@ -47,7 +47,7 @@ namespace {
 
 // scalar slots per level
 inline int slot(int level, int k) { return level * 8 + k; }
-enum { S_BETA = 0, S_NRM = 1, S_ALPHA = 2, S_R = 3, S_PR = 4, S_PP = 5 };
+enum { S_MR = 0, S_NRM = 1, S_ALPHA = 2, S_R = 3, S_PR = 4, S_PP = 5 };
 
 Vec vbuf(DevBuf& b, mg_prec p, size_t n, int nr = 1) {
   Vec v;
@@ -117,35 +117,47 @@ std::vector<double> read_slot(mg_ctx* c, int s, int nr, cudaStream_t st) {
   return v;
 }
 
-// x = MR_k(b) from a zero guess.  res (optional, level precision, not b):
-// receives the smoother's own residual b - A x, which MR keeps up to date.
-void mr_smooth(mg_ctx* c, int l, Vec x, Vec b, cudaStream_t st, const Vec* res = nullptr) {
+// x = MR_k(b) from a zero guess, or x += MR_k(b) (add).  res (optional, level
+// precision, not b): receives the smoother's own residual b - A x, which MR
+// keeps up to date.  The first step reads b itself and writes x and r, the
+// last one leaves r alone when nobody asks for it.
+void mr_smooth(mg_ctx* c, int l, Vec x, Vec b, cudaStream_t st, const Vec* res = nullptr,
+               bool add = false) {
   auto& w = c->ws->lv[l];
   Level& L = c->L[l];
+  const int nit = c->p.mr_iters;
+  if (nit == 0) {
+    if (!add) blas_zero(c, x, st);
+    if (res) blas_copy(c, *res, b, st);
+    return;
+  }
   if (l == 0 && smoother16_enabled(c)) {
     // the same MR steps on BF16 vectors with the BF16 copy of the operator
     Vec x16 = vbuf(w.s16x, MG_BF16, L.vec_elems(), x.nr);
     Vec r16 = vbuf(w.s16r, MG_BF16, L.vec_elems(), x.nr);
     Vec p16 = vbuf(w.s16p, MG_BF16, L.vec_elems(), x.nr);
-    blas_zero(c, x16, st);
     blas_copy(c, r16, b, st);
-    for (int k = 0; k < c->p.mr_iters; ++k) {
+    for (int k = 0; k < nit; ++k) {
       wilson16_apply(c, p16, r16, st);
-      blas_dot2(c, p16, r16, slot(l, S_PR), slot(l, S_PP), st);
-      blas_mr_update(c, x16, r16, p16, slot(l, S_PR), slot(l, S_PP), c->p.mr_omega, st);
+      blas_dot2(c, p16, r16, slot(l, S_PR), slot(l, S_PP), slot(l, S_MR), c->p.mr_omega, st);
+      blas_mr_update(c, x16, r16, p16, slot(l, S_MR), st, k == 0,
+                     k == nit - 1 && !res);
     }
-    blas_copy(c, x, x16, st);
+    if (add)
+      blas_add16(c, x, x16, st);
+    else
+      blas_copy(c, x, x16, st);
     if (res) blas_copy(c, *res, r16, st);
     return;
   }
   Vec r = res ? *res : vbuf(w.mrr, L.vprec, L.vec_elems(), x.nr);
   Vec p = vbuf(w.mrp, L.vprec, L.vec_elems(), x.nr);
-  blas_zero(c, x, st);
-  blas_copy(c, r, b, st);
-  for (int k = 0; k < c->p.mr_iters; ++k) {
-    level_apply(c, l, p, r, st);
-    blas_dot2(c, p, r, slot(l, S_PR), slot(l, S_PP), st);
-    blas_mr_update(c, x, r, p, slot(l, S_PR), slot(l, S_PP), c->p.mr_omega, st);
+  for (int k = 0; k < nit; ++k) {
+    const Vec& rk = k == 0 ? b : r;
+    level_apply(c, l, p, rk, st);
+    blas_dot2(c, p, rk, slot(l, S_PR), slot(l, S_PP), slot(l, S_MR), c->p.mr_omega, st);
+    blas_mr_update(c, x, r, p, slot(l, S_MR), st, k == 0 && !add,
+                   k == nit - 1 && !res, rk.p);
   }
 }
 
@@ -181,11 +193,13 @@ void schur_smooth(mg_ctx* c, int l, Vec z, Vec r, cudaStream_t st, const Vec* re
   eo_split(c, l, he, ho, r, st);
   eo_ainv(c, l, ht, he, st);
   eo_apply(c, l, EO_XC_MINUS_HOP, hr, ht, ho.p, 1, st);  // MR residual starts at b^
-  blas_zero(c, hx, st);
-  for (int k = 0; k < c->p.mr_iters; ++k) {
+  const int nit = c->p.mr_iters;
+  if (nit == 0) blas_zero(c, hx, st);
+  for (int k = 0; k < nit; ++k) {
     schur_apply(c, l, hp, hr, ht, st);
-    blas_dot2(c, hp, hr, slot(l, S_PR), slot(l, S_PP), st);
-    blas_mr_update(c, hx, hr, hp, slot(l, S_PR), slot(l, S_PP), c->p.mr_omega, st);
+    blas_dot2(c, hp, hr, slot(l, S_PR), slot(l, S_PP), slot(l, S_MR), c->p.mr_omega, st);
+    blas_mr_update(c, hx, hr, hp, slot(l, S_MR), st, k == 0,
+                   k == nit - 1 && !res);
   }
   eo_apply(c, l, EO_AINV_XC_MINUS_HOP, ht, hx, he.p, 0, st);
   eo_merge(c, l, z, ht, hx, st);
@@ -268,7 +282,7 @@ GcrOut gcr(mg_ctx* c, int l, Vec x, Vec b, bool precond, double tol, int maxiter
       Vec Zk = vbuf(*w.Z[k], L.vprec, n, nr), Wk = vbuf(*w.W[k], L.vprec, n, nr);
       if (precond) {
         if (outer && r.prec != L.vprec) {
-          blas_copy(c, rK, r, st);
+          if (k == 0) blas_copy(c, rK, r, st);  // later steps: blas_gcr_update's copy
           kcycle(c, l, Zk, rK, st, stats);
         } else {
           kcycle(c, l, Zk, r, st, stats);
@@ -292,11 +306,11 @@ GcrOut gcr(mg_ctx* c, int l, Vec x, Vec b, bool precond, double tol, int maxiter
         blas_axpy_multi(c, Wk, Ws, m, cs, -1.0, st);
         blas_axpy_multi(c, Zk, Zs, m, cs, -1.0, st);
       }
-      blas_norm2(c, Wk, slot(l, S_NRM), st, outer);
+      blas_norm2(c, Wk, slot(l, S_NRM), st, outer, true);
       blas_scale_invnorm(c, Wk, Zk, slot(l, S_NRM), st);
       blas_dot(c, Wk, r, slot(l, S_ALPHA), st);
-      blas_gcr_update(c, x, r, Zk, Wk, slot(l, S_ALPHA), st);
-      blas_norm2(c, r, slot(l, S_R), st);
+      blas_gcr_update(c, x, r, Zk, Wk, slot(l, S_ALPHA), slot(l, S_R),
+                      precond && outer && r.prec != L.vprec ? rK.p : nullptr, st);
       const std::vector<double> r2 = read_slot(c, slot(l, S_R), nr, st);
       out.iters++;
       done = check(r2);
@@ -335,16 +349,13 @@ void kcycle(mg_ctx* c, int l, Vec z, Vec r, cudaStream_t st, mg_solve_stats* sta
   auto& wc = c->ws->lv[nl];
   Vec rc = vbuf(wc.rhs, C.vprec, C.vec_elems(), nr), ec = vbuf(wc.x, C.vprec, C.vec_elems(), nr);
   const bool rb = c->p.red_black && L.have_schur;
-  auto smooth = [&](Vec out, Vec in, const Vec* res) {
-    if (rb)
-      schur_smooth(c, l, out, in, st, res);
-    else
-      mr_smooth(c, l, out, in, st, res);
-  };
   // pre-smooth; the smoother hands back kres = r - A z from its own
   // residual recurrence (equal to the recomputed residual in exact
   // arithmetic), which saves an operator apply per cycle
-  smooth(z, r, &kres);
+  if (rb)
+    schur_smooth(c, l, z, r, st, &kres);
+  else
+    mr_smooth(c, l, z, r, st, &kres);
   // coarse-grid correction
   restrict_apply(c, l, rc, kres, st);
   if (nl == c->nlevels - 1) {
@@ -364,13 +375,16 @@ void kcycle(mg_ctx* c, int l, Vec z, Vec r, cudaStream_t st, mg_solve_stats* sta
   } else {
     gcr(c, nl, ec, rc, true, c->p.inner_tol, c->p.inner_maxiter, st, stats, false);
   }
-  prolong_apply(c, l, tmp, ec, st);
-  blas_axpy_host(c, z, tmp, 1.0, 0.0, st);
+  prolong_apply(c, l, z, ec, st, true);
   // post-smooth
   level_apply(c, l, tmp, z, st);
   blas_sub(c, kres, r, tmp, st);
-  smooth(mrx, kres, nullptr);
-  blas_axpy_host(c, z, mrx, 1.0, 0.0, st);
+  if (rb) {
+    schur_smooth(c, l, mrx, kres, st);
+    blas_axpy_host(c, z, mrx, 1.0, 0.0, st);
+  } else {
+    mr_smooth(c, l, z, kres, st, nullptr, true);
+  }
 }
 
 }  // namespace

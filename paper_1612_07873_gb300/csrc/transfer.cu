@@ -557,7 +557,7 @@ __global__ void k_restrict(cpx<Rc>* __restrict__ coarse, const cpx<Rf>* __restri
 template <typename Rf, typename Rc>
 __global__ void k_prolong(cpx<Rf>* __restrict__ fine, const cpx<Rc>* __restrict__ coarse,
                           const cpx<Rf>* __restrict__ Vp, AggMap m, int nd, int nv, int nr,
-                          size_t fstride, size_t cstride) {
+                          size_t fstride, size_t cstride, int add) {
   const int rhs = blockIdx.x % nr;
   const size_t blk = blockIdx.x / nr, nblk = gridDim.x / nr;
   fine += rhs * fstride;
@@ -574,7 +574,7 @@ __global__ void k_prolong(cpx<Rf>* __restrict__ fine, const cpx<Rc>* __restrict_
     const cpx<Rf>* v = Vp + idx * nv;
     cpx<Rf> acc(Rf(0), Rf(0));
     for (int i = 0; i < nv; ++i) cmac(acc, v[i], cpx<Rf>(ec[i]));
-    fine[idx] = acc;
+    fine[idx] = add ? fine[idx] + acc : acc;
   }
 }
 
@@ -705,7 +705,7 @@ __global__ void __launch_bounds__(256) k_prolong12(cpx<Rf>* __restrict__ fine,
                                                   const cpx<Rc>* __restrict__ coarse,
                                                   const VT* __restrict__ Vp, AggMap m,
                                                   int nv, int nr, size_t fstride,
-                                                  size_t cstride) {
+                                                  size_t cstride, int add) {
   constexpr int ND = 12, CPL = VUnpack<VT, Rf>::CPL;
   constexpr int RPI = PW >= 12 ? 1 : (12 / PW > 6 ? 6 : 12 / PW);
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -741,6 +741,11 @@ __global__ void __launch_bounds__(256) k_prolong12(cpx<Rf>* __restrict__ fine,
         if (ok[j]) w[j][k] = ld_stream16(vr + 2 * k);
     }
     for (int b = 0; b < nr; ++b) {
+      // (add) the old values, loaded ahead of the products
+      cpx<Rf> old[RPI];
+#pragma unroll
+      for (int j = 0; j < RPI; ++j)
+        old[j] = add && ok[j] && q == 0 ? fine[b * fstride + frow[j]] : cpx<Rf>(Rf(0), Rf(0));
 #pragma unroll
       for (int j = 0; j < RPI; ++j) {
         const cpx<Rf>* c = cs + b * 2 * nv + coff[j];
@@ -756,7 +761,7 @@ __global__ void __launch_bounds__(256) k_prolong12(cpx<Rf>* __restrict__ fine,
         }
         acc.re += __shfl_xor_sync(0xffffffffu, acc.re, 1);
         acc.im += __shfl_xor_sync(0xffffffffu, acc.im, 1);
-        if (ok[j] && q == 0) fine[b * fstride + frow[j]] = acc;
+        if (ok[j] && q == 0) fine[b * fstride + frow[j]] = add ? old[j] + acc : acc;
       }
     }
   }
@@ -982,7 +987,7 @@ void restrict_apply(mg_ctx* c, int level, Vec coarse, Vec fine, cudaStream_t st)
   c->launches++;
 }
 
-void prolong_apply(mg_ctx* c, int level, Vec fine, Vec coarse, cudaStream_t st) {
+void prolong_apply(mg_ctx* c, int level, Vec fine, Vec coarse, cudaStream_t st, bool add) {
   Level& F = c->L[level];
   Level& C = c->L[level + 1];
   GB_REQUIRE(F.have_V, MG_ERR_STATE, "prolong: null vectors not set");
@@ -1008,16 +1013,16 @@ void prolong_apply(mg_ctx* c, int level, Vec fine, Vec coarse, cudaStream_t st) 
         if (coarse.prec == MG_F64)
           k_prolong12<float, double, bf16c, PW><<<C.g.vol, 256, smem2, st>>>(
               (cpx<float>*)fine.p, (const cpx<double>*)coarse.p, F.Vp16.as<bf16c>(), m, nv, nr,
-              fine.n, coarse.n);
+              fine.n, coarse.n, int(add));
         else
           k_prolong12<float, float, bf16c, PW><<<C.g.vol, 256, smem2, st>>>(
               (cpx<float>*)fine.p, (const cpx<float>*)coarse.p, F.Vp16.as<bf16c>(), m, nv, nr,
-              fine.n, coarse.n);
+              fine.n, coarse.n, int(add));
       } else {
         GB_TRANSFER_DISPATCH(F.vprec, coarse.prec, Rf, Rc,
                              (k_prolong12<Rf, Rc, cpx<Rf>, PW><<<C.g.vol, 256, smem2, st>>>(
                                  (cpx<Rf>*)fine.p, (const cpx<Rc>*)coarse.p,
-                                 F.Vp.as<cpx<Rf>>(), m, nv, nr, fine.n, coarse.n)));
+                                 F.Vp.as<cpx<Rf>>(), m, nv, nr, fine.n, coarse.n, int(add))));
       }
     };
     switch (pw) {
@@ -1038,7 +1043,7 @@ void prolong_apply(mg_ctx* c, int level, Vec fine, Vec coarse, cudaStream_t st) 
   GB_TRANSFER_DISPATCH(F.vprec, coarse.prec, Rf, Rc,
                        (k_prolong<Rf, Rc><<<unsigned(blocks) * nr, 256, 0, st>>>(
                            (cpx<Rf>*)fine.p, (const cpx<Rc>*)coarse.p, F.Vp.as<cpx<Rf>>(), m,
-                           F.nd, nv, nr, fine.n, coarse.n)));
+                           F.nd, nv, nr, fine.n, coarse.n, int(add))));
   GB_LAUNCH_CHECK();
   c->launches++;
 }
