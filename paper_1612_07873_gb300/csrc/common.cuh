@@ -127,6 +127,33 @@ __device__ __forceinline__ void fma2(f32x2& a, f32x2 b, f32x2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a) : "l"(b), "l"(c));
 }
 
+// -------------------------------------------- FP32 <-> FP64 conversions
+// Exact FP32 -> FP64 conversion by integer operations.  The hardware
+// conversion runs on the FP64 pipe (two lanes per clock and SM on GB300: 16
+// cycles a warp), which bounds the kernels that mix FP32 and FP64 vectors;
+// zeros, subnormals, infinities and NaN take it.
+static __device__ __noinline__ double f2d_special(float f) { return double(f); }
+__device__ __forceinline__ double f2d(float f) {
+  const uint32_t u = __float_as_uint(f), e = u & 0x7f800000u;
+  if (e == 0u || e == 0x7f800000u) {
+    // (a call: predicated or selected, the conversion would run every time)
+    return (u << 1) == 0u ? __hiloint2double(int(u), 0) : f2d_special(f);
+  }
+  const uint32_t hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u);
+  return __hiloint2double(int(hi), int(u << 29));
+}
+// FP64 -> FP32, round to nearest even, by integer operations likewise (results
+// in the normal range of FP32, below 2^127; others take the conversion)
+static __device__ __noinline__ float d2f_special(double d) { return float(d); }
+__device__ __forceinline__ float d2f(double d) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+  const uint32_t e = uint32_t(u >> 52) & 0x7ffu;
+  if (e - 897u >= 253u) return (u << 1) == 0ull ? __uint_as_float(uint32_t(u >> 32)) : d2f_special(d);
+  const unsigned long long t = (u & 0x7fffffffffffffffull) - (896ull << 52);
+  const uint32_t r = uint32_t((t + 0x0fffffffull + ((t >> 29) & 1ull)) >> 29);
+  return __uint_as_float(r | (uint32_t(u >> 32) & 0x80000000u));
+}
+
 // ------------------------------------------------------------------ storage
 // Complex element types of the link store.  16-bit forms carry a per-site
 // FP32 scale: value = scale * stored.

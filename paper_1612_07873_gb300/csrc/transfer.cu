@@ -58,6 +58,23 @@ AggMap make_map(const Level& f, const Level& c) {
   return m;
 }
 
+// first fine site of an aggregate, and the offset of its local site ls from it
+__device__ __forceinline__ int agg_origin(const AggMap& m, int xc) {
+  int cc[4];
+  site_coords(m.coarse, xc, cc);
+  return cc[0] * m.b[0] + m.fine.stride[1] * cc[1] * m.b[1] +
+         m.fine.stride[2] * cc[2] * m.b[2] + m.fine.stride[3] * cc[3] * m.b[3];
+}
+__device__ __forceinline__ int local_offset(const AggMap& m, int ls) {
+  int l0 = ls % m.b[0];
+  ls /= m.b[0];
+  int l1 = ls % m.b[1];
+  ls /= m.b[1];
+  int l2 = ls % m.b[2];
+  int l3 = ls / m.b[2];
+  return l0 + m.fine.stride[1] * l1 + m.fine.stride[2] * l2 + m.fine.stride[3] * l3;
+}
+
 // ---------------------------------------------------------------------------
 // Float-float complex numbers: value = (rh + rl) + i (ih + il) with
 // |rl| <= ulp(rh) / 2 (likewise il) whenever one is stored.  About 48
@@ -144,6 +161,12 @@ __device__ __forceinline__ ff ff_shfl_xor(ff a, int o) {
 __device__ __forceinline__ void ws_store(ffc& d, double2 v) { d = ffc_from(v); }
 __device__ __forceinline__ void ws_store(double2& d, double2 v) { d = v; }
 __device__ __forceinline__ double2 ws_load(const ffc& a) { return ffc_to(a); }
+// the same off the FP64 conversion path, for a kernel that does little else
+// (in the QR and the scatter its special-case calls cost more than they save)
+__device__ __forceinline__ double2 ws_widen(const ffc& a) {
+  return make_double2(f2d(a.rh) + f2d(a.rl), f2d(a.ih) + f2d(a.il));
+}
+__device__ __forceinline__ double2 ws_widen(const double2& a) { return a; }
 __device__ __forceinline__ double2 ws_load(const double2& a) { return a; }
 
 // raw [Nv][V][nd] -> W [agg][chi][Nv][rows]
@@ -458,6 +481,261 @@ __global__ void __launch_bounds__(NT) k_block_qr(ffc* __restrict__ W, int rows, 
   }
 }
 
+// Sum over a warp of 2 P float-float values per lane (P <= 4) by recursive
+// halving: in the first three steps a lane keeps half of its values (indexed
+// by lane bits 4, 3, 2), the last two steps add the remaining one: 9 additions
+// instead of 40.  Returns the total of value index (lane >> 2) & 7 in s (with
+// 8 values).
+__device__ __forceinline__ ff warp_sum8(ff (&x)[8], int lane) {
+#pragma unroll
+  for (int h = 4; h >= 1; h >>= 1) {
+    const int o = 4 * h;  // 16, 8, 4
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const ff give = up ? x[k] : x[k + h];
+      const ff keep = up ? x[k + h] : x[k];
+      x[k] = ff_add(keep, ff_shfl_xor(give, o));
+    }
+  }
+  ff t = x[0];
+  t = ff_add(t, ff_shfl_xor(t, 2));
+  t = ff_add(t, ff_shfl_xor(t, 1));
+  return t;
+}
+
+// The Gram-Schmidt of k_block_qr in panels of P columns, for blocks of at
+// most 256 RPT rows: a finished column q is loaded once per panel for the
+// inner products with its P columns and once for the update, instead of twice
+// per column (those loads, from L2, and the reductions behind them bounded the
+// column form: issue a third busy).  Within a panel the columns are
+// orthogonalised one after the other from registers.  The panel's columns are
+// read from the raw vectors, so no gather pass runs before.  Column order,
+// arithmetic, the second-pass criterion and the status bits are those of
+// k_block_qr; a column that needs the second pass repeats its projection on
+// all earlier columns.
+// 16^3x32, 24 vectors, 4^4 aggregates (1024 blocks of 1536 rows): gather and QR
+// 4.86 -> 3.29 ms.
+// Sec. 3.4 step 3: QR of every (aggregate, chirality) block.
+template <int RPT, int P>
+__global__ void __launch_bounds__(256, P * RPT >= 16 ? 2 : 3)
+    k_block_qr_panel(ffc* __restrict__ W, const double2* __restrict__ raw, AggMap m, int nd,
+                     int nv, int* status) {
+  constexpr int NW = 8;
+  static_assert(P <= 4, "panel width");
+  __shared__ ff sh[33];
+  __shared__ ff part[NW][kQrMaxVec][2 * P];
+  __shared__ ffc coef[kQrMaxVec][P];
+  __shared__ float fsum[NW];
+  const int half = nd / 2, rows = m.per * half;
+  const int xc = blockIdx.x >> 1, chi = blockIdx.x & 1;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  ffc* B = W + size_t(blockIdx.x) * nv * rows;
+  const size_t vstride = size_t(m.fine.vol) * nd;
+  // this thread's rows: entry of the raw vector
+  unsigned at[RPT];
+  {
+    const int base = agg_origin(m, xc);
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) {
+      const int row = tid + r * 256;
+      const int ls = row < rows ? row / half : 0;
+      at[r] = unsigned(base + local_offset(m, ls)) * nd + chi * half + (row - ls * half);
+    }
+  }
+  auto has = [&](int r) { return tid + r * 256 < rows; };
+  auto norm2 = [&](const ffc* v) {
+    ff s = {0.f, 0.f};
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) {
+      ff_mac(s, v[r].rh, v[r].rl, v[r].rh, v[r].rl);
+      ff_mac(s, v[r].ih, v[r].il, v[r].ih, v[r].il);
+    }
+    return s;
+  };
+  auto dot = [&](ff& dr, ff& di, const ffc& q, const ffc& v) {  // += conj(q) v
+    ff_mac(dr, q.rh, q.rl, v.rh, v.rl);
+    ff_mac(dr, q.ih, q.il, v.ih, v.il);
+    ff_mac(di, q.rh, q.rl, v.ih, v.il);
+    ff_mac(di, -q.ih, -q.il, v.rh, v.rl);
+  };
+  auto sub = [&](ffc& v, const ffc& c, const ffc& q) {  // v -= c q
+    ff_msub(v.rh, v.rl, c.rh, c.rl, q.rh, q.rl);
+    ff_msub(v.rh, v.rl, -c.ih, -c.il, q.ih, q.il);
+    ff_msub(v.ih, v.il, c.rh, c.rl, q.ih, q.il);
+    ff_msub(v.ih, v.il, c.ih, c.il, q.rh, q.rl);
+  };
+  // Frobenius norm of the block for the rank test (a threshold: FP32 will do)
+  float f = 0.f;
+  for (int i = 0; i < nv; ++i)
+#pragma unroll
+    for (int r = 0; r < RPT; ++r)
+      if (has(r)) {
+        const double2 v = raw[size_t(i) * vstride + at[r]];
+        const float a = float(v.x), b = float(v.y);
+        f = fmaf(a, a, fmaf(b, b, f));
+      }
+  for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+  if (lane == 0) fsum[warp] = f;
+  __syncthreads();
+  double scale = 0.0;
+  for (int w = 0; w < NW; ++w) scale += double(fsum[w]);
+  scale = sqrt(scale);
+
+  for (int i0 = 0; i0 < nv; i0 += P) {
+    const int pc = min(P, nv - i0);
+    ffc v[P][RPT];
+#pragma unroll
+    for (int c = 0; c < P; ++c)
+#pragma unroll
+      for (int r = 0; r < RPT; ++r)
+        v[c][r] = c < pc && has(r) ? ffc_from(raw[size_t(i0 + c) * vstride + at[r]])
+                                   : ffc{0.f, 0.f, 0.f, 0.f};
+    auto store8 = [&](ff (&x)[8], int j) {
+      const ff t = warp_sum8(x, lane);
+      const int k = (lane >> 2) & 7;
+      if ((lane & 3) == 0 && k < 2 * P) part[warp][j][k] = t;
+    };
+    {
+      // squared norms before the projection: entry i0
+      ff x[8];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        x[2 * c] = c < P ? norm2(v[c < P ? c : 0]) : ff{0.f, 0.f};
+        x[2 * c + 1] = ff{0.f, 0.f};
+      }
+      store8(x, i0);
+    }
+    for (int j = 0; j < i0; ++j) {
+      const ffc* q = B + size_t(j) * rows + tid;
+      ff x[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) x[k] = ff{0.f, 0.f};
+#pragma unroll
+      for (int r = 0; r < RPT; ++r)
+        if (has(r)) {
+          const ffc qv = q[r * 256];
+#pragma unroll
+          for (int c = 0; c < P; ++c) dot(x[2 * c], x[2 * c + 1], qv, v[c][r]);
+        }
+      store8(x, j);
+    }
+    __syncthreads();
+    for (int t = tid; t < (i0 + 1) * P; t += 256) {
+      const int j = t / P, c = t - j * P;
+      ff cr = {0.f, 0.f}, ci = {0.f, 0.f};
+      for (int w = 0; w < NW; ++w) {
+        cr = ff_add(cr, part[w][j][2 * c]);
+        ci = ff_add(ci, part[w][j][2 * c + 1]);
+      }
+      coef[j][c] = ffc{cr.hi, cr.lo, ci.hi, ci.lo};
+    }
+    __syncthreads();
+    double n0[P];
+#pragma unroll
+    for (int c = 0; c < P; ++c) n0[c] = ff_to(ff{coef[i0][c].rh, coef[i0][c].rl});
+    for (int j = 0; j < i0; ++j) {
+      const ffc* q = B + size_t(j) * rows + tid;
+#pragma unroll
+      for (int r = 0; r < RPT; ++r)
+        if (has(r)) {
+          const ffc qv = q[r * 256];
+#pragma unroll
+          for (int c = 0; c < P; ++c) sub(v[c][r], coef[j][c], qv);
+        }
+    }
+    __syncthreads();  // coef and part are rewritten below
+    // the panel's own columns, one after the other (c is uniform)
+#pragma unroll
+    for (int c = 0; c < P; ++c) {
+      if (c >= pc) break;
+      const int i = i0 + c;
+      double n1 = blk_sum_ff(norm2(v[c]), sh);
+      if (i > 0) {
+        // (see k_block_qr) status bit 2: float-float cannot resolve the column
+        if (n1 < 1e-4 * n0[c] && tid == 0) atomicOr(status, 2);
+        if (n1 < 0.5 * n0[c]) {
+          // second pass: the projection on all earlier columns again
+          for (int j = 0; j < i; ++j) {
+            const ffc* q = B + size_t(j) * rows + tid;
+            ff dr = {0.f, 0.f}, di = {0.f, 0.f};
+#pragma unroll
+            for (int r = 0; r < RPT; ++r)
+              if (has(r)) dot(dr, di, q[r * 256], v[c][r]);
+            for (int o = 16; o > 0; o >>= 1) {
+              dr = ff_add(dr, ff_shfl_xor(dr, o));
+              di = ff_add(di, ff_shfl_xor(di, o));
+            }
+            if (lane == 0) {
+              part[warp][j][0] = dr;
+              part[warp][j][1] = di;
+            }
+          }
+          __syncthreads();
+          if (tid < i) {
+            ff cr = {0.f, 0.f}, ci = {0.f, 0.f};
+            for (int w = 0; w < NW; ++w) {
+              cr = ff_add(cr, part[w][tid][0]);
+              ci = ff_add(ci, part[w][tid][1]);
+            }
+            coef[tid][0] = ffc{cr.hi, cr.lo, ci.hi, ci.lo};
+          }
+          __syncthreads();
+          for (int j = 0; j < i; ++j) {
+            const ffc* q = B + size_t(j) * rows + tid;
+#pragma unroll
+            for (int r = 0; r < RPT; ++r)
+              if (has(r)) sub(v[c][r], coef[j][0], q[r * 256]);
+          }
+          __syncthreads();
+          n1 = blk_sum_ff(norm2(v[c]), sh);
+        }
+      }
+      const double nrm = sqrt(n1);
+      float sh_inv = 0.f, sl_inv = 0.f;
+      if (nrm <= 1e-12 * scale) {
+        if (tid == 0) atomicOr(status, 1);
+      } else {
+        ff_split(1.0 / nrm, sh_inv, sl_inv);
+      }
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) {
+        ff_scale(v[c][r].rh, v[c][r].rl, sh_inv, sl_inv);
+        ff_scale(v[c][r].ih, v[c][r].il, sh_inv, sl_inv);
+        if (has(r)) B[size_t(i) * rows + tid + r * 256] = v[c][r];
+      }
+      if (c + 1 < P) {
+        // project the rest of the panel on it
+        ff x[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) x[k] = ff{0.f, 0.f};
+#pragma unroll
+        for (int c2 = c + 1; c2 < P; ++c2)
+#pragma unroll
+          for (int r = 0; r < RPT; ++r) dot(x[2 * c2], x[2 * c2 + 1], v[c][r], v[c2][r]);
+        store8(x, 0);
+        __syncthreads();
+        if (tid < P) {
+          ff cr = {0.f, 0.f}, ci = {0.f, 0.f};
+          for (int w = 0; w < NW; ++w) {
+            cr = ff_add(cr, part[w][0][2 * tid]);
+            ci = ff_add(ci, part[w][0][2 * tid + 1]);
+          }
+          coef[0][tid] = ffc{cr.hi, cr.lo, ci.hi, ci.lo};
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c2 = c + 1; c2 < P; ++c2) {
+          const ffc k = coef[0][c2];
+#pragma unroll
+          for (int r = 0; r < RPT; ++r) sub(v[c2][r], k, v[c][r]);
+        }
+      }
+    }
+    __syncthreads();  // the panel's columns are visible to the CTA; part, coef free
+  }
+}
+
 // QR of every (aggregate, chirality) block of W; false if a block is too tall.
 #define GB_QR_LAUNCH(KERN, WT)                                                       \
   bool launch_##KERN(WT* W, int rows, int nv, int nblk, int* status, cudaStream_t st) { \
@@ -482,31 +760,84 @@ __global__ void __launch_bounds__(NT) k_block_qr(ffc* __restrict__ W, int rows, 
   }
 // 256 threads up to 4096 rows (16 rows per thread), 1024 threads beyond;
 // false if a block is too tall or has too many vectors
-GB_QR_LAUNCH(k_block_qr, ffc)
 GB_QR_LAUNCH(k_block_qr64, double2)
 #undef GB_QR_LAUNCH
 
+int grid_for(size_t n) {
+  long long b = (long long)((n + 255) / 256);
+  if (b > 152 * 32) b = 152 * 32;
+  return int(b < 1 ? 1 : b);
+}
+
+// Float-float QR of every (aggregate, chirality) block of the raw vectors into
+// W: panels up to 2048 rows (the panel as wide as two or three CTAs' registers
+// allow), beyond that gathered and column by column; false if a block is too
+// tall.
+bool block_qr_ff(ffc* W, const double2* raw, const AggMap& m, int nd, int nv, int* status,
+                 cudaStream_t st) {
+  const int rows = m.per * nd / 2, nblk = m.coarse.vol * 2;
+  if (nv > kQrMaxVec || rows > 1024 * 24) return false;
+  if (rows <= 256)
+    k_block_qr_panel<1, 4><<<nblk, 256, 0, st>>>(W, raw, m, nd, nv, status);
+  else if (rows <= 512)
+    k_block_qr_panel<2, 4><<<nblk, 256, 0, st>>>(W, raw, m, nd, nv, status);
+  else if (rows <= 1024)
+    k_block_qr_panel<4, 4><<<nblk, 256, 0, st>>>(W, raw, m, nd, nv, status);
+  else if (rows <= 1536)
+    k_block_qr_panel<6, 3><<<nblk, 256, 0, st>>>(W, raw, m, nd, nv, status);
+  else if (rows <= 2048)
+    k_block_qr_panel<8, 2><<<nblk, 256, 0, st>>>(W, raw, m, nd, nv, status);
+  else {
+    const size_t elems = size_t(nv) * m.fine.vol * nd;
+    k_mgs_gather<ffc><<<grid_for(elems), 256, 0, st>>>(W, raw, m, nd, nv);
+    if (rows <= 4096)
+      k_block_qr<16, 256><<<nblk, 256, 0, st>>>(W, rows, nv, status);
+    else if (rows <= 8192)
+      k_block_qr<8, 1024><<<nblk, 1024, 0, st>>>(W, rows, nv, status);
+    else if (rows <= 16384)
+      k_block_qr<16, 1024><<<nblk, 1024, 0, st>>>(W, rows, nv, status);
+    else
+      k_block_qr<24, 1024><<<nblk, 1024, 0, st>>>(W, rows, nv, status);
+  }
+  return true;
+}
+
 // W -> Vp [V][nd][Nv] (R)
 // Sec. 3.4 step 3: the orthonormal blocks as prolongator rows.
+// CTA (block, slice) moves 32-row tiles of one (aggregate, chirality) block
+// through shared memory: rows of a column are read, vectors of a row written
+// contiguously, and the site arithmetic is per row, not per entry (24 vectors
+// of 16^3x32: 366 -> 187 us, 133 us to move the bytes).
 template <typename R, typename WT>
-__global__ void k_mgs_scatter(cpx<R>* __restrict__ Vp, const WT* __restrict__ W, AggMap m,
-                              int nd, int nv) {
-  const int half = nd / 2;
-  const int rows = m.per * half;
-  size_t total = size_t(nv) * m.fine.vol * nd;
-  for (size_t idx = blockIdx.x * size_t(blockDim.x) + threadIdx.x; idx < total;
-       idx += size_t(gridDim.x) * blockDim.x) {
-    // idx enumerates Vp order: (site, dof, vec)
-    int i = int(idx % nv);
-    size_t t = idx / nv;
-    int a = int(t % nd);
-    int s = int(t / nd);
-    int c[4];
-    site_coords(m.fine, s, c);
-    int ag = agg_of(m, c), ls = local_of(m, c);
-    int chi = a / half, ad = a - chi * half;
-    const double2 v = ws_load(W[((size_t(ag) * 2 + chi) * nv + i) * rows + size_t(ls) * half + ad]);
-    Vp[idx] = cpx<R>(R(v.x), R(v.y));
+__global__ void __launch_bounds__(256) k_mgs_scatter(cpx<R>* __restrict__ Vp,
+                                                     const WT* __restrict__ W, AggMap m, int nd,
+                                                     int nv) {
+  extern __shared__ __align__(16) unsigned char scat_smem[];
+  cpx<R>* tile = reinterpret_cast<cpx<R>*>(scat_smem);  // [32][nv + 1]
+  __shared__ size_t at[32];
+  const int half = nd / 2, rows = m.per * half;
+  const int xc = blockIdx.x >> 1, chi = blockIdx.x & 1;
+  const WT* B = W + size_t(blockIdx.x) * nv * rows;
+  const int base = agg_origin(m, xc);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int r0 = blockIdx.y * 32; r0 < rows; r0 += gridDim.y * 32) {
+    const int row = r0 + lane;
+    if (warp == 0 && row < rows) {
+      const int ls = row / half;
+      at[lane] = (size_t(base + local_offset(m, ls)) * nd + chi * half + (row - ls * half)) * nv;
+    }
+    for (int i = warp; i < nv; i += 8)
+      if (row < rows) {
+        const double2 v = ws_load(B[size_t(i) * rows + row]);
+        tile[lane * (nv + 1) + i] = cpx<R>(R(v.x), R(v.y));
+      }
+    __syncthreads();
+    const int n = min(32, rows - r0) * nv;
+    for (int t = threadIdx.x; t < n; t += 256) {
+      const int r = t / nv, i = t - r * nv;
+      Vp[at[r] + i] = tile[r * (nv + 1) + i];
+    }
+    __syncthreads();
   }
 }
 
@@ -584,22 +915,6 @@ __global__ void k_prolong(cpx<Rf>* __restrict__ fine, const cpx<Rc>* __restrict_
 // are tabulated once per CTA in shared memory and the per-row index work is
 // one table lookup.  Vp rows (Nv coefficients of one fine dof, 96 B / 192 B
 // for Nv = 24 in FP32 / FP64) are read as 16-byte vectors.
-
-__device__ __forceinline__ int agg_origin(const AggMap& m, int xc) {
-  int cc[4];
-  site_coords(m.coarse, xc, cc);
-  return cc[0] * m.b[0] + m.fine.stride[1] * cc[1] * m.b[1] +
-         m.fine.stride[2] * cc[2] * m.b[2] + m.fine.stride[3] * cc[3] * m.b[3];
-}
-__device__ __forceinline__ int local_offset(const AggMap& m, int ls) {
-  int l0 = ls % m.b[0];
-  ls /= m.b[0];
-  int l1 = ls % m.b[1];
-  ls /= m.b[1];
-  int l2 = ls % m.b[2];
-  int l3 = ls / m.b[2];
-  return l0 + m.fine.stride[1] * l1 + m.fine.stride[2] * l2 + m.fine.stride[3] * l3;
-}
 
 // A 16-byte word of Vp as CPL complex numbers in the fine vector precision:
 // Vp stored in the vector precision, or in BF16 (the fine-level copy used
@@ -769,30 +1084,41 @@ __global__ void __launch_bounds__(256) k_prolong12(cpx<Rf>* __restrict__ fine,
 
 // W [agg][chi][Nv][rows] -> out [Nv][V][nd] (FP64)
 // Sec. 3.4 step 3: orthonormal blocks back to the null-vector layout.
+// One CTA per (aggregate, chirality) block and slice of its rows; the site
+// arithmetic per row, not per entry, and the widening off the FP64 pipe (24
+// vectors of 16^3x32: 422 -> 188 us).
 template <typename WT>
-__global__ void k_blocked_to_vectors(double2* __restrict__ out, const WT* __restrict__ W,
-                                  AggMap m, int nd, int nv) {
-  const int half = nd / 2;
-  const int rows = m.per * half;
-  size_t total = size_t(nv) * m.fine.vol * nd;
-  for (size_t idx = blockIdx.x * size_t(blockDim.x) + threadIdx.x; idx < total;
-       idx += size_t(gridDim.x) * blockDim.x) {
-    int a = int(idx % nd);
-    size_t t = idx / nd;
-    int s = int(t % m.fine.vol);
-    int i = int(t / m.fine.vol);
-    int c[4];
-    site_coords(m.fine, s, c);
-    int ag = agg_of(m, c), ls = local_of(m, c);
-    int chi = a / half, ad = a - chi * half;
-    out[idx] = ws_load(W[((size_t(ag) * 2 + chi) * nv + i) * rows + size_t(ls) * half + ad]);
+__global__ void __launch_bounds__(256) k_blocked_to_vectors(double2* __restrict__ out,
+                                                            const WT* __restrict__ W, AggMap m,
+                                                            int nd, int nv) {
+  const int half = nd / 2, rows = m.per * half;
+  const int xc = blockIdx.x >> 1, chi = blockIdx.x & 1;
+  const WT* B = W + size_t(blockIdx.x) * nv * rows;
+  const int base = agg_origin(m, xc);
+  const size_t vstride = size_t(m.fine.vol) * nd;
+  for (int row = blockIdx.y * 256 + threadIdx.x; row < rows; row += gridDim.y * 256) {
+    const int ls = row / half;
+    double2* o = out + size_t(base + local_offset(m, ls)) * nd + chi * half + (row - ls * half);
+    const WT* w = B + row;
+    int i = 0;
+    for (; i + 4 <= nv; i += 4) {
+      WT v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = w[size_t(i + k) * rows];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) o[size_t(i + k) * vstride] = ws_widen(v[k]);
+    }
+    for (; i < nv; ++i) o[size_t(i) * vstride] = ws_widen(w[size_t(i) * rows]);
   }
 }
 
-int grid_for(size_t n) {
-  long long b = (long long)((n + 255) / 256);
-  if (b > 152 * 32) b = 152 * 32;
-  return int(b < 1 ? 1 : b);
+// slices of a block's rows: enough CTAs to fill the chip
+dim3 block_grid(const AggMap& m, int nd, int tile) {
+  const int nblk = m.coarse.vol * 2, rows = m.per * nd / 2;
+  int y = ceil_div(152 * 16, nblk);
+  const int most = ceil_div(rows, tile);
+  if (y > most) y = most;
+  return dim3(unsigned(nblk), unsigned(y < 1 ? 1 : y));
 }
 
 }  // namespace
@@ -814,10 +1140,8 @@ void block_orthonormalise(mg_ctx* c, int level, cudaStream_t st) {
   ProfScope ps(c->prof, st, "block_orth", level, double(elems) * 16.0 * 2,
                8.0 * nv * (nv - 1) * 2.0 * rows * nblk);
   clear_status(c, st);
-  k_mgs_gather<ffc><<<grid_for(elems), 256, 0, st>>>(F.orth64.as<ffc>(), F.raw.as<double2>(), m,
-                                                     nd, nv);
-  GB_LAUNCH_CHECK();
-  GB_REQUIRE(launch_k_block_qr(F.orth64.as<ffc>(), rows, nv, nblk, c->status.as<int>(), st),
+  GB_REQUIRE(block_qr_ff(F.orth64.as<ffc>(), F.raw.as<double2>(), m, nd, nv,
+                         c->status.as<int>(), st),
              MG_ERR_ARG, "aggregate block too large (rows > 24576 or nvec > 64)");
   GB_LAUNCH_CHECK();
   int qs = read_status(c, st);
@@ -833,10 +1157,12 @@ void block_orthonormalise(mg_ctx* c, int level, cudaStream_t st) {
     c->launches += 2;
   }
   auto scatter = [&](auto* W) {
+    const dim3 grid = block_grid(m, nd, 32);
+    const size_t smem = size_t(32) * (nv + 1) * prec_bytes_complex(F.vprec);
     if (F.vprec == MG_F64)
-      k_mgs_scatter<<<grid_for(elems), 256, 0, st>>>(F.Vp.as<cpx<double>>(), W, m, nd, nv);
+      k_mgs_scatter<<<grid, 256, smem, st>>>(F.Vp.as<cpx<double>>(), W, m, nd, nv);
     else
-      k_mgs_scatter<<<grid_for(elems), 256, 0, st>>>(F.Vp.as<cpx<float>>(), W, m, nd, nv);
+      k_mgs_scatter<<<grid, 256, smem, st>>>(F.Vp.as<cpx<float>>(), W, m, nd, nv);
   };
   if (F.orth_ff)
     scatter(F.orth64.as<ffc>());
@@ -1053,13 +1379,12 @@ void nullvecs_export(mg_ctx* c, int level, void* dst, cudaStream_t st) {
   Level& C = c->L[level + 1];
   GB_REQUIRE(F.have_V, MG_ERR_STATE, "get_nullvecs: not available");
   AggMap m = make_map(F, C);
-  const size_t elems = size_t(F.nvec) * F.g.vol * F.nd;
   if (F.orth_ff)
-    k_blocked_to_vectors<<<grid_for(elems), 256, 0, st>>>((double2*)dst, F.orth64.as<ffc>(), m,
-                                                         F.nd, F.nvec);
+    k_blocked_to_vectors<<<block_grid(m, F.nd, 256), 256, 0, st>>>(
+        (double2*)dst, F.orth64.as<ffc>(), m, F.nd, F.nvec);
   else
-    k_blocked_to_vectors<<<grid_for(elems), 256, 0, st>>>((double2*)dst, F.orth64.as<double2>(),
-                                                         m, F.nd, F.nvec);
+    k_blocked_to_vectors<<<block_grid(m, F.nd, 256), 256, 0, st>>>(
+        (double2*)dst, F.orth64.as<double2>(), m, F.nd, F.nvec);
   GB_LAUNCH_CHECK();
   c->launches++;
 }
@@ -1170,12 +1495,8 @@ extern "C" mg_status mg_block_orthonormalise_noalloc(const void* vecs_dev, void*
                cudaSuccess &&
            cudaStreamSynchronize(st) == cudaSuccess;
   };
-  k_mgs_gather<ffc><<<grid_for(elems), 256, 0, st>>>(slot.scratch, (const double2*)vecs_dev, m,
-                                                     ndof, nvec);
-  if (cudaGetLastError() != cudaSuccess)
-    return fail(MG_ERR_CUDA, "noalloc: gather launch failed");
   const int nblk = m.coarse.vol * 2;
-  if (!launch_k_block_qr(slot.scratch, rows, nvec, nblk, slot.status, st))
+  if (!block_qr_ff(slot.scratch, (const double2*)vecs_dev, m, ndof, nvec, slot.status, st))
     return fail(MG_ERR_ARG, "noalloc: aggregate block too large for the block QR");
   if (cudaGetLastError() != cudaSuccess)
     return fail(MG_ERR_CUDA, "noalloc: block QR launch failed");
@@ -1195,11 +1516,11 @@ extern "C" mg_status mg_block_orthonormalise_noalloc(const void* vecs_dev, void*
     launch_k_block_qr64(scratch64, rows, nvec, nblk, slot.status, st);
     if (cudaGetLastError() != cudaSuccess)
       return fail(MG_ERR_CUDA, "noalloc: block QR launch failed");
-    k_blocked_to_vectors<<<grid_for(elems), 256, 0, st>>>((double2*)out_dev, scratch64, m, ndof,
-                                                         nvec);
+    k_blocked_to_vectors<<<block_grid(m, ndof, 256), 256, 0, st>>>((double2*)out_dev, scratch64,
+                                                                   m, ndof, nvec);
   } else {
-    k_blocked_to_vectors<<<grid_for(elems), 256, 0, st>>>((double2*)out_dev, slot.scratch, m,
-                                                         ndof, nvec);
+    k_blocked_to_vectors<<<block_grid(m, ndof, 256), 256, 0, st>>>((double2*)out_dev,
+                                                                   slot.scratch, m, ndof, nvec);
   }
   if (cudaGetLastError() != cudaSuccess)
     return fail(MG_ERR_CUDA, "noalloc: scatter launch failed");

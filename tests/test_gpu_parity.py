@@ -418,3 +418,31 @@ def test_call_order_and_argument_errors(gpu_lib):
     with pytest.raises(gb.MGError) as e:
         gb.mg_create(p, to_dev(syn.gauge_field((6, 4, 4, 4), 0.1, 1)))
     assert e.value.status == gb.MG_ERR_ARG
+
+
+@pytest.mark.parametrize("dims,block,nv", [
+    ((4, 4, 4, 4), (2, 2, 2, 4), 5),       # 192 rows, panels of four, a last one of one
+    ((4, 4, 4, 8), (4, 2, 2, 4), 18),      # 384 rows
+    ((6, 4, 4, 4), (3, 4, 2, 4), 7),       # 576 rows
+    ((8, 4, 4, 4), (4, 4, 2, 4), 24),  # 768 rows
+    ((4, 4, 4, 4), (4, 4, 4, 4), 25),      # 1536 rows, panels of three, a last one of one
+    ((6, 4, 4, 4), (6, 4, 2, 4), 9),  # 1152 rows
+    ((6, 4, 4, 6), (6, 4, 2, 6), 3),       # 1728 rows, panels of two, a last one of one
+])
+@pytest.mark.parametrize("parallel", [False, True])
+def test_block_orthonormalise_panels(gpu_lib, dims, block, nv, parallel):
+    """Every panel width of the block QR, widths that do not divide the number
+    of vectors, and columns that need the second pass (parallel: column k gets
+    half of its norm from column 0, across and within panels)."""
+    gb = gpu_lib
+    mg, U = make_ctx(gb, dims, [block], [nv])
+    v = syn.gaussian_field((nv, lat.volume(dims), 12), 23)
+    if parallel:
+        for k in (1, nv - 1):
+            v[k] = 0.5 * v[k] + 2.0 * v[0]
+    gb.mg_set_nullvecs(mg.ctx, 0, to_dev(v))
+    out = torch.empty((nv, lat.volume(dims), 12), dtype=torch.complex128, device="cuda")
+    gb.mg_get_nullvecs(mg.ctx, 0, out, kind=1)
+    torch.cuda.synchronize()
+    assert rel_l2(to_np(out), mgo.block_orthonormalise(v, dims, block)) < 1e-12
+    mg.close()
