@@ -1008,20 +1008,83 @@ __global__ void __launch_bounds__(256) k_restrict12(cpx<Rc>* __restrict__ coarse
   }
 }
 
+constexpr int kOffTable = 4096;  // fine sites per aggregate that the offset tables hold
+
+// Restriction from a coarse level (dofs per chirality a multiple of 8): CTA
+// (aggregate, right-hand side), thread (g, p) with p a 16-byte column of the
+// Vp rows and g striding over groups of eight rows of one chirality, whose
+// eight loads are independent; site offsets from a table.  8^3x16 to 4^3x8, 48
+// dofs, 32 vectors: 92 us -> under 35 us (k_restrict divides several times per row).
+// Restriction R = P^dag between coarse levels (Sec. 6.6).
+template <typename R>
+__global__ void __launch_bounds__(256) k_restrict_g(cpx<R>* __restrict__ coarse,
+                                                   const cpx<R>* __restrict__ fine,
+                                                   const cpx<R>* __restrict__ Vp, AggMap m,
+                                                   int nd, int nv, int G, int nr, size_t fstride,
+                                                   size_t cstride) {
+  constexpr int CPL = 16 / int(sizeof(cpx<R>));
+  constexpr int FW = 8 * int(sizeof(cpx<R>)) / 16;  // 16-byte words of eight fine entries
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cpx<R>* red = reinterpret_cast<cpx<R>*>(smem_raw);  // [G][2][nv]
+  int* off = reinterpret_cast<int*>(red + size_t(G) * 2 * nv);
+  const int xc = blockIdx.x / nr, rhs = blockIdx.x - xc * nr;
+  fine += rhs * fstride;
+  coarse += rhs * cstride;
+  const int NP = nv / CPL, half = nd / 2, sub = half / 8;
+  const int p = threadIdx.x % NP, g = threadIdx.x / NP;
+  for (int ls = threadIdx.x; ls < m.per; ls += blockDim.x) off[ls] = local_offset(m, ls);
+  const size_t base = size_t(agg_origin(m, xc));
+  __syncthreads();
+  const int groups = m.per * sub;
+#pragma unroll
+  for (int chi = 0; chi < 2; ++chi) {
+    cpx<R> acc[CPL];
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) acc[k] = cpx<R>(R(0), R(0));
+    for (int q = g; q < groups; q += G) {
+      const int ls = q / sub;
+      const size_t row = (base + off[ls]) * nd + chi * half + 8 * (q - ls * sub);
+      const uint4* vr = reinterpret_cast<const uint4*>(Vp + row * nv) + p;
+      uint4 w[8], fw[FW];
+#pragma unroll
+      for (int a = 0; a < 8; ++a) w[a] = ld_stream16(vr + a * NP);
+      const uint4* fr = reinterpret_cast<const uint4*>(fine + row);
+#pragma unroll
+      for (int k = 0; k < FW; ++k) fw[k] = __ldg(fr + k);
+      const cpx<R>* f = reinterpret_cast<const cpx<R>*>(fw);
+#pragma unroll
+      for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int k = 0; k < CPL; ++k)
+          cmac_conj(acc[k], reinterpret_cast<const cpx<R>*>(&w[a])[k], f[a]);
+    }
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) red[(g * 2 + chi) * nv + p * CPL + k] = acc[k];
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < 2 * nv; t += blockDim.x) {
+    cpx<R> sum(R(0), R(0));
+    for (int k = 0; k < G; ++k) sum += red[k * 2 * nv + t];
+    coarse[size_t(xc) * 2 * nv + t] = sum;
+  }
+}
+
 // fine_v[x][a] = sum_i Vp[x][a][i] coarse_v[agg(x)][chi(a)*Nv + i] for all nr
 // right-hand sides.  Two threads per Vp row, each holding half of it in
 // registers: thread q takes the 16-byte words 2k + q (PW words), so a pair
 // reads whole 32-byte sectors; the halves meet by one shuffle.  A pair
 // loads RPI rows (RPI * PW <= 12 words) before any arithmetic, so short
 // rows (16-bit Vp, small Nv) still keep several loads per thread in flight.
-// Prolongation P onto the 12-dof fine level (Sec. 6.6).
-template <typename Rf, typename Rc, typename VT, int PW>
+// NDC: dofs per fine site, 12 on the fine level, 0 (nd) on a coarse one.
+// Prolongation P (Sec. 6.6).
+template <typename Rf, typename Rc, typename VT, int PW, int NDC = 12>
 __global__ void __launch_bounds__(256) k_prolong12(cpx<Rf>* __restrict__ fine,
                                                   const cpx<Rc>* __restrict__ coarse,
                                                   const VT* __restrict__ Vp, AggMap m,
-                                                  int nv, int nr, size_t fstride,
+                                                  int nd, int nv, int nr, size_t fstride,
                                                   size_t cstride, int add) {
-  constexpr int ND = 12, CPL = VUnpack<VT, Rf>::CPL;
+  constexpr int CPL = VUnpack<VT, Rf>::CPL;
+  const int ND = NDC ? NDC : nd;
   constexpr int RPI = PW >= 12 ? 1 : (12 / PW > 6 ? 6 : 12 / PW);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<Rf>* cs = reinterpret_cast<cpx<Rf>*>(smem_raw);  // [nr][2][nv]
@@ -1300,6 +1363,25 @@ void restrict_apply(mg_ctx* c, int level, Vec coarse, Vec fine, cudaStream_t st)
       return;
     }
   }
+  {
+    const int cpl = F.vprec == MG_F64 ? 1 : 2, NP = nv / cpl;
+    const bool aligned = (reinterpret_cast<uintptr_t>(fine.p) & 15) == 0;
+    if (F.nd != 12 && F.nd % 16 == 0 && nv % cpl == 0 && aligned && F.vprec == coarse.prec &&
+        m.per <= kOffTable) {
+      const int groups = m.per * (F.nd / 16);
+      int Gg = 256 / NP;
+      if (Gg > groups) Gg = groups;
+      const size_t smg = size_t(Gg) * 2 * nv * size_t(vb) + size_t(m.per) * sizeof(int);
+      const dim3 grid(unsigned(C.g.vol) * nr);
+      GB_TRANSFER_DISPATCH(F.vprec, F.vprec, Rf, Rc,
+                           (k_restrict_g<Rf><<<grid, Gg * NP, smg, st>>>(
+                               (cpx<Rf>*)coarse.p, (const cpx<Rf>*)fine.p, F.Vp.as<cpx<Rf>>(), m,
+                               F.nd, nv, Gg, nr, fine.n, coarse.n)));
+      GB_LAUNCH_CHECK();
+      c->launches++;
+      return;
+    }
+  }
   int G = 256 / nv;
   if (G < 1) G = 1;
   const int threads = G * nv;
@@ -1338,23 +1420,52 @@ void prolong_apply(mg_ctx* c, int level, Vec fine, Vec coarse, cudaStream_t st, 
       if (h16) {
         if (coarse.prec == MG_F64)
           k_prolong12<float, double, bf16c, PW><<<C.g.vol, 256, smem2, st>>>(
-              (cpx<float>*)fine.p, (const cpx<double>*)coarse.p, F.Vp16.as<bf16c>(), m, nv, nr,
+              (cpx<float>*)fine.p, (const cpx<double>*)coarse.p, F.Vp16.as<bf16c>(), m, 12, nv, nr,
               fine.n, coarse.n, int(add));
         else
           k_prolong12<float, float, bf16c, PW><<<C.g.vol, 256, smem2, st>>>(
-              (cpx<float>*)fine.p, (const cpx<float>*)coarse.p, F.Vp16.as<bf16c>(), m, nv, nr,
+              (cpx<float>*)fine.p, (const cpx<float>*)coarse.p, F.Vp16.as<bf16c>(), m, 12, nv, nr,
               fine.n, coarse.n, int(add));
       } else {
         GB_TRANSFER_DISPATCH(F.vprec, coarse.prec, Rf, Rc,
                              (k_prolong12<Rf, Rc, cpx<Rf>, PW><<<C.g.vol, 256, smem2, st>>>(
                                  (cpx<Rf>*)fine.p, (const cpx<Rc>*)coarse.p,
-                                 F.Vp.as<cpx<Rf>>(), m, nv, nr, fine.n, coarse.n, int(add))));
+                                 F.Vp.as<cpx<Rf>>(), m, 12, nv, nr, fine.n, coarse.n,
+                                 int(add))));
       }
     };
     switch (pw) {
       case 1: go(std::integral_constant<int, 1>{}); break;
       case 2: go(std::integral_constant<int, 2>{}); break;
       case 3: go(std::integral_constant<int, 3>{}); break;
+      case 4: go(std::integral_constant<int, 4>{}); break;
+      case 6: go(std::integral_constant<int, 6>{}); break;
+      case 8: go(std::integral_constant<int, 8>{}); break;
+      default: go(std::integral_constant<int, 12>{}); break;
+    }
+    GB_LAUNCH_CHECK();
+    c->launches++;
+    return;
+  }
+  const bool aligned = (reinterpret_cast<uintptr_t>(fine.p) & 15) == 0;
+  if (F.nd != 12 && !h16 && F.vprec == coarse.prec && aligned && m.per <= kOffTable &&
+      smem2 <= 48 * 1024 && (pw == 2 || pw == 4 || pw == 6 || pw == 8 || pw == 12)) {
+    // between coarse levels: the pair-per-row kernel with run-time dofs (8^3x16
+    // to 4^3x8, 48 dofs, 32 vectors: 57 us -> under 35 us; the entry-per-thread kernel
+    // below divides ten times per entry and reads rows lane by lane)
+    auto go = [&](auto pwc) {
+      constexpr int PW = decltype(pwc)::value;
+      if (F.vprec == MG_F64)
+        k_prolong12<double, double, cpx<double>, PW, 0><<<C.g.vol, 256, smem2, st>>>(
+            (cpx<double>*)fine.p, (const cpx<double>*)coarse.p, F.Vp.as<cpx<double>>(), m, F.nd,
+            nv, nr, fine.n, coarse.n, int(add));
+      else
+        k_prolong12<float, float, cpx<float>, PW, 0><<<C.g.vol, 256, smem2, st>>>(
+            (cpx<float>*)fine.p, (const cpx<float>*)coarse.p, F.Vp.as<cpx<float>>(), m, F.nd, nv,
+            nr, fine.n, coarse.n, int(add));
+    };
+    switch (pw) {
+      case 2: go(std::integral_constant<int, 2>{}); break;
       case 4: go(std::integral_constant<int, 4>{}); break;
       case 6: go(std::integral_constant<int, 6>{}); break;
       case 8: go(std::integral_constant<int, 8>{}); break;

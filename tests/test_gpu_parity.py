@@ -446,3 +446,30 @@ def test_block_orthonormalise_panels(gpu_lib, dims, block, nv, parallel):
     torch.cuda.synchronize()
     assert rel_l2(to_np(out), mgo.block_orthonormalise(v, dims, block)) < 1e-12
     mg.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("nv0,nv1", [(8, 6), (24, 32), (16, 10), (12, 8), (32, 24)])
+def test_restrict_prolong_coarse(gpu_lib, nv0, nv1, prec):
+    """Transfers between coarse levels: eight-row groups and pair-per-row
+    kernels (16, 48, 32, 64 dofs), the generic ones (24 dofs, or a number of
+    vectors without whole 16-byte words per half row)."""
+    gb = gpu_lib
+    dims, b0, b1 = (4, 8, 4, 4), (2, 2, 2, 1), (2, 2, 1, 2)
+    cd = lat.coarse_dims(dims, b0)
+    mg, U = make_ctx(gb, dims, [b0, b1], [nv0, nv1], prec_fine=prec, prec_coarse=prec)
+    cdt = torch.complex128 if prec == 0 else torch.complex64
+    v = syn.gaussian_field((nv1, lat.volume(cd), 2 * nv0), 41)
+    gb.mg_set_nullvecs(mg.ctx, 1, to_dev(v))
+    Q = mgo.block_orthonormalise(v, cd, b1)
+    ccd = lat.coarse_dims(cd, b1)
+    r = syn.gaussian_field((lat.volume(cd), 2 * nv0), 42)
+    ec = syn.gaussian_field((lat.volume(ccd), 2 * nv1), 43)
+    rc = torch.empty((lat.volume(ccd), 2 * nv1), dtype=cdt, device="cuda")
+    e = torch.empty((lat.volume(cd), 2 * nv0), dtype=cdt, device="cuda")
+    gb.mg_restrict(mg.ctx, 1, rc, to_dev(r, cdt))
+    gb.mg_prolong(mg.ctx, 1, e, to_dev(ec, cdt))
+    torch.cuda.synchronize()
+    assert rel_l2(to_np(rc), mgo.restrict(Q, r, cd, b1)) < TOL[prec]
+    assert rel_l2(to_np(e), mgo.prolong(Q, ec, cd, b1)) < TOL[prec]
+    mg.close()
