@@ -1036,6 +1036,23 @@ void blas_dot2(mg_ctx* c, Vec p, Vec r, int s_pr, int s_pp, int s_a, double omeg
   c->launches += 2;
 }
 
+double2* reduction_parts(mg_ctx* c, size_t count) { return partials(c, count); }
+
+void blas_dot2_finish(mg_ctx* c, int nparts, int nr, int s_pr, int s_pp, int s_a, double omega,
+                      cudaStream_t st) {
+  k_reduce_final_pair<<<nr, 256, 0, st>>>(c->red_partials.as<double2>(), nparts, srow(c, s_pr),
+                                          srow(c, s_pp), srow(c, s_a), omega);
+  GB_LAUNCH_CHECK();
+  c->launches++;
+}
+
+void blas_dot2_batched_finish(mg_ctx* c, int nparts, int nvec, cudaStream_t st) {
+  k_reduce_final_b<<<2 * nvec, 256, 0, st>>>(c->red_partials.as<double2>(), nparts,
+                                             c->batch_scalars.as<double2>());
+  GB_LAUNCH_CHECK();
+  c->launches++;
+}
+
 void blas_mr_update(mg_ctx* c, Vec x, Vec r, Vec p, int s_a, cudaStream_t st, bool first,
                     bool last, const void* rin) {
   check_nr(x);

@@ -40,6 +40,13 @@ void blas_norm2(mg_ctx* c, Vec a, int slot, cudaStream_t st, bool fp64_partials 
 // coefficient S[s_a][v] = omega S[s_pr][v] / S[s_pp][v].re (0 if that is 0)
 void blas_dot2(mg_ctx* c, Vec p, Vec r, int s_pr, int s_pp, int s_a, double omega,
                cudaStream_t st);
+// the end of blas_dot2 (blas_dot2_batched) for partial sums an operator kernel
+// left in the reduction buffer, [vector][2][nparts]
+void blas_dot2_finish(mg_ctx* c, int nparts, int nr, int s_pr, int s_pp, int s_a, double omega,
+                      cudaStream_t st);
+void blas_dot2_batched_finish(mg_ctx* c, int nparts, int nvec, cudaStream_t st);
+// the reduction buffer, at least count entries
+double2* reduction_parts(mg_ctx* c, size_t count);
 // MR step per vector: a = S[s_a] ; x += a r ; r -= a p.
 // first: x is taken as zero (not read); last: r is not updated.  rin: where the
 // residual is read from (null: r itself; FP32 / FP64 only)
@@ -84,7 +91,10 @@ void clear_status(mg_ctx* c, cudaStream_t st);
 // Build the fine operator of level 0 from the external gauge field.
 void fine_operator_build(mg_ctx* c, const void* gauge_ext, cudaStream_t st);
 // out = M in on `nvec` vectors (stride vstride complex elements apart)
-void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st);
+// nparts (optional): asks for <out_v, in_v> and |out_v|^2 too; receives the
+// number of partial sums left for blas_dot2_finish / blas_dot2_batched_finish,
+// 0 where the launch policy does not form them
+void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st, int* nparts = nullptr);
 
 // ---------------------------------------------------------------- coarse.cu
 // nrhs > 1: vectors interleaved [site][n][nrhs] (the public layout)

@@ -154,8 +154,16 @@ void mr_smooth(mg_ctx* c, int l, Vec x, Vec b, cudaStream_t st, const Vec* res =
   Vec p = vbuf(w.mrp, L.vprec, L.vec_elems(), x.nr);
   for (int k = 0; k < nit; ++k) {
     const Vec& rk = k == 0 ? b : r;
-    level_apply(c, l, p, rk, st);
-    blas_dot2(c, p, rk, slot(l, S_PR), slot(l, S_PP), slot(l, S_MR), c->p.mr_omega, st);
+    int nparts = 0;  // the fine operator may leave the inner products' partial sums
+    if (l == 0)
+      wilson_apply(c, p, rk, p.nr, st, &nparts);
+    else
+      level_apply(c, l, p, rk, st);
+    if (nparts)
+      blas_dot2_finish(c, nparts, p.nr, slot(l, S_PR), slot(l, S_PP), slot(l, S_MR),
+                       c->p.mr_omega, st);
+    else
+      blas_dot2(c, p, rk, slot(l, S_PR), slot(l, S_PP), slot(l, S_MR), c->p.mr_omega, st);
     blas_mr_update(c, x, r, p, slot(l, S_MR), st, k == 0 && !add,
                    k == nit - 1 && !res, rk.p);
   }
@@ -436,9 +444,9 @@ void setup_sweeps(mg_ctx* c, int l, const void* init, cudaStream_t st) {
   // with the FP32 multi-RHS stream for FP32 stores
   // (interleaved copies in the two halves of raw, free until the end)
   const bool mrhs = l > 0 && !f64 && coarse_apply_multi_fast(L, nv);
-  auto apply_all = [&](Vec out, Vec in) {
+  auto apply_all = [&](Vec out, Vec in, int* nparts = nullptr) {
     if (l == 0) {
-      wilson_apply(c, out, in, nv, st);
+      wilson_apply(c, out, in, nv, st, nparts);
     } else if (mrhs) {
       Vec vi = at(L.raw, 0, n), vo = at(L.raw, bytes, n);
       blas_transpose(c, vi, in, nv, true, st);
@@ -454,8 +462,12 @@ void setup_sweeps(mg_ctx* c, int l, const void* init, cudaStream_t st) {
   //   t = A x,  q = A t,  x <- x - (<q, t> / <q, q>) t
   for (int k = 0; k < c->p.setup_sweeps; ++k) {
     apply_all(T, X);
-    apply_all(Q, T);
-    blas_dot2_batched(c, Q, T, nv, st);
+    int nparts = 0;
+    apply_all(Q, T, &nparts);
+    if (nparts)
+      blas_dot2_batched_finish(c, nparts, nv, st);
+    else
+      blas_dot2_batched(c, Q, T, nv, st);
     blas_sweep_update_batched(c, X, T, nv, st);
   }
   blas_normalise_batched(c, X, nv, st);

@@ -650,12 +650,18 @@ struct WilsonBlock {
 // latency (issue slots 37-50 % busy with 6-10 warps per SM; two threads per
 // site doubled the warps and gained nothing).
 // MINB: resident CTAs per SM that the register budget allows; MULTI: several
-// vectors per launch.
-template <int BX, int BY, int BZ, int BT, int MINB, bool MULTI>
+// vectors per launch; DOT: also the inner products <out, in> and |out|^2 that
+// an MR step needs, as partial sums [vector][2][part] (one part per warp of a
+// CTA, and per block with several vectors; per-block sums in FP32, FP64 across
+// blocks): the pass that reads both vectors again goes.  32^3x64, one vector:
+// 70 us of reading for 15 us here; 24 vectors of 16^3x32: 101 us for
+// 44 us.
+template <int BX, int BY, int BZ, int BT, int MINB, bool MULTI, bool DOT>
 __global__ void __launch_bounds__(BX * BY * BZ * BT, MINB)
     k_wilson_blk(cpx<float>* __restrict__ out, const float4* __restrict__ A, Geom g, float diag,
                  size_t vstride, int nvec, int antiperiodic, int nblocks,
-                 const __grid_constant__ WilsonTileMaps maps, int* __restrict__ err) {
+                 const __grid_constant__ WilsonTileMaps maps, int* __restrict__ err,
+                 double2* __restrict__ part) {
   using WB = WilsonBlock<BX, BY, BZ, BT>;
   constexpr int NS = WB::NS;
   extern __shared__ __align__(128) unsigned char wsm[];
@@ -729,6 +735,9 @@ __global__ void __launch_bounds__(BX * BY * BZ * BT, MINB)
     ioff = 96u * uint32_t(WB::face_sp_rt(imu, iside));
   }
   int it = 0;  // tiles issued and consumed so far: tile `it` in buffer it & 1 (MULTI) or 0
+  constexpr int NW = NS / 32;
+  double2 spr = make_double2(0.0, 0.0);  // DOT: sums over this CTA's blocks
+  double spp = 0.0;
   for (int blk = blockIdx.x; blk < nblocks; blk += gridDim.x) {
     // block origin and valid extents
     int o[4], be[4];
@@ -864,9 +873,45 @@ __global__ void __launch_bounds__(BX * BY * BZ * BT, MINB)
           reinterpret_cast<uint4*>(op + h1)[i] = reinterpret_cast<const uint4*>(ay)[i];
         }
       }
+      if constexpr (DOT) {
+        load_spinor(st, q[0]);
+        cpx<float> pr(0.f, 0.f);
+        float pp = 0.f;
+        if (valid) {
+#pragma unroll
+          for (int i = 0; i < 6; ++i) {
+            cmac_conj(pr, ax[i], reinterpret_cast<const cpx<float>*>(q[0].x)[i]);
+            cmac_conj(pr, ay[i], reinterpret_cast<const cpx<float>*>(q[0].y)[i]);
+            pp = fmaf(ax[i].re, ax[i].re, fmaf(ax[i].im, ax[i].im, pp));
+            pp = fmaf(ay[i].re, ay[i].re, fmaf(ay[i].im, ay[i].im, pp));
+          }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          pr.re += __shfl_xor_sync(0xffffffffu, pr.re, o);
+          pr.im += __shfl_xor_sync(0xffffffffu, pr.im, o);
+          pp += __shfl_xor_sync(0xffffffffu, pp, o);
+        }
+        if (MULTI) {
+          if (lane == 0) {
+            const size_t np = size_t(nblocks) * NW, at = size_t(blk) * NW + (tid >> 5);
+            part[size_t(2 * v) * np + at] = make_double2(double(pr.re), double(pr.im));
+            part[size_t(2 * v + 1) * np + at] = make_double2(double(pp), 0.0);
+          }
+        } else if (lane == 0) {
+          spr.x += double(pr.re);
+          spr.y += double(pr.im);
+          spp += double(pp);
+        }
+      }
       // every thread is done with the tile before the copies of another one
       __syncthreads();
     }
+  }
+  if (DOT && !MULTI && lane == 0) {
+    const size_t np = size_t(gridDim.x) * NW, at = size_t(blockIdx.x) * NW + (tid >> 5);
+    part[at] = spr;
+    part[np + at] = make_double2(spp, 0.0);
   }
 }
 
@@ -881,9 +926,11 @@ int resident_ctas(K kern, int threads, size_t smem) {
 }
 
 // Host side of k_wilson_blk: the ten tensor maps (spinors of `in` over
-// nvec vectors stored back to back, two-row links) and the launch.
+// nvec vectors stored back to back, two-row links) and the launch.  nparts
+// (not null): with inner products; receives the parts per sum, left in the
+// reduction buffer.
 template <int BX, int BY, int BZ, int BT, int MINB, int MINM>
-void launch_wilson_blk(cpx<float>* out, const cpx<float>* in, const cpx<float>* U12,
+void launch_wilson_blk(mg_ctx* c, int* nparts, cpx<float>* out, const cpx<float>* in, const cpx<float>* U12,
                        const float4* A, const Geom& g, float diag, size_t vstride, int nvec,
                        int ap, int* err, cudaStream_t st) {
   using WB = WilsonBlock<BX, BY, BZ, BT>;
@@ -906,8 +953,10 @@ void launch_wilson_blk(cpx<float>* out, const cpx<float>* in, const cpx<float>* 
   }
   // several vectors: shared memory allows few CTAs, so registers are not
   // held down for more
-  auto k = nvec > 1 ? k_wilson_blk<BX, BY, BZ, BT, MINM, true>
-                    : k_wilson_blk<BX, BY, BZ, BT, MINB, false>;
+  auto k = nvec > 1 ? (nparts ? k_wilson_blk<BX, BY, BZ, BT, MINM, true, true>
+                              : k_wilson_blk<BX, BY, BZ, BT, MINM, true, false>)
+                    : (nparts ? k_wilson_blk<BX, BY, BZ, BT, MINB, false, true>
+                              : k_wilson_blk<BX, BY, BZ, BT, MINB, false, false>);
   // several vectors: a second spinor buffer after the links
   const size_t smem =
       size_t(WB::NSP) * 96 * (nvec > 1 ? 2 : 1) + size_t(WB::NLK) * 48;
@@ -917,7 +966,12 @@ void launch_wilson_blk(cpx<float>* out, const cpx<float>* in, const cpx<float>* 
   const int blocks = ceil_div(g.L[0], BX) * ceil_div(g.L[1], BY) * ceil_div(g.L[2], BZ) *
                      ceil_div(g.L[3], BT);
   const int grid = nvec > 1 ? blocks : std::min(blocks, resident_ctas(k, WB::NS, smem));
-  k<<<grid, WB::NS, smem, st>>>(out, A, g, diag, vstride, nvec, ap, blocks, m, err);
+  double2* part = nullptr;
+  if (nparts) {
+    *nparts = grid * (WB::NS / 32);
+    part = reduction_parts(c, size_t(*nparts) * 2 * nvec);
+  }
+  k<<<grid, WB::NS, smem, st>>>(out, A, g, diag, vstride, nvec, ap, blocks, m, err, part);
 }
 
 // the tiled form needs extents of at least a block and 16-byte aligned operands
@@ -997,7 +1051,8 @@ void fine_operator_build(mg_ctx* c, const void* gauge_ext, cudaStream_t st) {
   L.diag = 4.0 + c->p.mass;
 }
 
-void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st) {
+void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st, int* nparts) {
+  if (nparts) *nparts = 0;
   Level& L = c->L[0];
   GB_REQUIRE(out.prec == in.prec, MG_ERR_ARG, "wilson_apply: precision mismatch");
   GB_REQUIRE(out.p != in.p, MG_ERR_ARG, "wilson_apply: output aliases input");
@@ -1037,6 +1092,7 @@ void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st) {
     const float dg = float(L.diag);
     const unsigned gt = ceil_div(L.g.vol, 32);
     int* err = c->status.as<int>() + 1;
+    int* np = nullptr;  // (the autotuner times the plain launches)
     auto launch = [&](int q) {
       switch (q) {
         case 1: k_wilson<float, 12, 0><<<grid, 128, 0, st>>>(o, i, U12, Ac, L.g, dg, vs, nvec, ap); break;
@@ -1050,10 +1106,10 @@ void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st) {
         case 9: k_wilson_tile<true><<<gt, 128, 0, st>>>(o, i, U12, A, L.g, dg, vs, nvec, ap); break;
         case 10: k_wilson<float, 8, 0><<<grid, 128, 0, st>>>(o, i, U8, Ac, L.g, dg, vs, nvec, ap); break;
         case 11: k_wilson<float, 8, 4><<<grid, 128, 0, st>>>(o, i, U8, Ac, L.g, dg, vs, nvec, ap); break;
-        case 12: launch_wilson_blk<4, 4, 4, 2, 3, 2>(o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
-        case 13: launch_wilson_blk<4, 4, 2, 2, 6, 3>(o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
-        case 14: launch_wilson_blk<8, 2, 2, 2, 6, 3>(o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
-        case 15: launch_wilson_blk<8, 4, 2, 2, 3, 2>(o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
+        case 12: launch_wilson_blk<4, 4, 4, 2, 3, 2>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
+        case 13: launch_wilson_blk<4, 4, 2, 2, 6, 3>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
+        case 14: launch_wilson_blk<8, 2, 2, 2, 6, 3>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
+        case 15: launch_wilson_blk<8, 4, 2, 2, 3, 2>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
         default: k_wilson<float, 18, 0><<<grid, 128, 0, st>>>(o, i, U18, Ac, L.g, dg, vs, nvec, ap); break;
       }
     };
@@ -1073,7 +1129,9 @@ void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st) {
     }
     const std::string key = "wilson/v" + std::to_string(L.g.vol) + "/n" + std::to_string(nvec) +
                             "/c" + std::to_string(int(L.gauge12_ok));
-    launch(Tuner::get().choose(key, cands, st, launch));
+    const int q = Tuner::get().choose(key, cands, st, launch);
+    np = nparts;
+    launch(q);
   } else {
     k_wilson<double, 18, 0><<<grid, 128, 0, st>>>(
         (cpx<double>*)out.p, (const cpx<double>*)in.p, L.gauge64.as<cpx<double>>(),
