@@ -52,6 +52,11 @@ struct TempPool {
   ~TempPool() {
     if (pool) cudaMemPoolDestroy(pool);
   }
+  // the pool and a first block of n bytes, so that no call pays for them
+  void prime(size_t n, cudaStream_t st) {
+    if (n > kKeep) n = kKeep;
+    GB_CHECK(cudaFreeAsync(get(n, st), st));
+  }
   void* get(size_t n, cudaStream_t st) {
     std::call_once(once, [&] {
       cudaMemPoolProps pr = {};

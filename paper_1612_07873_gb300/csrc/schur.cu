@@ -742,6 +742,8 @@ void schur_prepare(mg_ctx* c, int level, cudaStream_t st) {
   if (read_status(c, st) & 2)
     throw Error(MG_ERR_NUMERICAL, "red-black: singular site-local block");
   L.have_schur = true;
+  // the temporary of mg_schur_apply on one vector
+  if (level == 0) c->temps.prime(L.vec_bytes() / 2, st);
 }
 
 void eo_apply(mg_ctx* c, int level, int mode, Vec out, Vec in, const void* xc, int p,
