@@ -122,6 +122,11 @@ __device__ __forceinline__ f32x2 pack2f(float a, float b) {
 __device__ __forceinline__ void unpack2f(f32x2 v, float& a, float& b) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
 }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 // a += b * c in both halves
 __device__ __forceinline__ void fma2(f32x2& a, f32x2 b, f32x2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(a) : "l"(b), "l"(c));

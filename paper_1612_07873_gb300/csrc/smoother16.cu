@@ -4,6 +4,8 @@
 // complex numbers (FP32 exponent range, so the shrinking residuals of late
 // outer iterations need no rescaling); all arithmetic runs in FP32.  The
 // outer FP64 GCR and the rest of the K-cycle are unchanged.
+#include <type_traits>
+
 #include "kernels.cuh"
 #include "tune.cuh"
 #include "wilson_ops.cuh"
@@ -128,6 +130,110 @@ __global__ void __launch_bounds__(128, MINB) k_wilson16(bf16c* __restrict__ out,
   for (int i = 0; i < 3; ++i) dst[i] = reinterpret_cast<const uint4*>(o)[i];
 }
 
+// Eq. (2) on BF16 vectors, two vectors per thread: links and clover are loaded
+// and widened once for both, and the colour products and accumulations run in
+// packed arithmetic (hop_halves2).  The one-vector kernel is bound by the issue
+// of its conversions and FMAs; eight vectors of 16^3x32 went from 84 to 72 us
+// (53 us to move the bytes at the copy rate), of 24^3x48 from 399 to 339 us.
+// 167 registers, three CTAs per SM: two CTAs took 88 us, four (128 registers, 48
+// bytes spilled) 72.  Vector 2 q + 1 of an odd count's last pair does not exist:
+// vector 2 q stands in for it and its result is not stored.
+template <int LC>
+__global__ void __launch_bounds__(128, 3)
+    k_wilson16_pair(bf16c* __restrict__ out, const bf16c* __restrict__ in,
+                    const bf16c* __restrict__ U, const __nv_bfloat16* __restrict__ A, Geom g,
+                    float diag, size_t vstride, int nvec, int antiperiodic) {
+  const int np = (nvec + 1) / 2;
+  const int va = 2 * int(blockIdx.x % np), vb = va + 1 < nvec ? va + 1 : va;
+  const int s = int(blockIdx.x / np) * blockDim.x + threadIdx.x;
+  if (s >= g.vol) return;
+  const bf16c* ina = in + va * vstride;
+  const bf16c* inb = in + vb * vstride;
+  int c[4];
+  site_coords(g, s, c);
+  auto load_spinor = [&](const bf16c* base, int site, cpx<float> psi[12]) {
+    const uint4* q = reinterpret_cast<const uint4*>(base + size_t(site) * 12);
+    uint4 w[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) w[i] = __ldg(q + i);
+#pragma unroll
+    for (int i = 0; i < 12; ++i) psi[i] = ld16(reinterpret_cast<const bf16c*>(w)[i]);
+  };
+  const bool tlast = antiperiodic && c[3] == g.L[3] - 1, tfirst = antiperiodic && c[3] == 0;
+  cpx2 ax[6], ay[6];
+  {
+    cpx<float> pa[12], pb[12];
+    load_spinor(ina, s, pa);
+    load_spinor(inb, s, pb);
+    const uint4* q = reinterpret_cast<const uint4*>(A + size_t(s) * 72);
+    uint4 w[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) w[i] = __ldg(q + i);
+    const __nv_bfloat16* a = reinterpret_cast<const __nv_bfloat16*>(w);
+#pragma unroll
+    for (int chi = 0; chi < 2; ++chi) {
+      float cl[36];
+#pragma unroll
+      for (int i = 0; i < 36; ++i) cl[i] = __bfloat162float(a[36 * chi + i]);
+      cpx<float> ra[6], rb[6];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) ra[i] = rb[i] = cpx<float>(0.f, 0.f);
+      clover_block_accum(cl, diag, pa + 6 * chi, ra);
+      clover_block_accum(cl, diag, pb + 6 * chi, rb);
+#pragma unroll
+      for (int i = 0; i < 6; ++i) (chi ? ay[i] : ax[i]) = pack_pair(ra[i], rb[i]);
+    }
+  }
+  auto hop = [&](auto muc, auto fwdc, int nb, size_t link, bool neg) {
+    cpx<float> u[9], pa[12], pb[12];
+    const unsigned* q = reinterpret_cast<const unsigned*>(U + link * LC);
+#pragma unroll
+    for (int e = 0; e < LC; ++e) {
+      const unsigned wv = __ldg(q + e);
+      u[e] = ld16(*reinterpret_cast<const bf16c*>(&wv));
+    }
+    load_spinor(ina, nb, pa);
+    load_spinor(inb, nb, pb);
+    if constexpr (LC == 6) {
+      const float sg = neg ? -1.f : 1.f;
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        const int b = (r + 1) % 3, cc = (r + 2) % 3;
+        u[6 + r] = sg * conj(u[b] * u[3 + cc] - u[cc] * u[3 + b]);
+      }
+    }
+    hop_halves2<decltype(muc)::value, decltype(fwdc)::value>(u, pa, pa + 6, pb, pb + 6, ax, ay,
+                                                             1.f);
+  };
+  const size_t V = g.vol;
+#define GB_HOP16(MU)                                                                     \
+  hop(std::integral_constant<int, MU>{}, std::true_type{}, neighbour(g, s, c, 1 + 2 * MU), \
+      MU * V + s, MU == 3 && tlast);                                                       \
+  {                                                                                        \
+    const int sb = neighbour(g, s, c, 2 + 2 * MU);                                         \
+    hop(std::integral_constant<int, MU>{}, std::false_type{}, sb, MU * V + sb,             \
+        MU == 3 && tfirst);                                                                \
+  }
+  GB_HOP16(0) GB_HOP16(1) GB_HOP16(2) GB_HOP16(3)
+#undef GB_HOP16
+  bf16c oa[12], ob[12];
+#pragma unroll
+  for (int i = 0; i < 12; ++i) {
+    cpx<float> x, y;
+    unpack_pair(i < 6 ? ax[i] : ay[i - 6], x, y);
+    oa[i] = st16(x);
+    ob[i] = st16(y);
+  }
+  uint4* da = reinterpret_cast<uint4*>(out + va * vstride + size_t(s) * 12);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) da[i] = reinterpret_cast<const uint4*>(oa)[i];
+  if (vb != va) {
+    uint4* db = reinterpret_cast<uint4*>(out + vb * vstride + size_t(s) * 12);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) db[i] = reinterpret_cast<const uint4*>(ob)[i];
+  }
+}
+
 }  // namespace
 
 bool smoother16_enabled(const mg_ctx* c) {
@@ -177,10 +283,15 @@ void wilson16_apply(mg_ctx* c, Vec out, Vec in, cudaStream_t st) {
   const __nv_bfloat16* A = L.clover16.as<__nv_bfloat16>();
   const float dg = float(L.diag);
   const int ap = c->p.t_antiperiodic;
-  // autotuned register budget: minimum CTAs per SM 0 (none), 3, 4 or 6
+  // autotuned register budget: minimum CTAs per SM 0 (none), 3, 4 or 6; several
+  // vectors also two per thread (13).  The tuner decides between them: pairs win
+  // for 2 vectors (24^3x48: 108 -> 94 us) and 8 (399 -> 339), not for 3, whose last
+  // pair is half empty (156 against 171)
+  const int pgrid = ceil_div(L.g.vol, 128) * ((nvec + 1) / 2);
   auto launch = [&](int q) {
     if (L.gauge12_ok) {
       switch (q) {
+        case 13: k_wilson16_pair<6><<<pgrid, 128, 0, st>>>(o, i, U, A, L.g, dg, vs, nvec, ap); break;
         case 3: k_wilson16<6, 3><<<grid, 128, 0, st>>>(o, i, U, A, L.g, dg, vs, nvec, ap); break;
         case 4: k_wilson16<6, 4><<<grid, 128, 0, st>>>(o, i, U, A, L.g, dg, vs, nvec, ap); break;
         case 6: k_wilson16<6, 6><<<grid, 128, 0, st>>>(o, i, U, A, L.g, dg, vs, nvec, ap); break;
@@ -188,6 +299,7 @@ void wilson16_apply(mg_ctx* c, Vec out, Vec in, cudaStream_t st) {
       }
     } else {
       switch (q) {
+        case 13: k_wilson16_pair<9><<<pgrid, 128, 0, st>>>(o, i, U, A, L.g, dg, vs, nvec, ap); break;
         case 3: k_wilson16<9, 3><<<grid, 128, 0, st>>>(o, i, U, A, L.g, dg, vs, nvec, ap); break;
         case 4: k_wilson16<9, 4><<<grid, 128, 0, st>>>(o, i, U, A, L.g, dg, vs, nvec, ap); break;
         case 6: k_wilson16<9, 6><<<grid, 128, 0, st>>>(o, i, U, A, L.g, dg, vs, nvec, ap); break;
@@ -197,7 +309,9 @@ void wilson16_apply(mg_ctx* c, Vec out, Vec in, cudaStream_t st) {
   };
   const std::string key = "wilson16/v" + std::to_string(L.g.vol) + "/n" + std::to_string(nvec) +
                           "/c" + std::to_string(int(L.gauge12_ok));
-  launch(Tuner::get().choose(key, {0, 3, 4, 6}, st, launch));
+  std::vector<int> cands{0, 3, 4, 6};
+  if (nvec > 1) cands.push_back(13);
+  launch(Tuner::get().choose(key, cands, st, launch));
   GB_LAUNCH_CHECK();
   c->launches++;
 }

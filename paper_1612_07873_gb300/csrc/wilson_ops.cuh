@@ -151,6 +151,115 @@ __device__ __forceinline__ void hop_halves(const cpx<R>* __restrict__ U, const c
   }
 }
 
+// One complex quantity of two vectors: both real parts in one register pair,
+// both imaginary parts in another.
+struct cpx2 {
+  f32x2 re, im;
+};
+__device__ __forceinline__ cpx2 pack_pair(cpx<float> a, cpx<float> b) {
+  return cpx2{pack2f(a.re, b.re), pack2f(a.im, b.im)};
+}
+__device__ __forceinline__ void unpack_pair(cpx2 v, cpx<float>& a, cpx<float>& b) {
+  unpack2f(v.re, a.re, b.re);
+  unpack2f(v.im, a.im, b.im);
+}
+
+// hop_halves on two vectors a, b with one link: the projections per vector,
+// the colour multiplication and the accumulation in packed arithmetic (half
+// the issue slots, and none of the register-read stalls of FMAs with three
+// distinct sources).
+template <int MU, bool FWD>
+__device__ __forceinline__ void hop_halves2(const cpx<float>* __restrict__ U,
+                                            const cpx<float> xa[6], const cpx<float> ya[6],
+                                            const cpx<float> xb[6], const cpx<float> yb[6],
+                                            cpx2 ax[6], cpx2 ay[6], float sg) {
+  // projected pairs; n: the negated part that the colour product needs
+  cpx2 h[2][3];
+  f32x2 n[2][3];
+  auto project = [&](const cpx<float>* x, const cpx<float>* y, int k, cpx<float> r[2]) {
+    cpx<float> b[2];
+    Bmul<MU>(y[k], y[3 + k], b[0], b[1]);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      if constexpr (MU == 3) {
+        r[s] = FWD ? x[3 * s + k] - b[s] : x[3 * s + k] + b[s];
+      } else {
+        r[s] = cpx<float>(fmaf(FWD ? -sg : sg, b[s].re, x[3 * s + k].re),
+                          fmaf(FWD ? -sg : sg, b[s].im, x[3 * s + k].im));
+      }
+    }
+  };
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    cpx<float> pa[2], pb[2];
+    project(xa, ya, k, pa);
+    project(xb, yb, k, pb);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      h[s][k] = pack_pair(pa[s], pb[s]);
+      // U h: re -= u.im h.im; U^dag h: im -= u.im h.re
+      n[s][k] = FWD ? pack2f(-pa[s].im, -pb[s].im) : pack2f(-pa[s].re, -pb[s].re);
+    }
+  }
+  const float hv = MU == 3 ? 0.5f : 0.5f * sg;
+  const f32x2 mh = pack2f(-0.5f, -0.5f), hs = pack2f(hv, hv), nh = pack2f(-hv, -hv);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    cpx2 w[2];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const cpx<float> u = FWD ? U[a * 3 + b] : U[b * 3 + a];
+      const f32x2 ur = pack2f(u.re, u.re), ui = pack2f(u.im, u.im);
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        if (b == 0) {
+          w[s].re = mul2(ur, h[s][b].re);
+          w[s].im = mul2(ur, h[s][b].im);
+        } else {
+          fma2(w[s].re, ur, h[s][b].re);
+          fma2(w[s].im, ur, h[s][b].im);
+        }
+        if (FWD) {
+          fma2(w[s].re, ui, n[s][b]);
+          fma2(w[s].im, ui, h[s][b].re);
+        } else {
+          fma2(w[s].re, ui, h[s][b].im);
+          fma2(w[s].im, ui, n[s][b]);
+        }
+      }
+    }
+    // first half -= w / 2; second half +- C_mu w / 2 (fwd +), the sign folded
+    // into hs / nh
+    const f32x2 p = FWD ? hs : nh, m = FWD ? nh : hs;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      fma2(ax[3 * s + a].re, mh, w[s].re);
+      fma2(ax[3 * s + a].im, mh, w[s].im);
+    }
+    if constexpr (MU == 0) {         // C w = (-i w1, -i w0)
+      fma2(ay[a].re, p, w[1].im);
+      fma2(ay[a].im, m, w[1].re);
+      fma2(ay[3 + a].re, p, w[0].im);
+      fma2(ay[3 + a].im, m, w[0].re);
+    } else if constexpr (MU == 1) {  // (w1, -w0)
+      fma2(ay[a].re, p, w[1].re);
+      fma2(ay[a].im, p, w[1].im);
+      fma2(ay[3 + a].re, m, w[0].re);
+      fma2(ay[3 + a].im, m, w[0].im);
+    } else if constexpr (MU == 2) {  // (-i w0, i w1)
+      fma2(ay[a].re, p, w[0].im);
+      fma2(ay[a].im, m, w[0].re);
+      fma2(ay[3 + a].re, m, w[1].im);
+      fma2(ay[3 + a].im, p, w[1].re);
+    } else {                         // (w0, w1)
+      fma2(ay[a].re, p, w[0].re);
+      fma2(ay[a].im, p, w[0].im);
+      fma2(ay[3 + a].re, p, w[1].re);
+      fma2(ay[3 + a].im, p, w[1].im);
+    }
+  }
+}
+
 // Runtime-mu dispatch of hop_accum.
 template <typename R>
 __device__ __forceinline__ void hop_accum_rt(int mu, bool fwd, const cpx<R>* __restrict__ U,

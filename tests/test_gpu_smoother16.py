@@ -55,6 +55,41 @@ def test_bf16_operator(gpu_lib, unitary, policy):
     mg.close()
 
 
+@pytest.mark.parametrize("unitary", [True, False])
+@pytest.mark.parametrize("nr", [2, 3])
+def test_bf16_operator_pairs(gpu_lib, nr, unitary):
+    """Two vectors per thread: the last pair whole and single, a volume that is
+    no multiple of the block.  The output is one BF16 rounding of the exact
+    product of the BF16 inputs with BF16 links and clover (relative L2 about
+    2^-9 each, and the third link row that two rounded ones form), as in the
+    one-vector kernel: within 5e-3 of the oracle, and within two roundings,
+    2^-8, of that kernel's own result; nothing past the last vector written."""
+    gb = gpu_lib
+    dims = (2, 4, 6, 6)
+    vol = lat.volume(dims)
+    U = syn.gauge_field(dims, 0.5, 5) * (1.0 if unitary else 1.05)
+    mg, _ = _ctx(gb, dims, [(2, 2, 2, 2)], [2], U=U)
+    psi = syn.gaussian_field((nr, vol, 12), 111)
+    xin = torch.from_numpy(np.stack([psi.real, psi.imag], -1)).to("cuda", torch.bfloat16)
+    out = torch.full((nr + 1,) + tuple(xin.shape[1:]), 7.0, device="cuda", dtype=torch.bfloat16)
+    one = torch.empty_like(xin)
+    key = f"wilson16/v{vol}/n{nr}/c{int(unitary)}"
+    try:
+        gb.mg_tune_set(key, 0)
+        gb.mg_wilson_clover_apply_bf16(mg.ctx, one, xin, nr)
+        gb.mg_tune_set(key, 13)
+        gb.mg_wilson_clover_apply_bf16(mg.ctx, out, xin, nr)
+        assert gb.mg_tune_get(key) == 13
+    finally:
+        gb.mg_tune_set(key, -1)
+    c = lambda t: (lambda o: o[..., 0] + 1j * o[..., 1])(t.float().cpu().numpy())
+    op = oracle_fine(U, dims)
+    assert rel_l2(c(out[:nr]), np.stack([op.apply(p) for p in psi])) < 5e-3
+    assert rel_l2(c(out[:nr]), c(one)) < 2.0 ** -8
+    assert bool((out[nr] == 7.0).all())
+    mg.close()
+
+
 def test_bf16_smoother_solve(gpu_lib):
     gb = gpu_lib
     dims = (8, 8, 8, 8)
