@@ -18,14 +18,20 @@
 // nothing overflows; the scaled lo keeps what a subnormal hi loses).  Three
 // products hi hi, hi lo, lo hi; the two small ones (scaled by 2048) have an
 // accumulator of their own, the dropped lo lo is 2^-24 of a product.  The
-// accumulators run over at most kUnit x 8 sites (12 steps of K = 16) and are
-// then added to FP32 registers, so the tensor cores' truncating accumulation
-// does not build up.
+// accumulators run over a unit of one or two chunks of eight sites (3 or 6
+// steps of K = 16) and are then added to FP32 registers: the tensor cores
+// truncate when they accumulate, and on the X blocks, whose sums have one
+// sign, that bias grows with the unit.  Relative error of the links against 64
+// bits, 24 vectors (the FP32 pipe's own sums in brackets): units of one chunk
+// 1.6e-7 on 2^4 [2.1e-7] and 4^4 [7.7e-7] aggregates, of two 3.1e-7 and
+// 3.0e-7, of four 3.1e-7 and 6.7e-7.  The time for 24^3x48 in 4^4 aggregates is
+// 5.41, 5.22 and 5.11 ms.  So two chunks where the aggregate has 64 sites or
+// more (FP32 pipe 3.9e-7), one below.
 //
 // What bounds it now: the T warps, on the latency of the P and link gathers
 // (issue 46 %, long-scoreboard stalls; the tensor pipe is 7 % busy).  24^3x48,
-// Nv = 24, 4^4 aggregates: 9.21 -> 5.16 ms for 281 GFLOP; error of the links
-// against 64 bits 7.7e-7 -> 6.7e-7.  Two-row links with two hops loaded
+// Nv = 24, 4^4 aggregates: 9.21 -> 5.22 ms for 281 GFLOP; error of the links
+// against 64 bits 7.7e-7 -> 3.0e-7.  Two-row links with two hops loaded
 // ahead: 5.8 ms (spills).
 // One resident CTA per SM walks the (xc, d) blocks, X blocks first.  Roles:
 // 16 Nv T threads, one column of one of the chunk's 8 sites each (Nv = 24:
@@ -46,7 +52,6 @@ namespace {
 
 constexpr int kCh = 8;         // fine sites per chunk: K = 48 per chirality
 constexpr int kRing = 2;       // operand stages (3: 4 % slower, less L1 left for P)
-constexpr int kUnit = 4;       // chunks per accumulator set
 constexpr int kMaxPer = 512;   // fine sites per aggregate (the site tables)
 constexpr float kLoScale = 2048.f;
 
@@ -187,8 +192,8 @@ __device__ __forceinline__ void t_column_y(const cpx<float>* __restrict__ U,
 template <int NV>
 __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
     k_galerkin_mma(const cpx<float>* __restrict__ U, const float* __restrict__ A, float diag,
-                   const cpx<float>* __restrict__ Vp, GalMap m, cpx<float>* __restrict__ out,
-                   int* __restrict__ err) {
+                   const cpx<float>* __restrict__ Vp, GalMap m, int unit,
+                   cpx<float>* __restrict__ out, int* __restrict__ err) {
   using G = GM<NV>;
   constexpr int N = G::N;
   extern __shared__ __align__(128) unsigned char sm[];
@@ -375,7 +380,7 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
         const int nch = (item_cnt(item_d(it)) + kCh - 1) / kCh;
         for (int c = 0; c < nch && ok; ++c, ++q) {
           const int set = w & 1;
-          const bool first = c % kUnit == 0;
+          const bool first = c % unit == 0;
           if (first && w >= 2 && !mbar_wait(&dempty[set], uint32_t((w >> 1) - 1) & 1u)) ok = false;
           const int sg = q % kRing;
           if (ok && !mbar_wait(&full[sg], uint32_t(q / kRing) & 1u)) ok = false;
@@ -399,7 +404,7 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
               mma_f16(dsmall + chi * N, al, bh, idesc, 1u);
             }
           mma_commit(&empty[sg]);
-          if (c % kUnit == kUnit - 1 || c == nch - 1) {
+          if (c % unit == unit - 1 || c == nch - 1) {
             mma_commit(&dfull[set]);
             ++w;
           }
@@ -420,7 +425,7 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
     bool ok = true;
     for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
       const int d = item_d(it), xc = item_xc(it);
-      const int nun = ((item_cnt(d) + kCh - 1) / kCh + kUnit - 1) / kUnit;
+      const int nun = ((item_cnt(d) + kCh - 1) / kCh + unit - 1) / unit;
       float acc[2 * N];
 #pragma unroll
       for (int i = 0; i < 2 * N; ++i) acc[i] = 0.f;
@@ -488,7 +493,7 @@ void launch_galerkin_mma(const Level& F, const GalMap& m, cpx<float>* out, int* 
   const int items = 9 * m.coarse.vol;
   k<<<items < sms ? items : sms, GM<NV>::THREADS, GM<NV>::SMEM, st>>>(
       F.gauge32.as<cpx<float>>(), F.clover32.as<float>(), float(F.diag), F.Vp.as<cpx<float>>(), m,
-      out, err);
+      m.per >= 64 ? 2 : 1, out, err);
   GB_LAUNCH_CHECK();
 }
 

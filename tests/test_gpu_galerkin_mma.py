@@ -43,3 +43,31 @@ def test_galerkin_tensor_cores(gpu_lib, dims, block, nv, antiperiodic):
     for s in range(9):
         assert np.linalg.norm(got[:, s] - want[:, s]) < 1e-5 * big, s
     mg.close()
+
+
+@pytest.mark.parametrize("dims,block", [
+    ((4, 4, 4, 4), (2, 2, 2, 2)),     # 16 sites: two units of a chunk
+    ((4, 4, 4, 8), (2, 2, 2, 4)),     # 32 sites: four units of a chunk
+    ((4, 4, 4, 8), (2, 4, 2, 4)),     # 64 sites: four units of two chunks
+    ((4, 4, 4, 8), (4, 4, 4, 4)),     # 256 sites: 16 units of two chunks
+])
+def test_galerkin_tensor_cores_accuracy(gpu_lib, dims, block):
+    """FP32 accuracy whatever the aggregate: P rounded to FP32 (2^-24 at most),
+    T a chain of about 20 FP32 operations (rms sqrt(20) 2^-24 / sqrt 3, 2.6
+    x 2^-24), the split operands (2^-23 at most each, dropped term included)
+    and at most six truncating accumulations in a unit (mean half a unit in
+    the last place, 3 x 2^-24): together under 6 x 2^-24 relative L2.  Units
+    of four chunks give 11 x 2^-24."""
+    gb = gpu_lib
+    nv = 24
+    mg, U = make_ctx(gb, dims, [block], [nv], prec_fine=1, prec_coarse=1, eps=0.5)
+    v = syn.gaussian_field((nv, lat.volume(dims), 12), 31)
+    gb.mg_set_nullvecs(mg.ctx, 0, to_dev(v))
+    gb.mg_build_coarse(mg.ctx, 0)
+    out = torch.empty((mg.levels[1]["volume"], 9, 2 * nv, 2 * nv), dtype=torch.complex128,
+                      device="cuda")
+    gb.mg_get_coarse_links(mg.ctx, 1, out)
+    gb.mg_device_status(mg.ctx)
+    want = mgo.galerkin(oracle_fine(U, dims), mgo.block_orthonormalise(v, dims, block), block).blocks
+    assert rel_l2(to_np(out), want) < 6 * 2.0 ** -24
+    mg.close()
