@@ -134,7 +134,10 @@ __global__ void __launch_bounds__(mr_groups(N) * (N / 4), mr_ctas(N, NR))
   static_assert(N % 16 == 0 && K % CG == 0 && NR % 4 == 0 && ITER % U == 0, "tile shape");
   extern __shared__ __align__(16) float xsm[];
   __shared__ int nb[9];
-  const int chunk = blockIdx.x, site = blockIdx.y;
+  // chunk-fastest: a site's chunks run close together and share its links in
+  // L2.  (One grid dimension: sites in gridDim.y would stop at 65535.)
+  const int nchunk = (nrhs + NR - 1) / NR;
+  const int site = int(blockIdx.x) / nchunk, chunk = int(blockIdx.x) - site * nchunk;
   const int tid = threadIdx.x;
   const int rp = tid % TPC, cg = tid / TPC;
   // the first links, in flight while x is gathered
@@ -582,7 +585,7 @@ void launch_stream_mr(const Level& L, void* y, const void* x, int nrhs, bool blo
   constexpr size_t smem = mr_smem(N, NR);
   auto kern = k_coarse_stream_mr<N, NR, U, DB>;
   GB_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-  kern<<<dim3(ceil_div(nrhs, NR), L.g.vol), mr_groups(N) * (N / 4), smem, st>>>(
+  kern<<<unsigned(ceil_div(nrhs, NR)) * unsigned(L.g.vol), mr_groups(N) * (N / 4), smem, st>>>(
       (cpx<float>*)y, (const cpx<float>*)x, L.links.as<uint4>(), L.g, nrhs,
       blocked ? size_t(L.g.vol) * N : 1, blocked ? 1 : size_t(nrhs));
 }
