@@ -18,6 +18,7 @@
 //  * the 9 gathered neighbour spinors sit in shared memory (9n complex).
 // 16-bit links carry one FP32 scale per site (value = scale * stored); the
 // arithmetic accumulates in FP32.
+#include <algorithm>
 #include <type_traits>
 
 #include "coarse_ops.cuh"
@@ -125,28 +126,23 @@ constexpr size_t mr_smem(int n, int nr) {
   return xs > red ? xs : red;
 }
 // Grid: chunk-fastest, so a site's chunks run close together and share its links
-// in L2; sites in y and, beyond what a dimension holds (65535), z.  (Chunks and
-// sites in one dimension cost a division ahead of the first load: 8^3x16, n = 64,
-// 2 right-hand sides 343 -> 368 us.)
-constexpr int kMrGridY = 32768;
-inline dim3 mr_grid(int nchunk, int vol) {
-  return dim3(unsigned(nchunk), unsigned(vol < kMrGridY ? vol : kMrGridY),
-              unsigned(ceil_div(vol, kMrGridY)));
-}
-__device__ __forceinline__ int mr_site() { return int(blockIdx.z * kMrGridY + blockIdx.y); }
+// in L2; sites in y, up to the 65535 that it holds, from site0 on (more sites:
+// more launches).  Chunks and sites in one dimension cost a division ahead of the
+// first load (8^3x16, n = 64, 2 right-hand sides 343 -> 368 us).
+constexpr int kMrGridY = 65535;
 
 // Eq. (3) on NR right-hand sides per link read.
 template <int N, int NR, int U, bool DB>
 __global__ void __launch_bounds__(mr_groups(N) * (N / 4), mr_ctas(N, NR))
     k_coarse_stream_mr(cpx<float>* __restrict__ y, const cpx<float>* __restrict__ x,
-                       const uint4* __restrict__ links, Geom g, int nrhs, size_t rs, size_t ss) {
+                       const uint4* __restrict__ links, Geom g, int site0, int nrhs, size_t rs,
+                       size_t ss) {
   constexpr int TPC = N / 4, CG = mr_groups(N), K = 9 * N, NT = CG * TPC, ITER = K / CG;
   constexpr int XS = mr_stride(NR), NP = NR / 2, RN = mr_row(N);
   static_assert(N % 16 == 0 && K % CG == 0 && NR % 4 == 0 && ITER % U == 0, "tile shape");
   extern __shared__ __align__(16) float xsm[];
   __shared__ int nb[9];
-  const int chunk = blockIdx.x, site = mr_site();
-  if (site >= g.vol) return;
+  const int chunk = blockIdx.x, site = site0 + int(blockIdx.y);
   const int tid = threadIdx.x;
   const int rp = tid % TPC, cg = tid / TPC;
   // the first links, in flight while x is gathered
@@ -271,6 +267,97 @@ __global__ void __launch_bounds__(mr_groups(N) * (N / 4), mr_ctas(N, NR))
 #pragma unroll
     for (int q = 1; q < CG; ++q) sum += red[(q * NR + r) * RN + row];
     y[size_t(r0 + r) * rs + (size_t(site) * N + row) * ss] = sum;
+  }
+}
+
+// The same apply with two rows per thread (one 16-byte chunk of a column) and
+// scalar arithmetic, for counts that NR divides: twice the threads per site and
+// no padded vectors.  On small blocks a site is a few kilobytes of links and the
+// wider kernel above has too few warps to hide their latency: 8^3x16, n = 16,
+// 2 / 12 / 20 right-hand sides 32.7 / 84.2 / 135 us against 36.9 / 94.4 / 152;
+// 5280 sites, n = 32, 2 right-hand sides 62.1 against 67.1; 144 sites, n = 48, 12
+// right-hand sides 16.6 against 18.5.  From n = 48 on a large lattice the other
+// one is ahead (8^3x16, n = 48, 8 right-hand sides 378 against 313 us).
+// UM caps the link loads a thread keeps in flight.
+// Eq. (3) on NR right-hand sides per link read.
+template <int N, int NR, int UM>
+__global__ void __launch_bounds__(8 * (N / 2))
+    k_coarse_stream_mr_2row(cpx<float>* __restrict__ y, const cpx<float>* __restrict__ x,
+                            const cpx<float>* __restrict__ links, Geom g, int site0, size_t rs,
+                            size_t ss) {
+  constexpr int RPC = 2, CG = 8, TPC = N / RPC, K = 9 * N, NT = CG * TPC, ITER = K / CG;
+  constexpr int U = batch_of(ITER, UM);
+  constexpr int XS = K * NR, RED = CG * NR * N;
+  static_assert(K % CG == 0 && NR % 2 == 0 && ITER % U == 0, "tile shape");
+  // neighbour values [k][r]; then the partial sums [cg][r][row]
+  __shared__ __align__(16) cpx<float> buf[XS > RED ? XS : RED];
+  __shared__ int nb[9];
+  const int chunk = blockIdx.x, site = site0 + int(blockIdx.y);
+  const int tid = threadIdx.x;
+  if (tid < 9) {
+    int c[4];
+    site_coords(g, site, c);
+    nb[tid] = neighbour(g, site, c, tid);
+  }
+  __syncthreads();
+  if (ss == 1) {  // back to back: read each vector's neighbour values in order
+    for (int i = tid; i < XS; i += NT) {
+      const int r = i / K, k = i - r * K;
+      const int d = k / N;
+      buf[k * NR + r] = x[size_t(chunk * NR + r) * rs + size_t(nb[d]) * N + (k - d * N)];
+    }
+  } else {
+    for (int i = tid; i < XS; i += NT) {
+      const int k = i / NR, r = i - k * NR;
+      const int d = k / N;
+      buf[i] = x[size_t(chunk * NR + r) * rs + (size_t(nb[d]) * N + (k - d * N)) * ss];
+    }
+  }
+  __syncthreads();
+  const int rp = tid % TPC;
+  const int cg = tid / TPC;
+  cpx<float> acc[NR][RPC];
+#pragma unroll
+  for (int r = 0; r < NR; ++r)
+#pragma unroll
+    for (int q = 0; q < RPC; ++q) acc[r][q] = cpx<float>(0.f, 0.f);
+  const uint4* L = reinterpret_cast<const uint4*>(links) + size_t(site) * K * TPC + rp;
+  for (int it = 0; it < ITER; it += U) {
+    uint4 v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = ld_stream16(L + size_t(cg + (it + u) * CG) * TPC);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      cpx<float> e[RPC];
+      Unpack<cpx<float>>::get(v[u], e);
+      const cpx<float>* xk = buf + (cg + (it + u) * CG) * NR;
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const cpx<float> xv = xk[r];
+#pragma unroll
+        for (int q = 0; q < RPC; ++q) cmac(acc[r][q], e[q], xv);
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < NR; ++r)
+#pragma unroll
+    for (int q = 0; q < RPC; ++q) buf[(cg * NR + r) * N + rp * RPC + q] = acc[r][q];
+  __syncthreads();
+  for (int o = tid; o < N * NR; o += NT) {
+    int row, r;
+    if (ss == 1) {
+      r = o / N;
+      row = o - r * N;
+    } else {
+      row = o / NR;
+      r = o - row * NR;
+    }
+    cpx<float> sum = buf[r * N + row];
+#pragma unroll
+    for (int q = 1; q < CG; ++q) sum += buf[(q * NR + r) * N + row];
+    y[size_t(chunk * NR + r) * rs + (size_t(site) * N + row) * ss] = sum;
   }
 }
 
@@ -592,11 +679,24 @@ template <int N, int NR, int U, bool DB>
 void launch_stream_mr(const Level& L, void* y, const void* x, int nrhs, bool blocked,
                       cudaStream_t st) {
   constexpr size_t smem = mr_smem(N, NR);
-  auto kern = k_coarse_stream_mr<N, NR, U, DB>;
-  GB_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-  kern<<<mr_grid(ceil_div(nrhs, NR), L.g.vol), mr_groups(N) * (N / 4), smem, st>>>(
-      (cpx<float>*)y, (const cpx<float>*)x, L.links.as<uint4>(), L.g, nrhs,
-      blocked ? size_t(L.g.vol) * N : 1, blocked ? 1 : size_t(nrhs));
+  static_assert(smem <= 48 * 1024, "no opt-in to more shared memory per launch");
+  for (int s0 = 0; s0 < L.g.vol; s0 += kMrGridY) {
+    const dim3 grid(ceil_div(nrhs, NR), std::min(kMrGridY, L.g.vol - s0));
+    k_coarse_stream_mr<N, NR, U, DB><<<grid, mr_groups(N) * (N / 4), smem, st>>>(
+        (cpx<float>*)y, (const cpx<float>*)x, L.links.as<uint4>(), L.g, s0, nrhs,
+        blocked ? size_t(L.g.vol) * N : 1, blocked ? 1 : size_t(nrhs));
+  }
+}
+
+template <int N, int NR, int UM>
+void launch_stream_mr_2row(const Level& L, void* y, const void* x, int nrhs, bool blocked,
+                           cudaStream_t st) {
+  for (int s0 = 0; s0 < L.g.vol; s0 += kMrGridY) {
+    const dim3 grid(nrhs / NR, std::min(kMrGridY, L.g.vol - s0));
+    k_coarse_stream_mr_2row<N, NR, UM><<<grid, 4 * N, 0, st>>>(
+        (cpx<float>*)y, (const cpx<float>*)x, L.links.as<cpx<float>>(), L.g, s0,
+        blocked ? size_t(L.g.vol) * N : 1, blocked ? 1 : size_t(nrhs));
+  }
 }
 
 // FP32 links, any nrhs > 1.  The autotuner picks the right-hand sides per
@@ -605,6 +705,9 @@ void launch_stream_mr(const Level& L, void* y, const void* x, int nrhs, bool blo
 //          8 right-hand sides (4 when nrhs is at most 4)
 //   2      4 right-hand sides (nrhs above 4), double-buffered: where the last
 //          chunk of 8 would be half empty, 12 of them for instance
+//   20 .. 22  two rows per thread (even nrhs, n <= 48), 8, 4 or 2 right-hand
+//          sides, whichever divides nrhs (n = 48: not 8, where the others are
+//          far ahead); with 8, batches of up to 4 / 6 / 9 columns
 bool try_stream_mr(const Level& L, void* y, const void* x, int nrhs, bool blocked,
                    cudaStream_t st) {
   auto go = [&](auto nc) {
@@ -612,6 +715,18 @@ bool try_stream_mr(const Level& L, void* y, const void* x, int nrhs, bool blocke
     constexpr int ITER = 9 * N / mr_groups(N);
     constexpr int U3 = batch_of(ITER, 3), U4 = batch_of(ITER, 4), U6 = batch_of(ITER, 6);
     auto launch = [&](int q) {
+      if constexpr (N <= 48) {
+        if (q >= 20) {
+          if constexpr (N <= 32) {
+            if (nrhs % 8 == 0)
+              return q == 22   ? launch_stream_mr_2row<N, 8, 9>(L, y, x, nrhs, blocked, st)
+                     : q == 21 ? launch_stream_mr_2row<N, 8, 6>(L, y, x, nrhs, blocked, st)
+                               : launch_stream_mr_2row<N, 8, 4>(L, y, x, nrhs, blocked, st);
+          }
+          return nrhs % 4 == 0 ? launch_stream_mr_2row<N, 4, 4>(L, y, x, nrhs, blocked, st)
+                               : launch_stream_mr_2row<N, 2, 4>(L, y, x, nrhs, blocked, st);
+        }
+      }
       if (nrhs <= 4) {
         if (q == 9)
           launch_stream_mr<N, 4, U6, false>(L, y, x, nrhs, blocked, st);
@@ -627,6 +742,10 @@ bool try_stream_mr(const Level& L, void* y, const void* x, int nrhs, bool blocke
     };
     std::vector<int> cands{4, 9};
     if (nrhs > 4) cands.push_back(2);
+    if (N <= 32 && nrhs % 8 == 0)
+      cands.insert(cands.end(), {20, 21, 22});
+    else if (N <= 48 && nrhs % 2 == 0 && nrhs % 8 != 0)
+      cands.push_back(20);
     const std::string key = "stream_mr/p" + std::to_string(int(L.prec)) + "/n" +
                             std::to_string(N) + "/v" + std::to_string(L.g.vol) + "/r" +
                             std::to_string(nrhs) + "/b" + std::to_string(int(blocked));
