@@ -455,8 +455,11 @@ mg_status mg_inner_product(mg_ctx* ctx, int level, const void* a, const void* b,
  * 16-bit links, or mg_coarse_apply_multi with ctx first) wait, before any
  * MMA, on an mbarrier that nothing arrives at; the wait gives up after its
  * one-second budget, the launch writes no output, and the next
- * mg_device_status returns MG_ERR_TIMEOUT.  MG_ERR_ARG for another name or
- * count outside 0..1000; count = 0 cancels.                               */
+ * mg_device_status returns MG_ERR_TIMEOUT.  what = "galerkin_mma_wait": the
+ * same for the thread that issues the MMAs of the next `count` tensor-core
+ * Galerkin builds (mg_build_coarse of an FP32 Wilson-clover level with 16 or
+ * 24 vectors); the other roles of the kernel leave with it.  MG_ERR_ARG for
+ * another name or count outside 0..1000; count = 0 cancels.               */
 mg_status mg_inject_fault(mg_ctx* ctx, const char* what, int count);
 
 /* Measured CUDA-core peak of fused multiply-adds on the current device, in

@@ -393,7 +393,8 @@ def mg_inner_product(ctx, level, a, b, fp64=True, stream=None):
 
 
 def mg_inject_fault(ctx, what, count=1):
-    """Host-side fault injection for error-path tests ("coarse_mma_wait")."""
+    """Host-side fault injection for error-path tests ("coarse_mma_wait",
+    "galerkin_mma_wait")."""
     _ok(LIB.mg_inject_fault(ctx, what.encode(), count), ctx)
 
 

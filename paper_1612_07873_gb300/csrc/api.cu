@@ -657,9 +657,10 @@ mg_status mg_inner_product(mg_ctx* c, int level, const void* a, const void* b, m
 mg_status mg_inject_fault(mg_ctx* c, const char* what, int count) {
   return guarded(c, [&] {
     GB_REQUIRE(what && count >= 0 && count <= 1000, MG_ERR_ARG, "inject_fault: bad arguments");
-    GB_REQUIRE(std::string(what) == "coarse_mma_wait", MG_ERR_ARG,
-               "inject_fault: unknown fault (known: coarse_mma_wait)");
-    c->inject_mma_stall = count;
+    const std::string name = what;
+    GB_REQUIRE(name == "coarse_mma_wait" || name == "galerkin_mma_wait", MG_ERR_ARG,
+               "inject_fault: unknown fault (known: coarse_mma_wait, galerkin_mma_wait)");
+    (name == "coarse_mma_wait" ? c->inject_mma_stall : c->inject_galerkin_stall) = count;
   });
 }
 

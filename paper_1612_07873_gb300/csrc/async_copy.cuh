@@ -47,6 +47,31 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   }
   return false;
 }
+// bounded wait of one role of a CTA: gives up when another role has set the
+// CTA's abort flag, and sets the flag and the error word when its own second has
+// passed, so that no role waits for one that has left
+__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity,
+                                              volatile int* abort_flag, int* err) {
+  constexpr uint64_t kBudgetNs = 1000000000ull;
+  if (mbar_try_wait(bar, parity)) return true;  // the common case: no timer read
+  const uint64_t t0 = global_ns();
+  for (uint32_t it = 0;; ++it) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if (*abort_flag) return false;
+    if ((it & 255u) == 255u && global_ns() - t0 > kBudgetNs) {
+      *abort_flag = 1;
+      atomicOr(err, 1);
+      return false;
+    }
+  }
+}
+// the same for a whole warp (all 32 lanes call it), with one answer for its
+// lanes: each polls for itself, and a lane that gave up alone would leave the
+// others waiting for it at the next warp-wide instruction
+__device__ __forceinline__ bool wait_or_abort_warp(uint64_t* bar, uint32_t parity,
+                                                   volatile int* abort_flag, int* err) {
+  return __all_sync(0xffffffffu, wait_or_abort(bar, parity, abort_flag, err));
+}
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }

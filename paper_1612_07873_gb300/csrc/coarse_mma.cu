@@ -317,22 +317,6 @@ __global__ void __launch_bounds__(128) k_coarse_mma(const MmaBatch batch, int nr
 constexpr int kWsThreads = 320;
 constexpr int kWsMaxStages = 8;
 
-__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity,
-                                              volatile int* abort_flag, int* err) {
-  constexpr uint64_t kBudgetNs = 1000000000ull;
-  if (mbar_try_wait(bar, parity)) return true;  // the common case: no timer read
-  const uint64_t t0 = global_ns();
-  for (uint32_t it = 0;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if ((it & 255u) == 255u && global_ns() - t0 > kBudgetNs) {
-      *abort_flag = 1;
-      atomicOr(err, 1);
-      return false;
-    }
-  }
-}
-
 // Shared-memory layout of the pipelined kernel: [A ring][link ring][spinor
 // ring][epilogue rows (split rows only)]; the A ring comes first, so the MMA
 // rows beyond 2 nrhs of its last half slot read up to 256 n bytes past it
@@ -925,12 +909,6 @@ void launch_mma_batch(int* err, const MmaBatch& batch, int nrhs, cudaStream_t st
   launch(Tuner::get().choose(key, cands, st, launch));
 }
 
-int take_injected_stall(mg_ctx* c) {
-  if (c->inject_mma_stall <= 0) return 0;
-  --c->inject_mma_stall;
-  return 1;
-}
-
 MmaLattice lattice_of(const Level& L, void* y, const void* x) {
   MmaLattice m;
   m.links = L.links_mma.as<uint4>();
@@ -948,7 +926,7 @@ void launch_mma(mg_ctx* c, const Level& L, void* y, const void* x, int nrhs, cud
   b.lat[0] = lattice_of(L, y, x);
   b.count = 1;
   b.total = L.g.vol;
-  b.stall = take_injected_stall(c);
+  b.stall = take_fault(c->inject_mma_stall);
   launch_mma_batch<BF16, N>(c->status.as<int>() + 1, b, nrhs, st, true, &c->mma_xc);
 }
 
@@ -1018,7 +996,7 @@ extern "C" mg_status mg_coarse_apply_multi(mg_ctx* const* ctxs, const int* level
       b.total += L.g.vol;
     }
     b.count = count;
-    b.stall = take_injected_stall(ctxs[0]);
+    b.stall = take_fault(ctxs[0]->inject_mma_stall);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int* err = ctxs[0]->status.as<int>() + 1;
     const bool bf16 = prec == MG_BF16;

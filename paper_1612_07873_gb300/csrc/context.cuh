@@ -85,6 +85,13 @@ struct TempBuf {
   ~TempBuf() { cudaFreeAsync(p, st); }
 };
 
+// One of `left` injected faults, if any is left: 1 for the launch to stall.
+inline int take_fault(int& left) {
+  if (left <= 0) return 0;
+  --left;
+  return 1;
+}
+
 // One recorded launch of an instrumented kernel class.
 struct ProfRecord {
   std::string name;
@@ -193,7 +200,8 @@ struct mg_ctx {
   std::string err;
   gbmg::Profiler prof;
   long long launches = 0;
-  int inject_mma_stall = 0;     // fault injection: stalled tensor-core launches to come
+  // fault injection (mg_inject_fault): stalled launches to come
+  int inject_mma_stall = 0, inject_galerkin_stall = 0;
   // tensor-core operand tiles of multi-RHS coarse applies (pre-converted x);
   // grown by appending, earlier buffers kept for graphs captured with them
   std::vector<std::unique_ptr<gbmg::DevBuf>> mma_xc;

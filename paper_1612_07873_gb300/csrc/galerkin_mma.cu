@@ -38,8 +38,10 @@
 // 12 warps), writing the split operands into a ring of kRing stages; one
 // thread issuing the 18 MMAs of a chunk; warps 0.. adding finished units from
 // TMEM (two sets of accumulators in turn) and storing the block.  Every wait
-// is bounded: on a timeout the error word is set, the MMAs in flight are
-// waited for (bounded), TMEM is freed and the CTA leaves.
+// is bounded: the role whose time runs out sets the error word and the CTA's
+// abort flag, which every waiting role reads, whole warps decide together
+// (wait_or_abort_warp), the MMAs in flight are waited for (bounded), TMEM is
+// freed and the CTA leaves.
 #include <cmath>
 
 #include "kernels.cuh"
@@ -193,7 +195,7 @@ template <int NV>
 __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
     k_galerkin_mma(const cpx<float>* __restrict__ U, const float* __restrict__ A, float diag,
                    const cpx<float>* __restrict__ Vp, GalMap m, int unit,
-                   cpx<float>* __restrict__ out, int* __restrict__ err) {
+                   cpx<float>* __restrict__ out, int* __restrict__ err, int stall) {
   using G = GM<NV>;
   constexpr int N = G::N;
   extern __shared__ __align__(128) unsigned char sm[];
@@ -201,7 +203,7 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
   // flags (bit e - 1: hop e leaves); then the sites of the eight faces
   int2* tab = reinterpret_cast<int2*>(sm + size_t(kRing) * G::STAGE);
   unsigned short* face = reinterpret_cast<unsigned short*>(tab + kMaxPer);
-  __shared__ uint64_t full[kRing], empty[kRing], dfull[2], dempty[2], fin;
+  __shared__ uint64_t full[kRing], empty[kRing], dfull[2], dempty[2], fin, stall_bar;
   __shared__ uint32_t tmem_sh;
   __shared__ volatile int abort_sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -219,6 +221,7 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
       mbar_init(&dempty[i], G::ND);
     }
     mbar_init(&fin, 1);
+    mbar_init(&stall_bar, 1);  // the injected stall's barrier; never arrived at
     fence_mbar_init();
     abort_sh = 0;
   }
@@ -253,10 +256,6 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = tmem_sh;
   const int cvol = m.coarse.vol, items = 9 * cvol;
-  auto fail = [&] {
-    if (lane == 0) atomicOr(err, 1);
-    abort_sh = 1;
-  };
   // block d of coarse site xc: items 0..cvol-1 are the X blocks, then the
   // eight face blocks of each site
   auto item_d = [&](int it) { return it < cvol ? 0 : 1 + ((it - cvol) & 7); };
@@ -330,8 +329,8 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
           for (int a = 0; a < 6; ++a) v0[a] = cpx<float>(0.f, 0.f);
         }
         const int sg = q % kRing;
-        if (q >= kRing && !mbar_wait(&empty[sg], uint32_t(q / kRing - 1) & 1u)) {
-          fail();
+        if (q >= kRing &&
+            !wait_or_abort_warp(&empty[sg], uint32_t(q / kRing - 1) & 1u, &abort_sh, err)) {
           ok = false;
           break;
         }
@@ -375,15 +374,17 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
     if (lane == 0) {
       constexpr uint32_t idesc = mma_idesc(128, N, false);
       int q = 0, w = 0;
-      bool ok = true;
+      // (fault injection, host-set: waits for what never comes)
+      bool ok = !stall || wait_or_abort(&stall_bar, 0u, &abort_sh, err);
       for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
         const int nch = (item_cnt(item_d(it)) + kCh - 1) / kCh;
         for (int c = 0; c < nch && ok; ++c, ++q) {
           const int set = w & 1;
           const bool first = c % unit == 0;
-          if (first && w >= 2 && !mbar_wait(&dempty[set], uint32_t((w >> 1) - 1) & 1u)) ok = false;
+          if (first && w >= 2)
+            ok = wait_or_abort(&dempty[set], uint32_t((w >> 1) - 1) & 1u, &abort_sh, err);
           const int sg = q % kRing;
-          if (ok && !mbar_wait(&full[sg], uint32_t(q / kRing) & 1u)) ok = false;
+          ok = ok && wait_or_abort(&full[sg], uint32_t(q / kRing) & 1u, &abort_sh, err);
           if (!ok) break;
           tc_fence_after();
           const uint32_t st = smem_u32(sm + size_t(sg) * G::STAGE);
@@ -410,7 +411,6 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
           }
         }
       }
-      if (!ok) fail();
       // every MMA issued has finished before TMEM and shared memory go
       mma_commit(&fin);
       mbar_wait(&fin, 0u);
@@ -431,8 +431,7 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
       for (int i = 0; i < 2 * N; ++i) acc[i] = 0.f;
       for (int un = 0; un < nun; ++un, ++w) {
         const int set = w & 1;
-        if (!mbar_wait(&dfull[set], uint32_t(w >> 1) & 1u)) {
-          fail();
+        if (!wait_or_abort_warp(&dfull[set], uint32_t(w >> 1) & 1u, &abort_sh, err)) {
           ok = false;
           break;
         }
@@ -482,7 +481,7 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
 }
 
 template <int NV>
-void launch_galerkin_mma(const Level& F, const GalMap& m, cpx<float>* out, int* err,
+void launch_galerkin_mma(mg_ctx* c, const Level& F, const GalMap& m, cpx<float>* out, int* err,
                          cudaStream_t st) {
   auto k = k_galerkin_mma<NV>;
   GB_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -493,7 +492,7 @@ void launch_galerkin_mma(const Level& F, const GalMap& m, cpx<float>* out, int* 
   const int items = 9 * m.coarse.vol;
   k<<<items < sms ? items : sms, GM<NV>::THREADS, GM<NV>::SMEM, st>>>(
       F.gauge32.as<cpx<float>>(), F.clover32.as<float>(), float(F.diag), F.Vp.as<cpx<float>>(), m,
-      m.per >= 64 ? 2 : 1, out, err);
+      m.per >= 64 ? 2 : 1, out, err, take_fault(c->inject_galerkin_stall));
   GB_LAUNCH_CHECK();
 }
 
@@ -516,9 +515,9 @@ bool galerkin_mma(mg_ctx* c, int level, cudaStream_t st) {
   if (m.per > kMaxPer) return false;
   int* err = c->status.as<int>() + 1;
   if (F.nvec == 24)
-    launch_galerkin_mma<24>(F, m, C.links.as<cpx<float>>(), err, st);
+    launch_galerkin_mma<24>(c, F, m, C.links.as<cpx<float>>(), err, st);
   else
-    launch_galerkin_mma<16>(F, m, C.links.as<cpx<float>>(), err, st);
+    launch_galerkin_mma<16>(c, F, m, C.links.as<cpx<float>>(), err, st);
   return true;
 }
 
