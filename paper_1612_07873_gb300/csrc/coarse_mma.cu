@@ -435,13 +435,17 @@ __global__ void __launch_bounds__(kWsThreads, 3)
     const int ntiles = (N / 8) << jsh;  // tiles of a half slot
     const int jl = lane & 7, kl0 = lane >> 3;
     uint32_t q = 0;
-    for (int gs = blockIdx.x; gs < batch.total && !abort_sh; gs += gridDim.x) {
+    bool go = true;
+    for (int gs = blockIdx.x; gs < batch.total && go; gs += gridDim.x) {
       for (int d = 0; d < NST; ++d, ++q) {
         if (int(q & 3u) != warp) continue;
         const uint32_t sl = q % uint32_t(SL), lph = (q / uint32_t(SL)) & 1u;
         const uint32_t sa = q % uint32_t(SA), aph = (q / uint32_t(SA)) & 1u;
-        if (!wait_or_abort(&load_full[sl], lph, &abort_sh, err)) break;
-        if (!wait_or_abort(&a_empty[sa], aph ^ 1u, &abort_sh, err)) break;
+        if (!wait_or_abort_warp(&load_full[sl], lph, &abort_sh, err) ||
+            !wait_or_abort_warp(&a_empty[sa], aph ^ 1u, &abort_sh, err)) {
+          go = false;
+          break;
+        }
         const cpx<float>* __restrict__ xr =
             reinterpret_cast<const cpx<float>*>(rring + size_t(sl) * lay.rb);
         unsigned char* __restrict__ A = aring + size_t(sa) * lay.ab;
@@ -492,7 +496,7 @@ __global__ void __launch_bounds__(kWsThreads, 3)
     uint32_t it = 0;
     for (int gs = blockIdx.x; gs < batch.total; gs += gridDim.x, ++it) {
       const uint32_t b = it & 1u, ph = (it >> 1) & 1u;
-      if (!wait_or_abort(&acc_full[b], ph, &abort_sh, err)) break;
+      if (!wait_or_abort_warp(&acc_full[b], ph, &abort_sh, err)) break;
       tc_fence_after();
       const MmaLattice& cur = batch.lat[lattice_of_site(gs)];
       const int site = gs - cur.site0;
