@@ -478,12 +478,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
     }
     __syncthreads();
     if (!mbar_wait(&vbar, vphase)) {
-      // the copies did not land within the budget: record it, give them a
-      // second bounded wait and leave
-      if (tid == 0) {
-        atomicOr(err, 1);
-        mbar_wait(&vbar, vphase);
-      }
+      // the copies did not land within the budget: record it (any thread: each
+      // has a time of its own; no warp-wide step follows), give them a second
+      // bounded wait and leave
+      atomicOr(err, 1);
+      if (tid == 0) mbar_wait(&vbar, vphase);
       return;
     }
     vphase ^= 1u;
