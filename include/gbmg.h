@@ -458,7 +458,9 @@ mg_status mg_inner_product(mg_ctx* ctx, int level, const void* a, const void* b,
  * mg_device_status returns MG_ERR_TIMEOUT.  what = "galerkin_mma_wait": the
  * same for the thread that issues the MMAs of the next `count` tensor-core
  * Galerkin builds (mg_build_coarse of an FP32 Wilson-clover level with 16 or
- * 24 vectors); the other roles of the kernel leave with it.  MG_ERR_ARG for
+ * 24 vectors); the other roles of the kernel leave with it.  what =
+ * "wilson_tile_wait": the next `count` tiled launches of the FP32 fine
+ * operator (policies 12..15) wait for bytes that never come.  MG_ERR_ARG for
  * another name or count outside 0..1000; count = 0 cancels.               */
 mg_status mg_inject_fault(mg_ctx* ctx, const char* what, int count);
 

@@ -394,7 +394,7 @@ def mg_inner_product(ctx, level, a, b, fp64=True, stream=None):
 
 def mg_inject_fault(ctx, what, count=1):
     """Host-side fault injection for error-path tests ("coarse_mma_wait",
-    "galerkin_mma_wait")."""
+    "galerkin_mma_wait", "wilson_tile_wait")."""
     _ok(LIB.mg_inject_fault(ctx, what.encode(), count), ctx)
 
 

@@ -658,9 +658,14 @@ mg_status mg_inject_fault(mg_ctx* c, const char* what, int count) {
   return guarded(c, [&] {
     GB_REQUIRE(what && count >= 0 && count <= 1000, MG_ERR_ARG, "inject_fault: bad arguments");
     const std::string name = what;
-    GB_REQUIRE(name == "coarse_mma_wait" || name == "galerkin_mma_wait", MG_ERR_ARG,
-               "inject_fault: unknown fault (known: coarse_mma_wait, galerkin_mma_wait)");
-    (name == "coarse_mma_wait" ? c->inject_mma_stall : c->inject_galerkin_stall) = count;
+    int* left = name == "coarse_mma_wait"     ? &c->inject_mma_stall
+                : name == "galerkin_mma_wait" ? &c->inject_galerkin_stall
+                : name == "wilson_tile_wait"  ? &c->inject_tile_stall
+                                              : nullptr;
+    GB_REQUIRE(left, MG_ERR_ARG,
+               "inject_fault: unknown fault (known: coarse_mma_wait, galerkin_mma_wait, "
+               "wilson_tile_wait)");
+    *left = count;
   });
 }
 

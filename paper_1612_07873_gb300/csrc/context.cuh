@@ -201,7 +201,7 @@ struct mg_ctx {
   gbmg::Profiler prof;
   long long launches = 0;
   // fault injection (mg_inject_fault): stalled launches to come
-  int inject_mma_stall = 0, inject_galerkin_stall = 0;
+  int inject_mma_stall = 0, inject_galerkin_stall = 0, inject_tile_stall = 0;
   // tensor-core operand tiles of multi-RHS coarse applies (pre-converted x);
   // grown by appending, earlier buffers kept for graphs captured with them
   std::vector<std::unique_ptr<gbmg::DevBuf>> mma_xc;

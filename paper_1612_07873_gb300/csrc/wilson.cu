@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(BX * BY * BZ * BT, MINB)
     k_wilson_blk(cpx<float>* __restrict__ out, const float4* __restrict__ A, Geom g, float diag,
                  size_t vstride, int nvec, int antiperiodic, int nblocks,
                  const __grid_constant__ WilsonTileMaps maps, int* __restrict__ err,
-                 double2* __restrict__ part) {
+                 double2* __restrict__ part, int stall) {
   using WB = WilsonBlock<BX, BY, BZ, BT>;
   constexpr int NS = WB::NS;
   extern __shared__ __align__(128) unsigned char wsm[];
@@ -770,8 +770,9 @@ __global__ void __launch_bounds__(BX * BY * BZ * BT, MINB)
       uint64_t* b = MULTI && (k & 1) ? &bar[1] : &bar[0];
       if (lane == 0) {
         fence_proxy_async_smem();
-        mbar_arrive_expect_tx(
-            b, uint32_t(WB::NSP) * 96u + (v == 0 ? uint32_t(WB::NLK) * 48u : 0u));
+        // (stall, host-set fault injection: waits for bytes that never come)
+        mbar_arrive_expect_tx(b, uint32_t(WB::NSP) * 96u +
+                                     (v == 0 ? uint32_t(WB::NLK) * 48u : 0u) + (stall ? 16u : 0u));
       }
       __syncwarp();
       if (lane < (v == 0 ? 17 : 9))
@@ -803,12 +804,14 @@ __global__ void __launch_bounds__(BX * BY * BZ * BT, MINB)
       const unsigned char* sp = (it & 1) ? sp1 : sp0;
       uint64_t* wb = MULTI && (it & 1) ? &bar[1] : &bar[0];
       const uint32_t ph = uint32_t(MULTI ? it >> 1 : it) & 1u;
-      if (!mbar_wait(wb, ph)) {
-        // the copies did not land within the budget: record it, give the
+      if (!__all_sync(0xffffffffu, mbar_wait(wb, ph))) {
+        // the copies did not land within the budget of some lane: its warp
+        // records that and leaves as a whole (lanes that left alone would be
+        // waited for at the next warp-wide step); the first warp gives the
         // copies in flight (this tile's and the next one's) a second bounded
-        // wait and leave
+        // wait.  The block barrier does not count warps that have left.
+        if (lane == 0) atomicOr(err, 1);
         if (tid == 0) {
-          atomicOr(err, 1);
           mbar_wait(wb, ph);
           if (MULTI && v + 1 < nvec)
             mbar_wait((it & 1) ? &bar[0] : &bar[1], uint32_t((it + 1) >> 1) & 1u);
@@ -932,7 +935,7 @@ int resident_ctas(K kern, int threads, size_t smem) {
 template <int BX, int BY, int BZ, int BT, int MINB, int MINM>
 void launch_wilson_blk(mg_ctx* c, int* nparts, cpx<float>* out, const cpx<float>* in, const cpx<float>* U12,
                        const float4* A, const Geom& g, float diag, size_t vstride, int nvec,
-                       int ap, int* err, cudaStream_t st) {
+                       int ap, int* err, cudaStream_t st, int stall) {
   using WB = WilsonBlock<BX, BY, BZ, BT>;
   WilsonTileMaps m;
   const cuuint64_t X = g.L[0], Y = g.L[1], Z = g.L[2], T = g.L[3];
@@ -971,7 +974,7 @@ void launch_wilson_blk(mg_ctx* c, int* nparts, cpx<float>* out, const cpx<float>
     *nparts = grid * (WB::NS / 32);
     part = reduction_parts(c, size_t(*nparts) * 2 * nvec);
   }
-  k<<<grid, WB::NS, smem, st>>>(out, A, g, diag, vstride, nvec, ap, blocks, m, err, part);
+  k<<<grid, WB::NS, smem, st>>>(out, A, g, diag, vstride, nvec, ap, blocks, m, err, part, stall);
 }
 
 // the tiled form needs extents of at least a block and 16-byte aligned operands
@@ -1093,6 +1096,7 @@ void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st, int* np
     const unsigned gt = ceil_div(L.g.vol, 32);
     int* err = c->status.as<int>() + 1;
     int* np = nullptr;  // (the autotuner times the plain launches)
+    int stall = 0;      // (fault injection)
     auto launch = [&](int q) {
       switch (q) {
         case 1: k_wilson<float, 12, 0><<<grid, 128, 0, st>>>(o, i, U12, Ac, L.g, dg, vs, nvec, ap); break;
@@ -1106,10 +1110,10 @@ void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st, int* np
         case 9: k_wilson_tile<true><<<gt, 128, 0, st>>>(o, i, U12, A, L.g, dg, vs, nvec, ap); break;
         case 10: k_wilson<float, 8, 0><<<grid, 128, 0, st>>>(o, i, U8, Ac, L.g, dg, vs, nvec, ap); break;
         case 11: k_wilson<float, 8, 4><<<grid, 128, 0, st>>>(o, i, U8, Ac, L.g, dg, vs, nvec, ap); break;
-        case 12: launch_wilson_blk<4, 4, 4, 2, 3, 2>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
-        case 13: launch_wilson_blk<4, 4, 2, 2, 6, 3>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
-        case 14: launch_wilson_blk<8, 2, 2, 2, 6, 3>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
-        case 15: launch_wilson_blk<8, 4, 2, 2, 3, 2>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st); break;
+        case 12: launch_wilson_blk<4, 4, 4, 2, 3, 2>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st, stall); break;
+        case 13: launch_wilson_blk<4, 4, 2, 2, 6, 3>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st, stall); break;
+        case 14: launch_wilson_blk<8, 2, 2, 2, 6, 3>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st, stall); break;
+        case 15: launch_wilson_blk<8, 4, 2, 2, 3, 2>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st, stall); break;
         default: k_wilson<float, 18, 0><<<grid, 128, 0, st>>>(o, i, U18, Ac, L.g, dg, vs, nvec, ap); break;
       }
     };
@@ -1131,6 +1135,7 @@ void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st, int* np
                             "/c" + std::to_string(int(L.gauge12_ok));
     const int q = Tuner::get().choose(key, cands, st, launch);
     np = nparts;
+    if (q >= 12 && q <= 15) stall = take_fault(c->inject_tile_stall);
     launch(q);
   } else {
     k_wilson<double, 18, 0><<<grid, 128, 0, st>>>(
