@@ -1277,7 +1277,7 @@ int read_status(mg_ctx* c, cudaStream_t st) {
 }
 
 void clear_status(mg_ctx* c, cudaStream_t st) {
-  GB_CHECK(cudaMemsetAsync(c->status.p, 0, c->status.bytes, st));
+  GB_CHECK(cudaMemsetAsync(c->status.p, 0, sizeof(int), st));
 }
 
 }  // namespace gbmg

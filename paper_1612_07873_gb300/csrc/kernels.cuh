@@ -84,6 +84,8 @@ void blas_transpose(mg_ctx* c, Vec out, Vec in, int nvec, bool to_interleaved, c
 // complex Gaussian (Re, Im iid N(0,1)) from a counter-based Philox4x32-10
 void blas_gaussian(mg_ctx* c, Vec v, uint64_t seed, uint64_t offset, cudaStream_t st);
 // a device status word check (host reads it; synchronises)
+// (word 0: the rank and singularity tests of one call; word 1, the record of
+// timed-out waits, is mg_device_status's to clear)
 int read_status(mg_ctx* c, cudaStream_t st);
 void clear_status(mg_ctx* c, cudaStream_t st);
 
