@@ -7,6 +7,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
 #include "common.cuh"
 
 namespace gbmg {
@@ -85,6 +87,16 @@ struct TempBuf {
   ~TempBuf() { cudaFreeAsync(p, st); }
 };
 
+// What the tiled launches of the fine operator need besides the vectors, for one
+// block shape: the tensor maps of the links, and per kernel (one vector or
+// several, with inner products or without) its attributes set and its resident
+// CTAs.  Made on first use, by one thread; constant from then on.
+struct TilePlan {
+  std::once_flag links_once, kern_once[4];
+  CUtensorMap links[5];
+  int ctas[4] = {0, 0, 0, 0};
+};
+
 // One of `left` injected faults, if any is left: 1 for the launch to stall.
 inline int take_fault(int& left) {
   if (left <= 0) return 0;
@@ -130,6 +142,7 @@ struct Level {
   // sign folded into the last slice; clover [V][2][36] packed Hermitian.
   DevBuf gauge64, gauge32, clover64, clover32;
   DevBuf clover32t;            // clover32 as [18 words of 16 B][V]
+  TilePlan tile[4];            // tiled launches, by block shape (policy 12 + k)
   // FP32 links compressed to their first two rows [mu][V][6] complex; the
   // third row is rebuilt as conj(row0 x row1) (times the boundary sign),
   // valid when the field is special unitary to FP32 precision (checked at

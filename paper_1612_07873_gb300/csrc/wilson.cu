@@ -928,32 +928,34 @@ int resident_ctas(K kern, int threads, size_t smem) {
   return sms * (per > 0 ? per : 1);
 }
 
-// Host side of k_wilson_blk: the ten tensor maps (spinors of `in` over
-// nvec vectors stored back to back, two-row links) and the launch.  nparts
-// (not null): with inner products; receives the parts per sum, left in the
-// reduction buffer.
+// Host side of k_wilson_blk: the five tensor maps of the vectors (`in`, nvec of
+// them stored back to back; those of the two-row links and the kernel's
+// attributes are the plan's) and the launch.  On small lattices this host work
+// is the call: ten maps, two attributes and the occupancy query on every call
+// made one 6^4 vector 11.7 us (8.0 now; thread per site 8.5).  nparts (not
+// null): with inner products; receives the parts per sum, left in the reduction
+// buffer.
 template <int BX, int BY, int BZ, int BT, int MINB, int MINM>
-void launch_wilson_blk(mg_ctx* c, int* nparts, cpx<float>* out, const cpx<float>* in, const cpx<float>* U12,
-                       const float4* A, const Geom& g, float diag, size_t vstride, int nvec,
-                       int ap, int* err, cudaStream_t st, int stall) {
+void launch_wilson_blk(mg_ctx* c, TilePlan& plan, int* nparts, cpx<float>* out,
+                       const cpx<float>* in, const cpx<float>* U12, const float4* A,
+                       const Geom& g, float diag, size_t vstride, int nvec, int ap, int* err,
+                       cudaStream_t st, int stall) {
   using WB = WilsonBlock<BX, BY, BZ, BT>;
-  WilsonTileMaps m;
   const cuuint64_t X = g.L[0], Y = g.L[1], Z = g.L[2], T = g.L[3];
-  const cuuint64_t sd[5] = {24 * X, Y, Z, T, cuuint64_t(nvec)};
-  const cuuint64_t ss[4] = {96 * X, 96 * X * Y, 96 * X * Y * Z, 96 * X * Y * Z * T};
-  const cuuint64_t ld[5] = {12 * X, Y, Z, T, 4};
-  const cuuint64_t ls[4] = {48 * X, 48 * X * Y, 48 * X * Y * Z, 48 * X * Y * Z * T};
-  const cuuint32_t box[5] = {24 * BX, BY, BZ, BT, 1};
-  const cuuint32_t lbox[5] = {12 * BX, BY, BZ, BT, 1};
-  m.sp[0] = make_map_5d(in, sd, ss, box);
-  m.lk[0] = make_map_5d(U12, ld, ls, lbox);
-  for (int mu = 0; mu < 4; ++mu) {
-    cuuint32_t fb[5] = {24 * BX, BY, BZ, BT, 1}, fl[5] = {12 * BX, BY, BZ, BT, 1};
-    fb[mu] = mu == 0 ? 24 : 1;
-    fl[mu] = mu == 0 ? 12 : 1;
-    m.sp[1 + mu] = make_map_5d(in, sd, ss, fb);
-    m.lk[1 + mu] = make_map_5d(U12, ld, ls, fl);
-  }
+  // maps over records of `w` floats: 0 the block, 1 + mu its face in mu
+  auto make_maps = [&](CUtensorMap m[5], const void* base, cuuint32_t w, cuuint64_t slices) {
+    const cuuint64_t d[5] = {w * X, Y, Z, T, slices}, r = 4 * w;
+    const cuuint64_t s[4] = {r * X, r * X * Y, r * X * Y * Z, r * X * Y * Z * T};
+    for (int k = 0; k < 5; ++k) {
+      cuuint32_t box[5] = {w * BX, BY, BZ, BT, 1};
+      if (k > 0) box[k - 1] = k == 1 ? w : 1;
+      m[k] = make_map_5d(base, d, s, box);
+    }
+  };
+  std::call_once(plan.links_once, [&] { make_maps(plan.links, U12, 12, 4); });
+  WilsonTileMaps m;
+  make_maps(m.sp, in, 24, cuuint64_t(nvec));
+  std::copy(plan.links, plan.links + 5, m.lk);
   // several vectors: shared memory allows few CTAs, so registers are not
   // held down for more
   auto k = nvec > 1 ? (nparts ? k_wilson_blk<BX, BY, BZ, BT, MINM, true, true>
@@ -963,12 +965,16 @@ void launch_wilson_blk(mg_ctx* c, int* nparts, cpx<float>* out, const cpx<float>
   // several vectors: a second spinor buffer after the links
   const size_t smem =
       size_t(WB::NSP) * 96 * (nvec > 1 ? 2 : 1) + size_t(WB::NLK) * 48;
-  GB_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-  GB_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                cudaSharedmemCarveoutMaxShared));
+  const int which = (nvec > 1 ? 2 : 0) + (nparts ? 1 : 0);
+  std::call_once(plan.kern_once[which], [&] {
+    GB_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    GB_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                  cudaSharedmemCarveoutMaxShared));
+    plan.ctas[which] = resident_ctas(k, WB::NS, smem);
+  });
   const int blocks = ceil_div(g.L[0], BX) * ceil_div(g.L[1], BY) * ceil_div(g.L[2], BZ) *
                      ceil_div(g.L[3], BT);
-  const int grid = nvec > 1 ? blocks : std::min(blocks, resident_ctas(k, WB::NS, smem));
+  const int grid = nvec > 1 ? blocks : std::min(blocks, plan.ctas[which]);
   double2* part = nullptr;
   if (nparts) {
     *nparts = grid * (WB::NS / 32);
@@ -1110,10 +1116,10 @@ void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st, int* np
         case 9: k_wilson_tile<true><<<gt, 128, 0, st>>>(o, i, U12, A, L.g, dg, vs, nvec, ap); break;
         case 10: k_wilson<float, 8, 0><<<grid, 128, 0, st>>>(o, i, U8, Ac, L.g, dg, vs, nvec, ap); break;
         case 11: k_wilson<float, 8, 4><<<grid, 128, 0, st>>>(o, i, U8, Ac, L.g, dg, vs, nvec, ap); break;
-        case 12: launch_wilson_blk<4, 4, 4, 2, 3, 2>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st, stall); break;
-        case 13: launch_wilson_blk<4, 4, 2, 2, 6, 3>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st, stall); break;
-        case 14: launch_wilson_blk<8, 2, 2, 2, 6, 3>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st, stall); break;
-        case 15: launch_wilson_blk<8, 4, 2, 2, 3, 2>(c, np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st, stall); break;
+        case 12: launch_wilson_blk<4, 4, 4, 2, 3, 2>(c, L.tile[0], np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st, stall); break;
+        case 13: launch_wilson_blk<4, 4, 2, 2, 6, 3>(c, L.tile[1], np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st, stall); break;
+        case 14: launch_wilson_blk<8, 2, 2, 2, 6, 3>(c, L.tile[2], np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st, stall); break;
+        case 15: launch_wilson_blk<8, 4, 2, 2, 3, 2>(c, L.tile[3], np, o, i, U12, At, L.g, dg, vs, nvec, ap, err, st, stall); break;
         default: k_wilson<float, 18, 0><<<grid, 128, 0, st>>>(o, i, U18, Ac, L.g, dg, vs, nvec, ap); break;
       }
     };
