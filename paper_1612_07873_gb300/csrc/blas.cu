@@ -23,8 +23,10 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 // kernels of <= 64 registers a thread); a second, partly filled wave would
 // leave SMs idle at the end.  nr vectors share the wave (their blocks run side
 // by side; one wave each made blocks of a few loads around two CTA-wide
-// reductions: 8 BF16 vectors of 16^3x32 44 us, 15 us to read them).  The grid
-// depends only on the lengths and the device.
+// reductions: 8 BF16 vectors of 16^3x32 44 us, 15 us to read them).  A thread
+// then sums nr times as many terms; FP32 sums are folded into FP64 often enough
+// (grid_loop_fold) that their length depends on neither.  The grid depends only
+// on the lengths and the device.
 int red_blocks(size_t n, int per_sm = 4, int nr = 1) {
   static const int sms = [] {
     int dev = 0, v = 0;
@@ -91,9 +93,9 @@ __device__ __forceinline__ cpx<T> to_acc(cpx<R> a) {
     return cpx<T>(a);
 }
 
-// Per-thread partial sums run in the arithmetic type T: FP32 when both
-// operands are FP32 (FP64 issue is scarce on GB300), FP64 otherwise; the
-// per-thread partials are combined in FP64.
+// Partial sums run in the arithmetic type T: FP32 when both operands are FP32
+// (FP64 issue is scarce on GB300), in runs of a few terms that are combined in
+// FP64 (grid_loop_fold); FP64 otherwise.
 template <typename Ra, typename Rb>
 using acc_t = typename std::conditional<std::is_same<Ra, float>::value &&
                                             std::is_same<Rb, float>::value,
@@ -120,6 +122,53 @@ __device__ __forceinline__ void grid_loop_acc(size_t n, F&& body) {
   for (; i < n; i += stride) body(i, 0);
 }
 
+// The same loop for FP32 accumulators: fold() moves them to FP64 after every
+// ROUNDS rounds and at the end, so that an accumulator holds ROUNDS rounds'
+// terms and the last three elements at most, whatever the length and the
+// grid.  (One FP32 sum per thread and accumulator lost 1e-5 of the squared norm
+// of 48 vectors of 16^3x32 in the worst case, 128 terms each.)
+constexpr int kFoldRounds = 4;
+template <int ROUNDS, typename F, typename G>
+__device__ __forceinline__ void grid_loop_fold(size_t n, F&& body, G&& fold) {
+  const size_t stride = size_t(gridDim.x) * blockDim.x;
+  size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x;
+  int c = 0;
+  for (; i + (kAcc - 1) * stride < n; i += kAcc * stride) {
+#pragma unroll
+    for (int k = 0; k < kAcc; ++k) body(i + k * stride, k);
+    if (ROUNDS > 0 && ++c == ROUNDS) {
+      fold();
+      c = 0;
+    }
+  }
+  for (; i < n; i += stride) body(i, 0);
+  fold();
+}
+// s += the accumulators, which start again at zero
+template <typename T>
+__device__ __forceinline__ void fold_acc(double& s, T (&a)[kAcc]) {
+  const T t = (a[0] + a[1]) + (a[2] + a[3]);
+  if constexpr (std::is_same<T, float>::value)
+    s += f2d(t);
+  else
+    s += t;
+#pragma unroll
+  for (int k = 0; k < kAcc; ++k) a[k] = T(0);
+}
+template <typename T>
+__device__ __forceinline__ void fold_acc(double2& s, cpx<T> (&a)[kAcc]) {
+  const cpx<double> t = to_acc<double>((a[0] + a[1]) + (a[2] + a[3]));
+  s.x += t.re;
+  s.y += t.im;
+#pragma unroll
+  for (int k = 0; k < kAcc; ++k) a[k] = cpx<T>(T(0), T(0));
+}
+// rounds between folds (0: only at the end, for FP64 accumulators)
+template <typename T>
+constexpr int fold_rounds() {
+  return std::is_same<T, float>::value ? kFoldRounds : 0;
+}
+
 // NORM: a == b, only the real part |a|^2 is formed (half the multiply-adds,
 // which matters where they are FP64)
 template <typename Ra, typename Rb, typename T, bool NORM = false>
@@ -131,16 +180,19 @@ __global__ void k_dot_partial(const cpx<Ra>* __restrict__ a, const cpx<Rb>* __re
   cpx<T> acc[kAcc];
 #pragma unroll
   for (int k = 0; k < kAcc; ++k) acc[k] = cpx<T>(T(0), T(0));
-  grid_loop_acc(n, [&](size_t i, int k) {
-    if constexpr (NORM) {
-      const cpx<T> x = to_acc<T>(a[i]);
-      acc[k].re = fma(x.re, x.re, fma(x.im, x.im, acc[k].re));
-    } else {
-      cmac_conj(acc[k], to_acc<T>(a[i]), to_acc<T>(b[i]));
-    }
-  });
-  const cpx<T> t = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-  double2 d = block_sum(make_double2(double(t.re), double(t.im)), sh);
+  double2 sum = make_double2(0.0, 0.0);
+  grid_loop_fold<fold_rounds<T>()>(
+      n,
+      [&](size_t i, int k) {
+        if constexpr (NORM) {
+          const cpx<T> x = to_acc<T>(a[i]);
+          acc[k].re = fma(x.re, x.re, fma(x.im, x.im, acc[k].re));
+        } else {
+          cmac_conj(acc[k], to_acc<T>(a[i]), to_acc<T>(b[i]));
+        }
+      },
+      [&] { fold_acc(sum, acc); });
+  double2 d = block_sum(sum, sh);
   if (threadIdx.x == 0) part[size_t(blockIdx.y) * gridDim.x + blockIdx.x] = d;
 }
 
@@ -222,7 +274,8 @@ struct VecList {
 
 // partial <X[j], y> per block at part[(v m + j) * gridDim.x + block].  FF:
 // float-float sums of exact products (FP32 operands, FP64-accurate);
-// otherwise sums in acc_t<R, R>.  Each j is its own accumulation chain.
+// otherwise sums in acc_t<R, R>, FP32 ones folded into FP64 every 16 terms.
+// Each j is its own accumulation chain.
 template <typename R, bool FF>
 __global__ void __launch_bounds__(256, 2) k_dot_multi(VecList X, const cpx<R>* __restrict__ y, int m, size_t n,
                             double2* __restrict__ part) {
@@ -238,9 +291,31 @@ __global__ void __launch_bounds__(256, 2) k_dot_multi(VecList X, const cpx<R>* _
     acc[j] = cpx<T>(T(0), T(0));
     rh[j] = rl[j] = ih[j] = il[j] = 0.f;
   }
+  constexpr bool FOLD = !FF && std::is_same<T, float>::value;
+  double2 sum[FOLD ? kCgs : 1];
+  if constexpr (FOLD) {
+#pragma unroll
+    for (int j = 0; j < kCgs; ++j) sum[j] = make_double2(0.0, 0.0);
+  }
+  auto fold = [&] {
+    if constexpr (FOLD) {
+#pragma unroll
+      for (int j = 0; j < kCgs; ++j)
+        if (j < m) {
+          sum[j].x += f2d(acc[j].re);
+          sum[j].y += f2d(acc[j].im);
+          acc[j] = cpx<T>(T(0), T(0));
+        }
+    }
+  };
+  int c = 0;
   for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < n;
        i += size_t(gridDim.x) * blockDim.x) {
     const cpx<R> yi = y[i];
+    if (FOLD && c++ == 4 * kFoldRounds) {
+      fold();
+      c = 1;
+    }
 #pragma unroll
     for (int j = 0; j < kCgs; ++j)
       if (j < m) {
@@ -257,12 +332,15 @@ __global__ void __launch_bounds__(256, 2) k_dot_multi(VecList X, const cpx<R>* _
         }
       }
   }
+  fold();
 #pragma unroll
   for (int j = 0; j < kCgs; ++j)
     if (j < m) {  // m is uniform: every thread takes the same branches
       double2 d;
       if constexpr (FF)
         d = make_double2(double(rh[j]) + double(rl[j]), double(ih[j]) + double(il[j]));
+      else if constexpr (FOLD)
+        d = sum[j];
       else
         d = make_double2(double(acc[j].re), double(acc[j].im));
       d = block_sum(d, sh);
@@ -401,16 +479,22 @@ __global__ void k_dot2_partial_b(const cpx<Ra>* __restrict__ p, const cpx<Rb>* _
     pr_k[k] = cpx<T>(T(0), T(0));
     pp_k[k] = T(0);
   }
-  grid_loop_acc(n, [&](size_t i, int k) {
-    cpx<T> x(p[i]), y(r[i]);
-    cmac_conj(pr_k[k], x, y);
-    pp_k[k] = fma(x.re, x.re, fma(x.im, x.im, pp_k[k]));
-  });
-  const cpx<T> a_pr = (pr_k[0] + pr_k[1]) + (pr_k[2] + pr_k[3]);
-  const T a_pp = (pp_k[0] + pp_k[1]) + (pp_k[2] + pp_k[3]);
-  double2 pr = block_sum(make_double2(double(a_pr.re), double(a_pr.im)), sh);
+  double2 s_pr = make_double2(0.0, 0.0);
+  double s_pp = 0.0;
+  grid_loop_fold<fold_rounds<T>()>(
+      n,
+      [&](size_t i, int k) {
+        cpx<T> x(p[i]), y(r[i]);
+        cmac_conj(pr_k[k], x, y);
+        pp_k[k] = fma(x.re, x.re, fma(x.im, x.im, pp_k[k]));
+      },
+      [&] {
+        fold_acc(s_pr, pr_k);
+        fold_acc(s_pp, pp_k);
+      });
+  double2 pr = block_sum(s_pr, sh);
   __syncthreads();
-  double2 pp = block_sum(make_double2(double(a_pp), 0.0), sh);
+  double2 pp = block_sum(make_double2(s_pp, 0.0), sh);
   if (threadIdx.x == 0) {
     const size_t base = size_t(blockIdx.y) * 2 * gridDim.x;
     part[base + blockIdx.x] = pr;
@@ -597,22 +681,25 @@ __global__ void __launch_bounds__(256)
   Rx acc[kAcc];
 #pragma unroll
   for (int k = 0; k < kAcc; ++k) acc[k] = Rx(0);
-  grid_loop_acc(n, [&](size_t i, int k) {
-    cpx<Rx> xi = x[i], ri = r[i];
-    if constexpr (std::is_same<T, float>::value) {
-      xi += to_acc<Rx>(a * cpx<T>(z[i]));
-      ri -= to_acc<Rx>(a * cpx<T>(w[i]));
-    } else {
-      cmac(xi, cpx<Rx>(a), cpx<Rx>(z[i]));
-      cmac(ri, -cpx<Rx>(a), cpx<Rx>(w[i]));
-    }
-    x[i] = xi;
-    r[i] = ri;
-    if (rk) rk[i] = narrow(ri);
-    acc[k] = fma(ri.re, ri.re, fma(ri.im, ri.im, acc[k]));
-  });
-  const double t = double((acc[0] + acc[1]) + (acc[2] + acc[3]));
-  const double2 d = block_sum(make_double2(t, 0.0), sh);
+  double sum = 0.0;
+  grid_loop_fold<fold_rounds<Rx>()>(
+      n,
+      [&](size_t i, int k) {
+        cpx<Rx> xi = x[i], ri = r[i];
+        if constexpr (std::is_same<T, float>::value) {
+          xi += to_acc<Rx>(a * cpx<T>(z[i]));
+          ri -= to_acc<Rx>(a * cpx<T>(w[i]));
+        } else {
+          cmac(xi, cpx<Rx>(a), cpx<Rx>(z[i]));
+          cmac(ri, -cpx<Rx>(a), cpx<Rx>(w[i]));
+        }
+        x[i] = xi;
+        r[i] = ri;
+        if (rk) rk[i] = narrow(ri);
+        acc[k] = fma(ri.re, ri.re, fma(ri.im, ri.im, acc[k]));
+      },
+      [&] { fold_acc(sum, acc); });
+  const double2 d = block_sum(make_double2(sum, 0.0), sh);
   if (threadIdx.x == 0) part[size_t(blockIdx.y) * gridDim.x + blockIdx.x] = d;
 }
 
@@ -686,23 +773,31 @@ __global__ void k_dot2_partial_h(const bf16c* __restrict__ p, const bf16c* __res
     cmac_conj(pr_k[k], x, y);
     pp_k[k] = fmaf(x.re, x.re, fmaf(x.im, x.im, pp_k[k]));
   };
+  double2 s_pr = make_double2(0.0, 0.0);
+  double s_pp = 0.0;
+  auto fold = [&] {
+    fold_acc(s_pr, pr_k);
+    fold_acc(s_pp, pp_k);
+  };
   if constexpr (W == 4) {
     const uint4* p4 = reinterpret_cast<const uint4*>(p);
     const uint4* r4 = reinterpret_cast<const uint4*>(r);
-    grid_loop_acc(n / 4, [&](size_t i, int k) {
-      const uint4 wp = p4[i], wr = r4[i];
+    grid_loop_fold<kFoldRounds / 4>(
+        n / 4,
+        [&](size_t i, int k) {
+          const uint4 wp = p4[i], wr = r4[i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        term(reinterpret_cast<const bf16c*>(&wp)[j], reinterpret_cast<const bf16c*>(&wr)[j], k);
-    });
+          for (int j = 0; j < 4; ++j)
+            term(reinterpret_cast<const bf16c*>(&wp)[j], reinterpret_cast<const bf16c*>(&wr)[j],
+                 k);
+        },
+        fold);
   } else {
-    grid_loop_acc(n, [&](size_t i, int k) { term(p[i], r[i], k); });
+    grid_loop_fold<kFoldRounds>(n, [&](size_t i, int k) { term(p[i], r[i], k); }, fold);
   }
-  const cpx<float> a_pr = (pr_k[0] + pr_k[1]) + (pr_k[2] + pr_k[3]);
-  const float a_pp = (pp_k[0] + pp_k[1]) + (pp_k[2] + pp_k[3]);
-  double2 pr = block_sum(make_double2(double(a_pr.re), double(a_pr.im)), sh);
+  double2 pr = block_sum(s_pr, sh);
   __syncthreads();
-  double2 pp = block_sum(make_double2(double(a_pp), 0.0), sh);
+  double2 pp = block_sum(make_double2(s_pp, 0.0), sh);
   if (threadIdx.x == 0) {
     const size_t base = size_t(blockIdx.y) * 2 * gridDim.x;
     part[base + blockIdx.x] = pr;
