@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(256, P * RPT >= 16 ? 2 : 3)
   __shared__ ff sh[33];
   __shared__ ff part[NW][kQrMaxVec][2 * P];
   __shared__ ffc coef[kQrMaxVec][P];
-  __shared__ float fsum[NW];
+  __shared__ double left[kQrMaxVec];  // norm that a column keeps after the projections
   const int half = nd / 2, rows = m.per * half;
   const int xc = blockIdx.x >> 1, chi = blockIdx.x & 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -565,22 +565,10 @@ __global__ void __launch_bounds__(256, P * RPT >= 16 ? 2 : 3)
     ff_msub(v.ih, v.il, c.rh, c.rl, q.ih, q.il);
     ff_msub(v.ih, v.il, c.ih, c.il, q.rh, q.rl);
   };
-  // Frobenius norm of the block for the rank test (a threshold: FP32 will do)
-  float f = 0.f;
-  for (int i = 0; i < nv; ++i)
-#pragma unroll
-    for (int r = 0; r < RPT; ++r)
-      if (has(r)) {
-        const double2 v = raw[size_t(i) * vstride + at[r]];
-        const float a = float(v.x), b = float(v.y);
-        f = fmaf(a, a, fmaf(b, b, f));
-      }
-  for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-  if (lane == 0) fsum[warp] = f;
-  __syncthreads();
-  double scale = 0.0;
-  for (int w = 0; w < NW; ++w) scale += double(fsum[w]);
-  scale = sqrt(scale);
+  // squared Frobenius norm of the columns so far, the sum of their squared norms
+  // (float-float like every other one): the rank test is against that of the
+  // whole block, so it is decided at the end
+  double fro = 0.0;
 
   for (int i0 = 0; i0 < nv; i0 += P) {
     const int pc = min(P, nv - i0);
@@ -633,7 +621,10 @@ __global__ void __launch_bounds__(256, P * RPT >= 16 ? 2 : 3)
     __syncthreads();
     double n0[P];
 #pragma unroll
-    for (int c = 0; c < P; ++c) n0[c] = ff_to(ff{coef[i0][c].rh, coef[i0][c].rl});
+    for (int c = 0; c < P; ++c) {
+      n0[c] = ff_to(ff{coef[i0][c].rh, coef[i0][c].rl});
+      fro += n0[c];
+    }
     for (int j = 0; j < i0; ++j) {
       const ffc* q = B + size_t(j) * rows + tid;
 #pragma unroll
@@ -692,12 +683,9 @@ __global__ void __launch_bounds__(256, P * RPT >= 16 ? 2 : 3)
         }
       }
       const double nrm = sqrt(n1);
+      if (tid == 0) left[i] = nrm;
       float sh_inv = 0.f, sl_inv = 0.f;
-      if (nrm <= 1e-12 * scale) {
-        if (tid == 0) atomicOr(status, 1);
-      } else {
-        ff_split(1.0 / nrm, sh_inv, sl_inv);
-      }
+      if (!(n1 <= 1e-24 * fro)) ff_split(1.0 / nrm, sh_inv, sl_inv);
 #pragma unroll
       for (int r = 0; r < RPT; ++r) {
         ff_scale(v[c][r].rh, v[c][r].rl, sh_inv, sl_inv);
@@ -734,6 +722,9 @@ __global__ void __launch_bounds__(256, P * RPT >= 16 ? 2 : 3)
     }
     __syncthreads();  // the panel's columns are visible to the CTA; part, coef free
   }
+  // (the last panel's barrier: `left` is complete)
+  const double scale = sqrt(fro);
+  if (tid < nv && left[tid] <= 1e-12 * scale) atomicOr(status, 1);
 }
 
 // QR of every (aggregate, chirality) block of W; false if a block is too tall.
