@@ -12,37 +12,40 @@
 // T rows 2 c, 2 c + 1 = Re, Im of column c, P rows i, Nv + i = Re, Im of
 // vector i: every product of the four a complex multiply needs, none twice.
 //
-// Accuracy: every FP32 operand v is split into two FP16 numbers, hi = fp16(v),
-// lo = fp16(2048 (v - hi)), which hold it to 2^-24 |v| (entries of P are at
-// most 1, |T| is bounded by the operator's norm, checked by the launcher, so
-// nothing overflows; the scaled lo keeps what a subnormal hi loses).  Three
-// products hi hi, hi lo, lo hi; the two small ones (scaled by 2048) have an
-// accumulator of their own, the dropped lo lo is 2^-24 of a product.  The
-// accumulators run over a unit of one or two chunks of eight sites (3 or 6
-// steps of K = 16) and are then added to FP32 registers: the tensor cores
-// truncate when they accumulate, and on the X blocks, whose sums have one
-// sign, that bias grows with the unit.  Relative error of the links against 64
-// bits, 24 vectors (the FP32 pipe's own sums in brackets): units of one chunk
-// 1.6e-7 on 2^4 [2.1e-7] and 4^4 [7.7e-7] aggregates, of two 3.1e-7 and
-// 3.0e-7, of four 3.1e-7 and 6.7e-7.  The time for 24^3x48 in 4^4 aggregates is
-// 5.41, 5.22 and 5.11 ms.  So two chunks where the aggregate has 64 sites or
-// more (FP32 pipe 3.9e-7), one below.
+// Accuracy: every FP32 operand v is split into three BF16 numbers, each the
+// rounding of what the ones before it leave: 3 x 8 bits, so that their sum is v
+// itself (BF16 has FP32's exponents: entries of any size, down to 2^-110).  Six
+// products hold v w to 2^-26 of it: hi hi in one accumulator; hi mid, mid hi, hi
+// lo, mid mid, lo hi, 2^-8 of it and less, in another.  (FP16 pairs held an
+// operand to 2^-23, and numbers below 2^-13 to a fixed 2^-36: with vectors 1e-6 of
+// the others at the faces of their aggregate, face blocks were 0.1 to 0.3 of their
+// norm off.)  The
+// accumulators run over a unit of one chunk of eight sites (3 steps of K = 16) on
+// the X blocks, of two on the face blocks, and are then added to FP32 registers:
+// the tensor cores truncate when they accumulate, and on the X blocks, whose sums
+// have one sign, that bias grows with the unit.  Relative error of the links
+// against 64 bits, 24 vectors (the FP32 pipe's own sums in brackets): Gaussian
+// vectors 1.2e-7 on 2^4 [2.1e-7] and 1.3e-7 on 4^4 [7.7e-7] aggregates; one site
+// of each 2x4^3 aggregate large and the others 1e-3 of it, 1.9e-7 [1.1e-6]; sites
+// at the faces 1e-6 of the inner ones, worst face block 1.4e-7 [5.3e-7].  Units of
+// two chunks on the X blocks too: 1.6e-7 on 4^4, 5.97 against 6.00 ms for 24^3x48;
+// of one everywhere: 6.09 ms.
 //
 // What bounds it now: the T warps, on the latency of the P and link gathers
-// (issue 46 %, long-scoreboard stalls; the tensor pipe is 7 % busy).  24^3x48,
-// Nv = 24, 4^4 aggregates: 9.21 -> 5.22 ms for 281 GFLOP; error of the links
-// against 64 bits 7.7e-7 -> 3.0e-7.  Two-row links with two hops loaded
-// ahead: 5.8 ms (spills).
+// (issue 46 %, long-scoreboard stalls; the tensor pipe is 14 % busy).  24^3x48,
+// Nv = 24, 4^4 aggregates, 281 GFLOP: 9.21 -> 5.58 ms (FP16 pairs: 5.25, the
+// third piece's stores and shared memory), the call with its export 9.67 ->
+// 6.00.  Two-row links with two hops loaded ahead were slower (spills).
 // One resident CTA per SM walks the (xc, d) blocks, X blocks first.  Roles:
 // 16 Nv T threads, one column of one of the chunk's 8 sites each (Nv = 24:
 // 12 warps), writing the split operands into a ring of kRing stages; one
-// thread issuing the 18 MMAs of a chunk; warps 0.. adding finished units from
+// thread issuing the 36 MMAs of a chunk; warps 0.. adding finished units from
 // TMEM (two sets of accumulators in turn) and storing the block.  Every wait
 // is bounded: the role whose time runs out sets the error word and the CTA's
 // abort flag, which every waiting role reads, whole warps decide together
 // (wait_or_abort_warp), the MMAs in flight are waited for (bounded), TMEM is
 // freed and the CTA leaves.
-#include <cmath>
+#include <cuda_bf16.h>
 
 #include "kernels.cuh"
 #include "tcgen05.cuh"
@@ -53,9 +56,9 @@ namespace gbmg {
 namespace {
 
 constexpr int kCh = 8;         // fine sites per chunk: K = 48 per chirality
-constexpr int kRing = 2;       // operand stages (3: 4 % slower, less L1 left for P)
+constexpr int kRing = 2;       // operand stages (a third does not fit)
 constexpr int kMaxPer = 512;   // fine sites per aggregate (the site tables)
-constexpr float kLoScale = 2048.f;
+constexpr int kUnitX = 1, kUnitY = 2;  // chunks accumulated in TMEM, X and face blocks
 
 template <int NV>
 struct GM {
@@ -65,10 +68,13 @@ struct GM {
   static constexpr int THREADS = 128 + TT;
   static constexpr int ND = (4 * NV + 31) / 32;    // warps that drain
   static constexpr uint32_t LBO = 128, SBO = 6 * 128 + 16;  // +16: fewer bank conflicts
-  static constexpr uint32_t ASZ = 16 * SBO, BSZ = uint32_t(N / 8) * SBO;
-  static constexpr uint32_t STAGE = 4 * ASZ + 4 * BSZ;
+  // (the MMA's T rows from 4 NV to 128 read on into the next operand; their
+  // accumulator rows are never read)
+  static constexpr uint32_t ASZ = uint32_t(NV / 2) * SBO, BSZ = uint32_t(N / 8) * SBO;
+  static constexpr uint32_t STAGE = 6 * ASZ + 6 * BSZ;
   static constexpr uint32_t TMEM = N * 8 <= 256 ? 256 : 512;
   static constexpr size_t SMEM = size_t(kRing) * STAGE + kMaxPer * (8 + 16);
+  static_assert(16 * SBO <= ASZ + BSZ * 6, "the last T operand's rows end inside the stage");
   static_assert(N * 8 <= 512 && TT % 32 == 0 && N % 16 == 0 && ND <= 3, "tile shape");
 };
 
@@ -78,13 +84,15 @@ struct GalMap {
   int per;
 };
 
-// fp16 split of two numbers
-__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
-  const __half2 h = __floats2half2_rn(a, b);
-  const float2 f = __half22float2(h);
-  const __half2 l = __floats2half2_rn((a - f.x) * kLoScale, (b - f.y) * kLoScale);
-  hi = *reinterpret_cast<const uint32_t*>(&h);
-  lo = *reinterpret_cast<const uint32_t*>(&l);
+// two numbers as three BF16 pairs: w[0] + w[1] + w[2] is each of them exactly
+__device__ __forceinline__ void split3(float a, float b, uint32_t (&w)[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    w[k] = *reinterpret_cast<const uint32_t*>(&h);
+    a -= __uint_as_float(w[k] << 16);
+    b -= __uint_as_float(w[k] & 0xffff0000u);
+  }
 }
 
 template <int E>
@@ -194,7 +202,7 @@ __device__ __forceinline__ void t_column_y(const cpx<float>* __restrict__ U,
 template <int NV>
 __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
     k_galerkin_mma(const cpx<float>* __restrict__ U, const float* __restrict__ A, float diag,
-                   const cpx<float>* __restrict__ Vp, GalMap m, int unit,
+                   const cpx<float>* __restrict__ Vp, GalMap m,
                    cpx<float>* __restrict__ out, int* __restrict__ err, int stall) {
   using G = GM<NV>;
   constexpr int N = G::N;
@@ -265,19 +273,18 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
     return mu == 0 ? m.b[0] : mu == 1 ? m.b[1] : mu == 2 ? m.b[2] : m.b[3];
   };
   auto item_cnt = [&](int d) { return d == 0 ? m.per : m.per / face_b(d); };
+  auto item_unit = [&](int d) { return d == 0 ? kUnitX : kUnitY; };  // chunks per unit
 
   if (warp >= 4) {
     // ---------------------------------------------------------- T threads
     const int t = tid - 128;
     const int sp = t / (kCh * NV), sl = (t / NV) % kCh, j = t % NV;
     const int col = sp * NV + j;
-    // operand offsets of this thread's k pairs, k = 6 sl + 2 p
-    uint32_t ko[3];
-#pragma unroll
-    for (int p = 0; p < 3; ++p) {
-      const int k = 6 * sl + 2 * p;
-      ko[p] = uint32_t((k >> 3) * 128 + (k & 7) * 2);
-    }
+    // operand offsets of this thread's three k pairs.  The order of k is free as
+    // long as both operands have the same: site sl's first two pairs are k = 4 sl
+    // .. 4 sl + 3, one 8-byte word, its third k = 32 + 2 sl.
+    const uint32_t ko8 = uint32_t((sl >> 1) * 128 + (sl & 1) * 8);
+    const uint32_t ko4 = uint32_t((4 + (sl >> 2)) * 128 + (sl & 3) * 4);
     auto ro = [&](int row) { return uint32_t((row >> 3) * G::SBO + (row & 7) * 16); };
     const uint32_t ra = ro(2 * col), rai = ro(2 * col + 1), rb = ro(j), rbi = ro(NV + j);
     int q = 0;
@@ -335,35 +342,27 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
           break;
         }
         unsigned char* st = sm + size_t(sg) * G::STAGE;
+        // rows r (real parts) and ri (imaginary parts) of an operand's three
+        // pieces, sz bytes apart
+        auto put = [&](unsigned char* base, uint32_t sz, uint32_t r, uint32_t ri,
+                       const cpx<float>* v) {
 #pragma unroll
-        for (int chi = 0; chi < 2; ++chi) {
-          unsigned char* ah = st + (chi * 2) * G::ASZ;
-          unsigned char* al = ah + G::ASZ;
+          for (int im = 0; im < 2; ++im) {
+            uint32_t w[3][3];  // [pair][piece]
 #pragma unroll
-          for (int p = 0; p < 3; ++p) {
-            uint32_t h, l;
-            const cpx<float> a = o[6 * chi + 2 * p], b = o[6 * chi + 2 * p + 1];
-            split2(a.re, b.re, h, l);
-            *reinterpret_cast<uint32_t*>(ah + ra + ko[p]) = h;
-            *reinterpret_cast<uint32_t*>(al + ra + ko[p]) = l;
-            split2(a.im, b.im, h, l);
-            *reinterpret_cast<uint32_t*>(ah + rai + ko[p]) = h;
-            *reinterpret_cast<uint32_t*>(al + rai + ko[p]) = l;
+            for (int p = 0; p < 3; ++p)
+              split3(im ? v[2 * p].im : v[2 * p].re, im ? v[2 * p + 1].im : v[2 * p + 1].re, w[p]);
+            unsigned char* row = base + (im ? ri : r);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+              *reinterpret_cast<uint2*>(row + k * sz + ko8) = make_uint2(w[0][k], w[1][k]);
+              *reinterpret_cast<uint32_t*>(row + k * sz + ko4) = w[2][k];
+            }
           }
-        }
-        unsigned char* bh = st + 4 * G::ASZ + (sp * 2) * G::BSZ;
-        unsigned char* bl = bh + G::BSZ;
-#pragma unroll
-        for (int p = 0; p < 3; ++p) {
-          uint32_t h, l;
-          const cpx<float> a = v0[2 * p], b = v0[2 * p + 1];
-          split2(a.re, b.re, h, l);
-          *reinterpret_cast<uint32_t*>(bh + rb + ko[p]) = h;
-          *reinterpret_cast<uint32_t*>(bl + rb + ko[p]) = l;
-          split2(a.im, b.im, h, l);
-          *reinterpret_cast<uint32_t*>(bh + rbi + ko[p]) = h;
-          *reinterpret_cast<uint32_t*>(bl + rbi + ko[p]) = l;
-        }
+        };
+        put(st, G::ASZ, ra, rai, o);
+        put(st + 3 * G::ASZ, G::ASZ, ra, rai, o + 6);
+        put(st + 6 * G::ASZ + 3 * sp * G::BSZ, G::BSZ, rb, rbi, v0);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&full[sg]);
@@ -372,12 +371,12 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
   } else if (warp == 3) {
     // ---------------------------------------------------------- MMA issue
     if (lane == 0) {
-      constexpr uint32_t idesc = mma_idesc(128, N, false);
+      constexpr uint32_t idesc = mma_idesc(128, N, true);
       int q = 0, w = 0;
       // (fault injection, host-set: waits for what never comes)
       bool ok = !stall || wait_or_abort(&stall_bar, 0u, &abort_sh, err);
       for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
-        const int nch = (item_cnt(item_d(it)) + kCh - 1) / kCh;
+        const int nch = (item_cnt(item_d(it)) + kCh - 1) / kCh, unit = item_unit(item_d(it));
         for (int c = 0; c < nch && ok; ++c, ++q) {
           const int set = w & 1;
           const bool first = c % unit == 0;
@@ -393,16 +392,21 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
           for (int chi = 0; chi < 2; ++chi)
 #pragma unroll
             for (int ks = 0; ks < 3; ++ks) {
-              const uint32_t a0 = st + (chi * 2) * G::ASZ + ks * 256;
-              const uint32_t b0 = st + 4 * G::ASZ + (chi * 2) * G::BSZ + ks * 256;
-              const uint64_t ah = smem_desc(a0, G::LBO, G::SBO);
-              const uint64_t al = smem_desc(a0 + G::ASZ, G::LBO, G::SBO);
-              const uint64_t bh = smem_desc(b0, G::LBO, G::SBO);
-              const uint64_t bl = smem_desc(b0 + G::BSZ, G::LBO, G::SBO);
+              const uint32_t a0 = st + (chi * 3) * G::ASZ + ks * 256;
+              const uint32_t b0 = st + 6 * G::ASZ + (chi * 3) * G::BSZ + ks * 256;
+              uint64_t a[3], b[3];
+#pragma unroll
+              for (int k = 0; k < 3; ++k) {
+                a[k] = smem_desc(a0 + k * G::ASZ, G::LBO, G::SBO);
+                b[k] = smem_desc(b0 + k * G::BSZ, G::LBO, G::SBO);
+              }
               const uint32_t acc = (first && ks == 0) ? 0u : 1u;
-              mma_f16(dmain + chi * N, ah, bh, idesc, acc);
-              mma_f16(dsmall + chi * N, ah, bl, idesc, acc);
-              mma_f16(dsmall + chi * N, al, bh, idesc, 1u);
+              mma_f16(dsmall + chi * N, a[0], b[2], idesc, acc);
+              mma_f16(dsmall + chi * N, a[1], b[1], idesc, 1u);
+              mma_f16(dsmall + chi * N, a[2], b[0], idesc, 1u);
+              mma_f16(dsmall + chi * N, a[0], b[1], idesc, 1u);
+              mma_f16(dsmall + chi * N, a[1], b[0], idesc, 1u);
+              mma_f16(dmain + chi * N, a[0], b[0], idesc, acc);
             }
           mma_commit(&empty[sg]);
           if (c % unit == unit - 1 || c == nch - 1) {
@@ -425,7 +429,7 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
     bool ok = true;
     for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
       const int d = item_d(it), xc = item_xc(it);
-      const int nun = ((item_cnt(d) + kCh - 1) / kCh + unit - 1) / unit;
+      const int unit = item_unit(d), nun = ((item_cnt(d) + kCh - 1) / kCh + unit - 1) / unit;
       float acc[2 * N];
 #pragma unroll
       for (int i = 0; i < 2 * N; ++i) acc[i] = 0.f;
@@ -444,7 +448,7 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
           for (int k = 0; k < 16; ++k) acc[i + k] += v[k];
           tmem_ld16(tl + uint32_t(set) * 4 * N + 2 * N + i, v);
 #pragma unroll
-          for (int k = 0; k < 16; ++k) acc[i + k] = fmaf(v[k], 1.f / kLoScale, acc[i + k]);
+          for (int k = 0; k < 16; ++k) acc[i + k] += v[k];
         }
         tc_fence_before();
         __syncwarp();
@@ -492,7 +496,7 @@ void launch_galerkin_mma(mg_ctx* c, const Level& F, const GalMap& m, cpx<float>*
   const int items = 9 * m.coarse.vol;
   k<<<items < sms ? items : sms, GM<NV>::THREADS, GM<NV>::SMEM, st>>>(
       F.gauge32.as<cpx<float>>(), F.clover32.as<float>(), float(F.diag), F.Vp.as<cpx<float>>(), m,
-      m.per >= 64 ? 2 : 1, out, err, take_fault(c->inject_galerkin_stall));
+      out, err, take_fault(c->inject_galerkin_stall));
   GB_LAUNCH_CHECK();
 }
 
@@ -501,12 +505,9 @@ void launch_galerkin_mma(mg_ctx* c, const Level& F, const GalMap& m, cpx<float>*
 bool galerkin_mma(mg_ctx* c, int level, cudaStream_t st) {
   const Level& F = c->L[level];
   const Level& C = c->L[level + 1];
-  // FP32 Wilson-clover level with SU(3) links, 16 or 24 vectors; |T| <=
-  // |diag| + |A| + 8 stays far inside FP16's range (the clover blocks are at
-  // most 6 csw for unitary links)
+  // FP32 Wilson-clover level with SU(3) links, 16 or 24 vectors
   if (level != 0 || F.vprec != MG_F32 || C.vprec != MG_F32 || !F.gauge12_ok) return false;
   if (F.nvec != 16 && F.nvec != 24) return false;
-  if (!(std::fabs(F.diag) + 8.0 * std::fabs(c->p.csw) + 8.0 < 16384.0)) return false;
   GalMap m;
   m.fine = F.g;
   m.coarse = C.g;
