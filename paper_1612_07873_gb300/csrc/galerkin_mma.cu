@@ -36,7 +36,7 @@
 // Nv = 24, 4^4 aggregates, 281 GFLOP: 9.21 -> 5.58 ms (FP16 pairs: 5.25, the
 // third piece's stores and shared memory), the call with its export 9.67 ->
 // 6.00.  Two-row links with two hops loaded ahead were slower (spills).
-// One resident CTA per SM walks the (xc, d) blocks, X blocks first.  Roles:
+// One resident CTA per SM walks its (xc, d) blocks, X blocks first.  Roles:
 // 16 Nv T threads, one column of one of the chunk's 8 sites each (Nv = 24:
 // 12 warps), writing the split operands into a ring of kRing stages; one
 // thread issuing the 36 MMAs of a chunk; warps 0.. adding finished units from
@@ -46,6 +46,8 @@
 // (wait_or_abort_warp), the MMAs in flight are waited for (bounded), TMEM is
 // freed and the CTA leaves.
 #include <cuda_bf16.h>
+
+#include <algorithm>
 
 #include "kernels.cuh"
 #include "tcgen05.cuh"
@@ -82,6 +84,9 @@ struct GalMap {
   Geom fine, coarse;
   int b[4];
   int per;
+  // the last round of X blocks has `rem`, so `spare` CTAs go without; those take
+  // the first `some` face blocks
+  int rem, spare, some;
 };
 
 // two numbers as three BF16 pairs: w[0] + w[1] + w[2] is each of them exactly
@@ -199,7 +204,7 @@ __device__ __forceinline__ void t_column_y(const cpx<float>* __restrict__ U,
 }
 
 // Sec. 3.4 step 4: P^dag M P into the nine blocks of Eq. (3).
-template <int NV>
+template <int NV, bool DEAL>
 __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
     k_galerkin_mma(const cpx<float>* __restrict__ U, const float* __restrict__ A, float diag,
                    const cpx<float>* __restrict__ Vp, GalMap m,
@@ -268,6 +273,25 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
   // eight face blocks of each site
   auto item_d = [&](int it) { return it < cvol ? 0 : 1 + ((it - cvol) & 7); };
   auto item_xc = [&](int it) { return it < cvol ? it : (it - cvol) >> 3; };
+  // A role's walk over the CTA's blocks, dealt out round robin.  DEAL: X blocks
+  // round robin; on the CTAs that got one X block less, their share of the first
+  // m.some face blocks; then all others round robin.
+  auto rest = [&] {
+    const int turn = int(blockIdx.x) - m.rem;
+    return cvol + m.some + (turn < 0 ? turn + int(gridDim.x) : turn);
+  };
+  auto faces = [&] {
+    const int y = cvol + int(blockIdx.x) - m.rem;
+    return y >= cvol && y < cvol + m.some ? y : rest();
+  };
+  auto first_item = [&] {
+    return !DEAL || int(blockIdx.x) < cvol ? int(blockIdx.x) : faces();
+  };
+  auto next_item = [&](int it) {
+    if (!DEAL || it >= cvol + m.some) return it + int(gridDim.x);
+    if (it < cvol) return it + int(gridDim.x) < cvol ? it + int(gridDim.x) : faces();
+    return it + m.spare < cvol + m.some ? it + m.spare : rest();
+  };
   auto face_b = [&](int d) {
     const int mu = (d - 1) >> 1;
     return mu == 0 ? m.b[0] : mu == 1 ? m.b[1] : mu == 2 ? m.b[2] : m.b[3];
@@ -289,7 +313,7 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
     const uint32_t ra = ro(2 * col), rai = ro(2 * col + 1), rb = ro(j), rbi = ro(NV + j);
     int q = 0;
     bool ok = true;
-    for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+    for (int it = first_item(); it < items && ok; it = next_item(it)) {
       const int d = item_d(it), xc = item_xc(it), cnt = item_cnt(d);
       int cc[4];
       site_coords(m.coarse, xc, cc);
@@ -375,7 +399,7 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
       int q = 0, w = 0;
       // (fault injection, host-set: waits for what never comes)
       bool ok = !stall || wait_or_abort(&stall_bar, 0u, &abort_sh, err);
-      for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+      for (int it = first_item(); it < items && ok; it = next_item(it)) {
         const int nch = (item_cnt(item_d(it)) + kCh - 1) / kCh, unit = item_unit(item_d(it));
         for (int c = 0; c < nch && ok; ++c, ++q) {
           const int set = w & 1;
@@ -427,7 +451,7 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
     const bool odd = row & 1;
     int w = 0;
     bool ok = true;
-    for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+    for (int it = first_item(); it < items && ok; it = next_item(it)) {
       const int d = item_d(it), xc = item_xc(it);
       const int unit = item_unit(d), nun = ((item_cnt(d) + kCh - 1) / kCh + unit - 1) / unit;
       float acc[2 * N];
@@ -485,16 +509,27 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
 }
 
 template <int NV>
-void launch_galerkin_mma(mg_ctx* c, const Level& F, const GalMap& m, cpx<float>* out, int* err,
+void launch_galerkin_mma(mg_ctx* c, const Level& F, GalMap m, cpx<float>* out, int* err,
                          cudaStream_t st) {
-  auto k = k_galerkin_mma<NV>;
-  GB_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                int(GM<NV>::SMEM)));
   int dev = 0, sms = 0;
   GB_CHECK(cudaGetDevice(&dev));
   GB_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int items = 9 * m.coarse.vol;
-  k<<<items < sms ? items : sms, GM<NV>::THREADS, GM<NV>::SMEM, st>>>(
+  const int items = 9 * m.coarse.vol, grid = items < sms ? items : sms;
+  // An X block costs as much as 1.8 face blocks per chunk of sites (4^4 aggregates:
+  // 133 us against 18 for 16 vectors, 150 against 22 for 24), so with few rounds of
+  // large ones the CTAs that got one less are given face blocks for it: 189 coarse
+  // sites, 16 vectors, 449 -> 373 us.  From about four rounds on, and on small
+  // aggregates, the plain order is as even and 1 to 5 % faster.
+  int xch = ceil_div(m.per, kCh), ych = 0;
+  for (int mu = 0; mu < 4; ++mu) ych += 2 * ceil_div(m.per / m.b[mu], kCh);
+  m.rem = m.coarse.vol % grid;
+  m.spare = m.rem ? grid - m.rem : 0;
+  m.some = std::min(8 * m.coarse.vol, m.spare * std::max(1, int(1.8 * 8 * xch / ych + 0.5)));
+  auto k = m.per >= 64 && m.coarse.vol < 4 * grid ? k_galerkin_mma<NV, true>
+                                                  : k_galerkin_mma<NV, false>;
+  GB_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                int(GM<NV>::SMEM)));
+  k<<<grid, GM<NV>::THREADS, GM<NV>::SMEM, st>>>(
       F.gauge32.as<cpx<float>>(), F.clover32.as<float>(), float(F.diag), F.Vp.as<cpx<float>>(), m,
       out, err, take_fault(c->inject_galerkin_stall));
   GB_LAUNCH_CHECK();
