@@ -1066,14 +1066,17 @@ __global__ void __launch_bounds__(256) k_restrict_g(cpx<R>* __restrict__ coarse,
 // reads whole 32-byte sectors; the halves meet by one shuffle.  A pair
 // loads RPI rows (RPI * PW <= 12 words) before any arithmetic, so short
 // rows (16-bit Vp, small Nv) still keep several loads per thread in flight.
-// NDC: dofs per fine site, 12 on the fine level, 0 (nd) on a coarse one.
+// NDC: dofs per fine site, 12 on the fine level, 0 (nd) on a coarse one.  ADD:
+// fine += instead of =.  (As a run-time choice its registers and selects made the
+// plain form up to 13 % slower on short rows: 24x12x16^2, Nv = 8, restriction and
+// prolongation 26.1 -> 27.9 us.)
 // Prolongation P (Sec. 6.6).
-template <typename Rf, typename Rc, typename VT, int PW, int NDC = 12>
+template <typename Rf, typename Rc, typename VT, int PW, bool ADD, int NDC = 12>
 __global__ void __launch_bounds__(256) k_prolong12(cpx<Rf>* __restrict__ fine,
                                                   const cpx<Rc>* __restrict__ coarse,
                                                   const VT* __restrict__ Vp, AggMap m,
                                                   int nd, int nv, int nr, size_t fstride,
-                                                  size_t cstride, int add) {
+                                                  size_t cstride) {
   constexpr int CPL = VUnpack<VT, Rf>::CPL;
   const int ND = NDC ? NDC : nd;
   constexpr int RPI = PW >= 12 ? 1 : (12 / PW > 6 ? 6 : 12 / PW);
@@ -1110,11 +1113,13 @@ __global__ void __launch_bounds__(256) k_prolong12(cpx<Rf>* __restrict__ fine,
         if (ok[j]) w[j][k] = ld_stream16(vr + 2 * k);
     }
     for (int b = 0; b < nr; ++b) {
-      // (add) the old values, loaded ahead of the products
-      cpx<Rf> old[RPI];
+      // ADD: the old values, loaded ahead of the products
+      cpx<Rf> old[ADD ? RPI : 1];
+      if constexpr (ADD) {
 #pragma unroll
-      for (int j = 0; j < RPI; ++j)
-        old[j] = add && ok[j] && q == 0 ? fine[b * fstride + frow[j]] : cpx<Rf>(Rf(0), Rf(0));
+        for (int j = 0; j < RPI; ++j)
+          old[j] = ok[j] && q == 0 ? fine[b * fstride + frow[j]] : cpx<Rf>(Rf(0), Rf(0));
+      }
 #pragma unroll
       for (int j = 0; j < RPI; ++j) {
         const cpx<Rf>* c = cs + b * 2 * nv + coff[j];
@@ -1130,7 +1135,10 @@ __global__ void __launch_bounds__(256) k_prolong12(cpx<Rf>* __restrict__ fine,
         }
         acc.re += __shfl_xor_sync(0xffffffffu, acc.re, 1);
         acc.im += __shfl_xor_sync(0xffffffffu, acc.im, 1);
-        if (ok[j] && q == 0) fine[b * fstride + frow[j]] = add ? old[j] + acc : acc;
+        if (ok[j] && q == 0) {
+          if constexpr (ADD) acc = old[j] + acc;
+          fine[b * fstride + frow[j]] = acc;
+        }
       }
     }
   }
@@ -1406,24 +1414,30 @@ void prolong_apply(mg_ctx* c, int level, Vec fine, Vec coarse, cudaStream_t st, 
   const int pw = nv % (2 * cpl) == 0 ? nv / (2 * cpl) : 0;  // 16-byte words per half row
   if (F.nd == 12 && (pw == 1 || pw == 2 || pw == 3 || pw == 4 || pw == 6 || pw == 8 || pw == 12) &&
       smem2 <= 48 * 1024) {
-    auto go = [&](auto pwc) {
+    auto launch = [&](auto pwc, auto addc) {
       constexpr int PW = decltype(pwc)::value;
+      constexpr bool ADD = decltype(addc)::value;
       if (h16) {
         if (coarse.prec == MG_F64)
-          k_prolong12<float, double, bf16c, PW><<<C.g.vol, 256, smem2, st>>>(
+          k_prolong12<float, double, bf16c, PW, ADD><<<C.g.vol, 256, smem2, st>>>(
               (cpx<float>*)fine.p, (const cpx<double>*)coarse.p, F.Vp16.as<bf16c>(), m, 12, nv, nr,
-              fine.n, coarse.n, int(add));
+              fine.n, coarse.n);
         else
-          k_prolong12<float, float, bf16c, PW><<<C.g.vol, 256, smem2, st>>>(
+          k_prolong12<float, float, bf16c, PW, ADD><<<C.g.vol, 256, smem2, st>>>(
               (cpx<float>*)fine.p, (const cpx<float>*)coarse.p, F.Vp16.as<bf16c>(), m, 12, nv, nr,
-              fine.n, coarse.n, int(add));
+              fine.n, coarse.n);
       } else {
         GB_TRANSFER_DISPATCH(F.vprec, coarse.prec, Rf, Rc,
-                             (k_prolong12<Rf, Rc, cpx<Rf>, PW><<<C.g.vol, 256, smem2, st>>>(
+                             (k_prolong12<Rf, Rc, cpx<Rf>, PW, ADD><<<C.g.vol, 256, smem2, st>>>(
                                  (cpx<Rf>*)fine.p, (const cpx<Rc>*)coarse.p,
-                                 F.Vp.as<cpx<Rf>>(), m, 12, nv, nr, fine.n, coarse.n,
-                                 int(add))));
+                                 F.Vp.as<cpx<Rf>>(), m, 12, nv, nr, fine.n, coarse.n)));
       }
+    };
+    auto go = [&](auto pwc) {
+      if (add)
+        launch(pwc, std::true_type{});
+      else
+        launch(pwc, std::false_type{});
     };
     switch (pw) {
       case 1: go(std::integral_constant<int, 1>{}); break;
@@ -1444,16 +1458,23 @@ void prolong_apply(mg_ctx* c, int level, Vec fine, Vec coarse, cudaStream_t st, 
     // between coarse levels: the pair-per-row kernel with run-time dofs (8^3x16
     // to 4^3x8, 48 dofs, 32 vectors: 57 us -> under 35 us; the entry-per-thread kernel
     // below divides ten times per entry and reads rows lane by lane)
-    auto go = [&](auto pwc) {
+    auto launch = [&](auto pwc, auto addc) {
       constexpr int PW = decltype(pwc)::value;
+      constexpr bool ADD = decltype(addc)::value;
       if (F.vprec == MG_F64)
-        k_prolong12<double, double, cpx<double>, PW, 0><<<C.g.vol, 256, smem2, st>>>(
+        k_prolong12<double, double, cpx<double>, PW, ADD, 0><<<C.g.vol, 256, smem2, st>>>(
             (cpx<double>*)fine.p, (const cpx<double>*)coarse.p, F.Vp.as<cpx<double>>(), m, F.nd,
-            nv, nr, fine.n, coarse.n, int(add));
+            nv, nr, fine.n, coarse.n);
       else
-        k_prolong12<float, float, cpx<float>, PW, 0><<<C.g.vol, 256, smem2, st>>>(
+        k_prolong12<float, float, cpx<float>, PW, ADD, 0><<<C.g.vol, 256, smem2, st>>>(
             (cpx<float>*)fine.p, (const cpx<float>*)coarse.p, F.Vp.as<cpx<float>>(), m, F.nd, nv,
-            nr, fine.n, coarse.n, int(add));
+            nr, fine.n, coarse.n);
+    };
+    auto go = [&](auto pwc) {
+      if (add)
+        launch(pwc, std::true_type{});
+      else
+        launch(pwc, std::false_type{});
     };
     switch (pw) {
       case 2: go(std::integral_constant<int, 2>{}); break;
