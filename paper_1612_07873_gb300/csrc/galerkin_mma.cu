@@ -28,14 +28,14 @@
 // vectors 1.2e-7 on 2^4 [2.1e-7] and 1.3e-7 on 4^4 [7.7e-7] aggregates; one site
 // of each 2x4^3 aggregate large and the others 1e-3 of it, 1.9e-7 [1.1e-6]; sites
 // at the faces 1e-6 of the inner ones, worst face block 1.4e-7 [5.3e-7].  Units of
-// two chunks on the X blocks too: 1.6e-7 on 4^4, 5.97 against 6.00 ms for 24^3x48;
-// of one everywhere: 6.09 ms.
+// two chunks on the X blocks too: 1.6e-7 on 4^4, 0.5 % faster; of one everywhere:
+// 1.5 % slower.
 //
 // What bounds it now: the T warps, on the latency of the P and link gathers
 // (issue 46 %, long-scoreboard stalls; the tensor pipe is 14 % busy).  24^3x48,
-// Nv = 24, 4^4 aggregates, 281 GFLOP: 9.21 -> 5.58 ms (FP16 pairs: 5.25, the
-// third piece's stores and shared memory), the call with its export 9.67 ->
-// 6.00.  Two-row links with two hops loaded ahead were slower (spills).
+// Nv = 24, 4^4 aggregates, 281 GFLOP: 9.21 -> 5.43 ms (FP16 pairs 5.25: the third
+// piece's conversions and stores), the call with its export 9.67 -> 5.89 ms.
+// Two-row links with two hops loaded ahead were slower (spills).
 // One resident CTA per SM walks its (xc, d) blocks, X blocks first.  Roles:
 // 16 Nv T threads, one column of one of the chunk's 8 sites each (Nv = 24:
 // 12 warps), writing the split operands into a ring of kRing stages; one
@@ -302,7 +302,11 @@ __global__ void __launch_bounds__(GM<NV>::THREADS, 1)
   if (warp >= 4) {
     // ---------------------------------------------------------- T threads
     const int t = tid - 128;
-    const int sp = t / (kCh * NV), sl = (t / NV) % kCh, j = t % NV;
+    // two sites side by side in a warp: their operand words fill each other's gaps,
+    // 8-byte stores without bank conflicts (one column after the other: half of
+    // the banks unused, 5.55 instead of 5.43 ms)
+    const int sp = t / (kCh * NV), pair = (t / (2 * NV)) % (kCh / 2);
+    const int sl = 2 * pair + (t & 1), j = (t % (2 * NV)) >> 1;
     const int col = sp * NV + j;
     // operand offsets of this thread's three k pairs.  The order of k is free as
     // long as both operands have the same: site sl's first two pairs are k = 4 sl
