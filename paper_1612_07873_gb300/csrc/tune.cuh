@@ -12,6 +12,7 @@
 #include <cstdlib>
 #include <fstream>
 #include <mutex>
+#include <set>
 #include <string>
 #include <unordered_map>
 #include <utility>
@@ -119,10 +120,30 @@ class Tuner {
   void set(const std::string& key, int choice) {
     std::lock_guard<std::mutex> lk(mu_);
     load();
-    if (choice < 0)
+    if (choice < 0) {
       best_.erase(key);
-    else
+      pinned_.erase(key);
+    } else {
       best_[key] = choice;
+      pinned_.insert(key);
+    }
+  }
+  // the fastest of the candidates first..last when `key` was tuned, if it came
+  // within slack_ms of the pick; -1 if none did or the key is pinned or unknown
+  int within(const std::string& key, int first, int last, float slack_ms) {
+    std::lock_guard<std::mutex> lk(mu_);
+    auto it = timings_.find(key);
+    if (it == timings_.end() || pinned_.count(key)) return -1;
+    int pick = -1;
+    float best = 1e30f, ms = 1e30f;
+    for (const auto& t : it->second) {
+      best = std::min(best, t.second);
+      if (t.first >= first && t.first <= last && t.second < ms) {
+        ms = t.second;
+        pick = t.first;
+      }
+    }
+    return ms <= best + slack_ms ? pick : -1;
   }
   // the candidates timed when `key` was last tuned, with ms per launch
   std::vector<std::pair<int, float>> report(const std::string& key) {
@@ -156,6 +177,7 @@ class Tuner {
   std::mutex mu_;
   std::unordered_map<std::string, int> best_;
   std::unordered_map<std::string, std::vector<std::pair<int, float>>> timings_;
+  std::set<std::string> pinned_;
   bool loaded_ = false;
   bool enabled_ = true;
   std::string path_;

@@ -1139,7 +1139,15 @@ void wilson_apply(mg_ctx* c, Vec out, Vec in, int nvec, cudaStream_t st, int* np
     }
     const std::string key = "wilson/v" + std::to_string(L.g.vol) + "/n" + std::to_string(nvec) +
                             "/c" + std::to_string(int(L.gauge12_ok));
-    const int q = Tuner::get().choose(key, cands, st, launch);
+    int q = Tuner::get().choose(key, cands, st, launch);
+    if (nparts && (q < 12 || q > 15)) {
+      // the inner products come with a tiled launch; after another one they are a
+      // pass of their own, at least its launches and half of its reads longer
+      // (16^3x8: the plain kernel won by 0.1 us, the MR step lost 5)
+      const float pass_ms = 3e-3f + 96.f * float(nvec) * float(L.g.vol) / 6.8e9f;
+      const int t = Tuner::get().within(key, 12, 15, pass_ms);
+      if (std::find(cands.begin(), cands.end(), t) != cands.end()) q = t;
+    }
     np = nparts;
     if (q >= 12 && q <= 15) stall = take_fault(c->inject_tile_stall);
     launch(q);
