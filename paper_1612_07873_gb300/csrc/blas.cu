@@ -122,48 +122,72 @@ __device__ __forceinline__ void grid_loop_acc(size_t n, F&& body) {
   for (; i < n; i += stride) body(i, 0);
 }
 
-// The same loop for FP32 accumulators: fold() moves them to FP64 after every
-// ROUNDS rounds and at the end, so that an accumulator holds ROUNDS rounds'
-// terms and the last three elements at most, whatever the length and the
-// grid.  (One FP32 sum per thread and accumulator lost 1e-5 of the squared norm
-// of 48 vectors of 16^3x32 in the worst case, 128 terms each.)
+// The same loop for FP32 accumulators: fold() moves them to FP64 where another
+// round would follow ROUNDS rounds (0: never), so that an accumulator holds
+// ROUNDS rounds' terms and the last three elements at most, whatever the length
+// and the grid.  (One FP32 sum per thread and accumulator lost 1e-5 of the squared
+// norm of 48 vectors of 16^3x32 in the worst case, 128 terms each.)  Returns
+// whether a fold was made: vectors of one wave have none, and an FP64 addition of
+// zero per sum would show there (16 cycles a warp: 2.7 -> 3.2 us for the norm of
+// 256 coarse sites).
 constexpr int kFoldRounds = 4;
 template <int ROUNDS, typename F, typename G>
-__device__ __forceinline__ void grid_loop_fold(size_t n, F&& body, G&& fold) {
+__device__ __forceinline__ bool grid_loop_fold(size_t n, F&& body, G&& fold) {
   const size_t stride = size_t(gridDim.x) * blockDim.x;
   size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x;
   int c = 0;
+  bool folded = false;
   for (; i + (kAcc - 1) * stride < n; i += kAcc * stride) {
+    if (ROUNDS > 0 && c++ == ROUNDS) {
+      fold();
+      folded = true;
+      c = 1;
+    }
 #pragma unroll
     for (int k = 0; k < kAcc; ++k) body(i + k * stride, k);
-    if (ROUNDS > 0 && ++c == ROUNDS) {
-      fold();
-      c = 0;
-    }
   }
   for (; i < n; i += stride) body(i, 0);
-  fold();
+  return folded;
+}
+// the sum of the accumulators, widened
+__device__ __forceinline__ double widen1(float a) { return f2d(a); }
+__device__ __forceinline__ double widen1(double a) { return a; }
+template <typename T>
+__device__ __forceinline__ double acc_sum(const T (&a)[kAcc]) {
+  return widen1((a[0] + a[1]) + (a[2] + a[3]));
+}
+template <typename T>
+__device__ __forceinline__ double2 acc_sum(const cpx<T> (&a)[kAcc]) {
+  const cpx<T> t = (a[0] + a[1]) + (a[2] + a[3]);
+  return make_double2(widen1(t.re), widen1(t.im));
 }
 // s += the accumulators, which start again at zero
 template <typename T>
 __device__ __forceinline__ void fold_acc(double& s, T (&a)[kAcc]) {
-  const T t = (a[0] + a[1]) + (a[2] + a[3]);
-  if constexpr (std::is_same<T, float>::value)
-    s += f2d(t);
-  else
-    s += t;
+  s += acc_sum(a);
 #pragma unroll
   for (int k = 0; k < kAcc; ++k) a[k] = T(0);
 }
 template <typename T>
 __device__ __forceinline__ void fold_acc(double2& s, cpx<T> (&a)[kAcc]) {
-  const cpx<double> t = to_acc<double>((a[0] + a[1]) + (a[2] + a[3]));
-  s.x += t.re;
-  s.y += t.im;
+  const double2 t = acc_sum(a);
+  s.x += t.x;
+  s.y += t.y;
 #pragma unroll
   for (int k = 0; k < kAcc; ++k) a[k] = cpx<T>(T(0), T(0));
 }
-// rounds between folds (0: only at the end, for FP64 accumulators)
+// what the last fold left and the accumulators hold
+template <typename T>
+__device__ __forceinline__ double close_acc(double s, const T (&a)[kAcc], bool folded) {
+  const double t = acc_sum(a);
+  return folded ? s + t : t;
+}
+template <typename T>
+__device__ __forceinline__ double2 close_acc(double2 s, const cpx<T> (&a)[kAcc], bool folded) {
+  const double2 t = acc_sum(a);
+  return folded ? make_double2(s.x + t.x, s.y + t.y) : t;
+}
+// rounds between folds (0: none, for FP64 accumulators)
 template <typename T>
 constexpr int fold_rounds() {
   return std::is_same<T, float>::value ? kFoldRounds : 0;
@@ -181,7 +205,7 @@ __global__ void k_dot_partial(const cpx<Ra>* __restrict__ a, const cpx<Rb>* __re
 #pragma unroll
   for (int k = 0; k < kAcc; ++k) acc[k] = cpx<T>(T(0), T(0));
   double2 sum = make_double2(0.0, 0.0);
-  grid_loop_fold<fold_rounds<T>()>(
+  const bool folded = grid_loop_fold<fold_rounds<T>()>(
       n,
       [&](size_t i, int k) {
         if constexpr (NORM) {
@@ -192,7 +216,7 @@ __global__ void k_dot_partial(const cpx<Ra>* __restrict__ a, const cpx<Rb>* __re
         }
       },
       [&] { fold_acc(sum, acc); });
-  double2 d = block_sum(sum, sh);
+  double2 d = block_sum(close_acc(sum, acc, folded), sh);
   if (threadIdx.x == 0) part[size_t(blockIdx.y) * gridDim.x + blockIdx.x] = d;
 }
 
@@ -297,8 +321,10 @@ __global__ void __launch_bounds__(256, 2) k_dot_multi(VecList X, const cpx<R>* _
 #pragma unroll
     for (int j = 0; j < kCgs; ++j) sum[j] = make_double2(0.0, 0.0);
   }
+  bool folded = false;
   auto fold = [&] {
     if constexpr (FOLD) {
+      folded = true;
 #pragma unroll
       for (int j = 0; j < kCgs; ++j)
         if (j < m) {
@@ -332,16 +358,16 @@ __global__ void __launch_bounds__(256, 2) k_dot_multi(VecList X, const cpx<R>* _
         }
       }
   }
-  fold();
 #pragma unroll
   for (int j = 0; j < kCgs; ++j)
     if (j < m) {  // m is uniform: every thread takes the same branches
       double2 d;
       if constexpr (FF)
         d = make_double2(double(rh[j]) + double(rl[j]), double(ih[j]) + double(il[j]));
-      else if constexpr (FOLD)
-        d = sum[j];
-      else
+      else if constexpr (FOLD) {
+        d = make_double2(f2d(acc[j].re), f2d(acc[j].im));
+        if (folded) d = make_double2(sum[j].x + d.x, sum[j].y + d.y);
+      } else
         d = make_double2(double(acc[j].re), double(acc[j].im));
       d = block_sum(d, sh);
       if (threadIdx.x == 0) part[(size_t(v) * m + j) * gridDim.x + blockIdx.x] = d;
@@ -481,7 +507,7 @@ __global__ void k_dot2_partial_b(const cpx<Ra>* __restrict__ p, const cpx<Rb>* _
   }
   double2 s_pr = make_double2(0.0, 0.0);
   double s_pp = 0.0;
-  grid_loop_fold<fold_rounds<T>()>(
+  const bool folded = grid_loop_fold<fold_rounds<T>()>(
       n,
       [&](size_t i, int k) {
         cpx<T> x(p[i]), y(r[i]);
@@ -492,9 +518,9 @@ __global__ void k_dot2_partial_b(const cpx<Ra>* __restrict__ p, const cpx<Rb>* _
         fold_acc(s_pr, pr_k);
         fold_acc(s_pp, pp_k);
       });
-  double2 pr = block_sum(s_pr, sh);
+  double2 pr = block_sum(close_acc(s_pr, pr_k, folded), sh);
   __syncthreads();
-  double2 pp = block_sum(make_double2(s_pp, 0.0), sh);
+  double2 pp = block_sum(make_double2(close_acc(s_pp, pp_k, folded), 0.0), sh);
   if (threadIdx.x == 0) {
     const size_t base = size_t(blockIdx.y) * 2 * gridDim.x;
     part[base + blockIdx.x] = pr;
@@ -682,7 +708,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
   for (int k = 0; k < kAcc; ++k) acc[k] = Rx(0);
   double sum = 0.0;
-  grid_loop_fold<fold_rounds<Rx>()>(
+  const bool folded = grid_loop_fold<fold_rounds<Rx>()>(
       n,
       [&](size_t i, int k) {
         cpx<Rx> xi = x[i], ri = r[i];
@@ -699,7 +725,7 @@ __global__ void __launch_bounds__(256)
         acc[k] = fma(ri.re, ri.re, fma(ri.im, ri.im, acc[k]));
       },
       [&] { fold_acc(sum, acc); });
-  const double2 d = block_sum(make_double2(sum, 0.0), sh);
+  const double2 d = block_sum(make_double2(close_acc(sum, acc, folded), 0.0), sh);
   if (threadIdx.x == 0) part[size_t(blockIdx.y) * gridDim.x + blockIdx.x] = d;
 }
 
@@ -779,10 +805,11 @@ __global__ void k_dot2_partial_h(const bf16c* __restrict__ p, const bf16c* __res
     fold_acc(s_pr, pr_k);
     fold_acc(s_pp, pp_k);
   };
+  bool folded;
   if constexpr (W == 4) {
     const uint4* p4 = reinterpret_cast<const uint4*>(p);
     const uint4* r4 = reinterpret_cast<const uint4*>(r);
-    grid_loop_fold<kFoldRounds / 4>(
+    folded = grid_loop_fold<kFoldRounds / 4>(
         n / 4,
         [&](size_t i, int k) {
           const uint4 wp = p4[i], wr = r4[i];
@@ -793,11 +820,11 @@ __global__ void k_dot2_partial_h(const bf16c* __restrict__ p, const bf16c* __res
         },
         fold);
   } else {
-    grid_loop_fold<kFoldRounds>(n, [&](size_t i, int k) { term(p[i], r[i], k); }, fold);
+    folded = grid_loop_fold<kFoldRounds>(n, [&](size_t i, int k) { term(p[i], r[i], k); }, fold);
   }
-  double2 pr = block_sum(s_pr, sh);
+  double2 pr = block_sum(close_acc(s_pr, pr_k, folded), sh);
   __syncthreads();
-  double2 pp = block_sum(make_double2(s_pp, 0.0), sh);
+  double2 pp = block_sum(make_double2(close_acc(s_pp, pp_k, folded), 0.0), sh);
   if (threadIdx.x == 0) {
     const size_t base = size_t(blockIdx.y) * 2 * gridDim.x;
     part[base + blockIdx.x] = pr;
