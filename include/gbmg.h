@@ -232,7 +232,11 @@ mg_status mg_gcr_solve_multi(mg_ctx* ctx, void* x_dev, const void* b_dev, int nr
  * extent of the level even): y_o = S x_o with S = A_o - H_oe A_e^-1 H_eo the
  * Schur complement of level l's operator on the odd sites.  Compact parity
  * vectors: the odd site s is entry s >> 1, [nrhs][V/2][ndof] in the level's
- * vector precision.  MG_ERR_STATE if the level has no red-black form.      */
+ * vector precision.  MG_ERR_STATE if the level has no red-black form.
+ * Stream-ordered like the other applies: the call returns without waiting
+ * for `stream`.  Its temporary, nrhs half vectors, comes from a memory pool
+ * of the context, which keeps up to 1 GB of it until mg_destroy; MG_ERR_CUDA
+ * inside a stream capture.                                                 */
 mg_status mg_schur_apply(mg_ctx* ctx, int level, void* y_dev, const void* x_dev, int nrhs,
                          void* stream);
 

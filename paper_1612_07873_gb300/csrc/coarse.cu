@@ -105,11 +105,11 @@ __global__ void __launch_bounds__(CG*(N / Unpack<S>::RPC))
 // shared memory as planes [k][re r0..][im r0..], pairs of right-hand sides
 // form one FMA operand, link entries are duplicated.  CTAs are small (8
 // column groups, 96 threads at n = 48, five per SM), so one's gather and
-// reduction overlap the others' streams.  8^3x16, n = 48: 8 right-hand sides
-// 365 -> 297 us (HBM bound 208; two rows per thread and scalar FMAs before),
-// 32: 1336 -> 1089, 3: 652 -> 221 (odd counts ran the generic kernel).  The
-// links through a bulk-copy ring in shared memory: 460 us; 16 column groups
-// per CTA: 471 us.
+// reduction overlap the others' streams.  8^3x16, n = 48, whole calls: 8
+// right-hand sides 380 -> 315 us (HBM bound 208; two rows per thread and scalar
+// FMAs before), 3: 652 -> 209, 31: 4.73 -> 1.16 ms (odd counts ran the generic
+// kernel).  The links through a bulk-copy ring in shared memory: 460 us; 16
+// column groups per CTA: 471 us.
 // U: link columns a thread loads per batch; DB: the next batch is loaded
 // before the current one is used.  CG column groups split the 9n columns;
 // their sums meet in shared memory.

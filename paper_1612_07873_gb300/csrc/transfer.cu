@@ -515,7 +515,7 @@ __device__ __forceinline__ ff warp_sum8(ff (&x)[8], int lane) {
 // k_block_qr; a column that needs the second pass repeats its projection on
 // all earlier columns.
 // 16^3x32, 24 vectors, 4^4 aggregates (1024 blocks of 1536 rows): gather and QR
-// 4.86 -> 3.29 ms.
+// 4.86 -> 3.17 ms.
 // Sec. 3.4 step 3: QR of every (aggregate, chirality) block.
 template <int RPT, int P>
 __global__ void __launch_bounds__(256, P * RPT >= 16 ? 2 : 3)
