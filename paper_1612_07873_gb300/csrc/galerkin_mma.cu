@@ -17,19 +17,18 @@
 // itself (BF16 has FP32's exponents: entries of any size, down to 2^-110).  Six
 // products hold v w to 2^-26 of it: hi hi in one accumulator; hi mid, mid hi, hi
 // lo, mid mid, lo hi, 2^-8 of it and less, in another.  (FP16 pairs held an
-// operand to 2^-23, and numbers below 2^-13 to a fixed 2^-36: with vectors 1e-6 of
-// the others at the faces of their aggregate, face blocks were 0.1 to 0.3 of their
-// norm off.)  The
-// accumulators run over a unit of one chunk of eight sites (3 steps of K = 16) on
-// the X blocks, of two on the face blocks, and are then added to FP32 registers:
-// the tensor cores truncate when they accumulate, and on the X blocks, whose sums
-// have one sign, that bias grows with the unit.  Relative error of the links
-// against 64 bits, 24 vectors (the FP32 pipe's own sums in brackets): Gaussian
-// vectors 1.2e-7 on 2^4 [2.1e-7] and 1.3e-7 on 4^4 [7.7e-7] aggregates; one site
-// of each 2x4^3 aggregate large and the others 1e-3 of it, 1.9e-7 [1.1e-6]; sites
-// at the faces 1e-6 of the inner ones, worst face block 1.4e-7 [5.3e-7].  Units of
-// two chunks on the X blocks too: 1.6e-7 on 4^4, 0.5 % faster; of one everywhere:
-// 1.5 % slower.
+// operand to 2^-23, and numbers below 2^-13 to a fixed 2^-36: with vectors 1e-6
+// of the others at the faces of their aggregate, face blocks were 0.1 to 0.3 of
+// their norm off.)  The accumulators run over a unit of one chunk of eight sites
+// (3 steps of K = 16) on the X blocks, of two on the face blocks, and are then
+// added to FP32 registers: the tensor cores truncate when they accumulate, and on
+// the X blocks, whose sums have one sign, that bias grows with the unit.
+// Relative error of the links against 64 bits, 24 vectors (the FP32 pipe's own
+// sums in brackets): Gaussian vectors 1.2e-7 on 2^4 [2.1e-7] and 1.3e-7 on 4^4
+// [7.7e-7] aggregates; one site of each 2x4^3 aggregate large and the others 1e-3
+// of it, 1.9e-7 [1.1e-6]; sites at the faces 1e-6 of the inner ones, worst face
+// block 1.4e-7 [5.3e-7].  Units of two chunks on the X blocks too: 1.6e-7 on 4^4,
+// 0.5 % faster; of one everywhere: 1.5 % slower.
 //
 // What bounds it now: the T warps, on the latency of the P and link gathers
 // (issue 46 %, long-scoreboard stalls; the tensor pipe is 14 % busy).  24^3x48,
